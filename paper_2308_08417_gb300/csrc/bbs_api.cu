@@ -89,7 +89,8 @@ struct Plan {
     bool stage = false;
     bool gmres_ws = false;  // GMRES basis in the workspace
     bool ilu = false;       // ILU(0): level schedule in the workspace, factors in shared memory
-    int lanes = 32;         // < 32: packed kernel, 32 / lanes systems per one-warp block
+    int lanes = 32;         // < 32: packed kernel, 32 / lanes systems per warp
+    unsigned warps = 1;     // packed: warps per block
     size_t slice = 0;       // packed: shared-memory bytes per system
     size_t ws_gmres = 0, ws_f32 = 0, ws_ilu = 0;
     size_t ws_tables = 0;   // packed CSR: ELL column table, value map and flag
@@ -224,6 +225,10 @@ bbs_status make_plan(const bbs_handle* h, const bbs_batch_matrix* A, const bbs_o
             }
             p->lanes = L;
             p->R = R;
+            const long long warps = ((long long)A->num_batch + 32 / L - 1) / (32 / L);
+            if (o->solver == BBS_SOLVER_BICGSTAB && !ilu && smem * bbs::kPackedWarps <= (size_t)h->max_smem_optin &&
+                warps > (long long)bbs::kPackedWarps * h->sms)
+                p->warps = bbs::kPackedWarps;
             p->threads = 32;
             p->n_pad = n_pad;
             p->stage = true;
@@ -295,8 +300,30 @@ bbs_status make_plan(const bbs_handle* h, const bbs_batch_matrix* A, const bbs_o
     if (o->values_in_smem == 1)
         stage = base + stage_bytes <= limit;
     else if (o->values_in_smem == 0)
-        stage = base + stage_bytes <= kAutoStageBytes;
+        // (the fixed-point BiCGSTAB needs staged values: 1,000 systems of n = 2,025,
+        // 9-point: staged, one block on an SM, 3.26 ms, streamed FP64 4.73 ms)
+        stage = base + stage_bytes <= (o->solver == BBS_SOLVER_BICGSTAB && o->precond == BBS_PREC_JACOBI && !mixed
+                                           ? limit : kAutoStageBytes);
     if (base > limit) return fail(BBS_ERR_UNSUPPORTED, "shared memory need %zu exceeds %zu", base, limit);
+    if (stage && tps == 0 && !mixed && o->solver == BBS_SOLVER_BICGSTAB && o->precond == BBS_PREC_JACOBI) {
+        // The fixed-point kernel is bound by latency, not by a pipe: its warps
+        // spread evenly over the SM's four schedulers in powers of two (n = 625,
+        // 5-point, 6,400 systems: 3 warps 4.97 ms, 4 warps 3.51 ms; n = 1,600: 7
+        // warps 4.60 ms, 8 warps 4.22 ms), and long rows leave few blocks on an
+        // SM, where two rows per thread fill it (n = 144, 43 values a row, 16,384
+        // systems: 1 warp 19.9 ms, 2 warps 9.5 ms, 3 to 5 warps 8.4 ms).
+        int t = 32;
+        while (t < p->threads) t *= 2;
+        if (vps > 24 * (size_t)n)
+            while (t < 256 && n > 2 * t) t *= 2;
+        // one block fills an SM's shared memory: 8 warps (n = 144, dense: 18.1 ms
+        // with 4, 14.3 ms with 8)
+        if (base + stage_bytes > kAutoStageBytes && n > 32 * 4) t = 256;
+        if (t <= 256) {
+            p->threads = t;
+            p->R = (n + t - 1) / t;
+        }
+    }
     p->stage = stage;
     p->stage_off = base;
     p->smem = base + (stage ? stage_bytes : 0);
@@ -497,7 +524,8 @@ bbs_status bbs_describe(const bbs_handle* h, const bbs_batch_matrix* A, const bb
         info->kernel = p.ilu ? "bicgstab_ilu_packed_kernel"
                        : o->solver == BBS_SOLVER_CG ? "cg_packed_kernel"
                        : o->solver == BBS_SOLVER_GMRES ? "gmres_packed_kernel" : "bicgstab_packed_kernel";
-        info->grid = (A->num_batch + 32 / p.lanes - 1) / (32 / p.lanes);
+        const int warps = (A->num_batch + 32 / p.lanes - 1) / (32 / p.lanes);
+        info->grid = (warps + (int)p.warps - 1) / (int)p.warps;
         info->threads_per_system = p.lanes;
     } else {
         info->kernel = p.ilu ? "bicgstab_ilu_kernel"
@@ -509,9 +537,9 @@ bbs_status bbs_describe(const bbs_handle* h, const bbs_batch_matrix* A, const bb
         info->grid = A->num_batch;
         info->threads_per_system = p.threads;
     }
-    info->block = p.threads;
+    info->block = p.threads * (int)p.warps;
     info->rows_per_thread = p.R;
-    info->smem_bytes = (int64_t)p.smem;
+    info->smem_bytes = (int64_t)(p.smem * p.warps);
     info->values_staged = p.stage ? 1 : 0;
     info->launches = A->num_batch == 0 ? 0 : 1 + ((p.ws_f32 > 0 || p.ilu) ? 1 : 0) + (p.ws_tables > 0 ? 1 : 0);
     return BBS_OK;
@@ -634,10 +662,11 @@ bbs_status bbs_solve(bbs_handle* h, const bbs_batch_matrix* A, const double* b, 
                          : o->solver == BBS_SOLVER_CG ? bbs::cg_packed_fn(A->fmt, p.lanes, p.R)
                          : o->solver == BBS_SOLVER_GMRES ? bbs::gmres_packed_fn(A->fmt, p.lanes, p.R)
                                                          : bbs::bicgstab_packed_fn(A->fmt, p.lanes, p.R);
-        if ((e = allow_smem(fn, p.smem)) != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
+        if ((e = allow_smem(fn, p.smem * p.warps)) != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
         void* args[] = {&P, &csched};  // the ILU(0) kernels take the schedule as a second argument
-        const unsigned blocks = (unsigned)((A->num_batch + per_block - 1) / per_block);
-        e = cudaLaunchKernel(fn, dim3(blocks), dim3(32), args, p.smem, st);
+        const unsigned warps = (unsigned)((A->num_batch + per_block - 1) / per_block);
+        const unsigned blocks = (warps + p.warps - 1) / p.warps;
+        e = cudaLaunchKernel(fn, dim3(blocks), dim3(32 * p.warps), args, p.smem * p.warps, st);
         return e == cudaSuccess ? BBS_OK : cuda_fail(e, "packed solver launch");
     }
     const void* fn = pick_kernel(o, A->fmt, p.R, p.stage, A->ell_k, p.threads);

@@ -1,6 +1,6 @@
 // bicgstab kernels (plain and Jacobi-folded) instantiated for the ELL format, R = 1..kMaxR rows per thread.
 #include "bbs_kernels.h"
-#include "bbs_solvers.cuh"
+#include "bbs_fixed.cuh"
 
 namespace bbs {
 const void* bicgstab_fn_ell(int R) {

@@ -25,6 +25,7 @@
 // confirmation with at most kMaxRestarts restarts.
 #pragma once
 
+#include "bbs_fixed.cuh"
 #include "bbs_solvers.cuh"
 
 namespace bbs {
@@ -321,6 +322,30 @@ __device__ __forceinline__ void bicgstab_packed_system(const PackedOp<FMT, R>& o
         *io.rel_res = sqrt(res2 / nb2);
         *io.status = status;
         if (io.inner != nullptr) *io.inner = 0;
+    }
+}
+
+// BiCGSTAB of a warp's groups: with Jacobi in block fixed point (the integer
+// pipe); the groups it leaves (and all of them without Jacobi) in FP64. The
+// FP64 form is compiled as a function of its own.
+template <int FMT, int L, int R>
+__device__ __noinline__ void bicgstab_packed_fp64(const PackedOp<FMT, R> op, const SysIO io, bool valid,
+                                                  const SolveCfg C, const TeamSmem sm, const Team tm) {
+    bicgstab_packed_system<FMT, L, R>(op, io, valid, C, sm, tm);
+}
+
+template <int FMT, int L, int R>
+__device__ __forceinline__ void bicgstab_packed_any(const PackedOp<FMT, R>& op, const SysIO& io, bool valid,
+                                                    const SolveCfg& C, const TeamSmem& sm, const Team& tm) {
+    bool left = valid;
+    if (C.precond == 1) {  // every lane takes part, those without a system too
+        const bool done =
+            fx::bicgstab_fixed<FMT, staged_fmt<FMT>(), R>(op.A, op.S, io, valid, C, sm, fx::Lanes<L>{tm.lane}, tm);
+        left = valid && !done;
+    }
+    if (__any_sync(kFull, left)) {
+        __syncwarp();
+        bicgstab_packed_fp64<FMT, L, R>(op, io, left, C, sm, tm);
     }
 }
 
@@ -800,12 +825,11 @@ struct PackedGroup {
     bool valid;
     int sys;
     PackedOp<FMT, R> op;
-    // blk: the batch's block of 32 / L systems this warp solves (blockIdx.x
-    // unless the kernel strides over the batch)
+    // blk: the batch's block, 32 / L systems for each of its warps
     __device__ __forceinline__ PackedGroup(const SolveParams& P, unsigned char* raw, int blk) {
         constexpr int S = 32 / L;
         const int lane = threadIdx.x & 31, g = lane / L;
-        const int s = blk * S + g;
+        const int s = (blk * (blockDim.x >> 5) + (threadIdx.x >> 5)) * S + g;
         valid = s < P.num_batch;
         sys = valid ? s : P.num_batch - 1;
         tm.tid = lane & (L - 1);
@@ -814,7 +838,7 @@ struct PackedGroup {
         tm.warp = 0;
         tm.nwarps = 1;
         tm.bar = 0;
-        unsigned char* slice = raw + (size_t)g * P.slice;
+        unsigned char* slice = raw + (size_t)((threadIdx.x >> 5) * S + g) * P.slice;
         sm.red = nullptr;
         sm.xa = reinterpret_cast<double*>(slice);
         sm.xb = sm.xa + P.n_pad;
@@ -860,13 +884,16 @@ __device__ __forceinline__ bool packed_reject(const SolveParams& P, const Packed
     return false;
 }
 
-// One warp per block, 32 / L systems per warp.
+// 32 / L systems per warp; blocks of one warp, or of kPackedWarps that keep in
+// step (fixed point: their instruction fetches then hit; 65,536 systems of n =
+// 144: 6.37 ms with one warp to a block, 5.56 ms with four). Small batches keep
+// one warp to a block, which spreads them over the SMs.
 template <int FMT, int L, int R>
-__global__ void __launch_bounds__(32, packed_min_blocks(R)) bicgstab_packed_kernel(const SolveParams P) {
+__global__ void __launch_bounds__(32 * kPackedWarps, packed_min_blocks(R) / kPackedWarps) bicgstab_packed_kernel(const SolveParams P) {
     extern __shared__ __align__(16) unsigned char raw[];
     const PackedGroup<FMT, L, R> G(P, raw, blockIdx.x);
     if (packed_reject(P, G)) return;
-    bicgstab_packed_system<FMT, L, R>(G.op, sys_io(P, G.sys), G.valid, solve_cfg(P, G.sys), G.sm, G.tm);
+    bicgstab_packed_any<FMT, L, R>(G.op, sys_io(P, G.sys), G.valid, solve_cfg(P, G.sys), G.sm, G.tm);
 }
 
 // GMRES: the group's small arrays follow its staged values in the slice.

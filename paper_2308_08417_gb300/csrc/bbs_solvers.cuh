@@ -858,18 +858,4 @@ BBS_UNIFORM_KERNEL(cg_kernel, cg_system)
 BBS_UNIFORM_KERNEL(gmres_kernel, gmres_system)
 #undef BBS_UNIFORM_KERNEL
 
-// The folded BiCGSTAB keeps six vectors in registers; at 5-6 rows per thread
-// a cap of 128 registers holds them without spilling and doubles the systems
-// an SM keeps resident (the FP64 pipe needs many warps to stay busy).
-__host__ __device__ constexpr int folded_min_blocks(int R) { return (R == 5 || R == 6) ? 2 : 1; }
-
-template <int FMT, int R>
-__global__ void __launch_bounds__(max_threads_for(R), folded_min_blocks(R))
-    bicgstab_folded_kernel(const SolveParams P) {
-    extern __shared__ __align__(16) unsigned char raw[];
-    const Team tm = Team::block();
-    const int sys = blockIdx.x;
-    const auto op = make_op<FMT, R>(P, sys, raw, tm);
-    bicgstab_scaled_system<FMT, R>(op, sys_io(P, sys), solve_cfg(P, sys), team_smem(raw, P.n_pad), tm);
-}
 }  // namespace bbs

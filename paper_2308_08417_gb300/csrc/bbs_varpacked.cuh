@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(32, packed_min_blocks(R)) varpacked_kernel(con
     if constexpr (SOLVER == 1)
         cg_packed_system<FMT_CSR, L, R>(op, io, valid, P.cfg, sm, tm);
     else
-        bicgstab_packed_system<FMT_CSR, L, R>(op, io, valid, P.cfg, sm, tm);
+        bicgstab_packed_any<FMT_CSR, L, R>(op, io, valid, P.cfg, sm, tm);
 }
 
 // Kernel of class (L, R) for the solver (0 BiCGSTAB, 1 CG); one table per L.

@@ -1,0 +1,88 @@
+"""The block fixed-point BiCGSTAB at the edges of its layouts and ranges, against the CPU oracle."""
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2308_08417_gb300 import workloads as W
+from tests.parity import compare, host_rel_residual
+from tests.test_gpu_parity import gpu_solve
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def bbs():
+    from paper_2308_08417_gb300 import _build, bbs as mod
+
+    _build.build()
+    return mod
+
+
+@pytest.fixture(scope="module")
+def handle(bbs):
+    return bbs.Handle(0)
+
+
+def check(bbs, handle, pat, vals, b, fmt, x0=None, label="", **opts):
+    A = W.make_batch(pat, vals, fmt)
+    g = gpu_solve(bbs, handle, A, b, x0, **opts)
+    r = oracle.solve_batch(A, b, x0)
+    D = W.to_dense(pat, vals).reshape(-1, pat.n, pat.n)
+    fails = compare(*g[:4], r[0], r[1], r[3], rel_host=host_rel_residual(D, g[0], b), label=f"{label} {fmt} {opts}")
+    assert not fails, "\n".join(fails)
+
+
+@pytest.mark.parametrize("fmt", ["csr", "ell", "dense"])
+@pytest.mark.parametrize("n", [66, 72])
+def test_rows_longer_than_one_carry(bbs, handle, fmt, n):
+    """Full rows: more than the 64 terms a product sums between carries, on one
+    warp, on several and packed; n = 72 keeps dense digits by columns."""
+    rng = np.random.default_rng(n)
+    pat = W.random_pattern(n, n * n, rng)
+    vals = W.general_values(pat, 5, rng, 0.05, 0.5)
+    b = rng.uniform(-1, 1, (5, n))
+    for tps in (16, 32, 64, 96):
+        check(bbs, handle, pat, vals, b, fmt, threads_per_system=tps)
+
+
+@pytest.mark.parametrize("fmt,tps", [("csr", 0), ("ell", 8), ("dense", 4), ("csr", 32), ("dense", 32)])
+def test_fewer_rows_than_lanes_and_blocks_of_several_warps(bbs, handle, fmt, tps):
+    """3 rows on 4 to 32 lanes, and batches that fill blocks of four warps with
+    a ragged end (groups, and whole warps, without a system)."""
+    rng = np.random.default_rng(7)
+    for n, B in ((3, 21), (20, 6001)):
+        if tps and -(-n // tps) > 10:
+            continue
+        pat = W.stencil_pattern("1d3", n)
+        check(bbs, handle, pat, W.stencil_values(pat, B, rng, 0.05, 0.5), rng.uniform(-1, 1, (B, n)), fmt,
+              threads_per_system=tps)
+
+
+@pytest.mark.parametrize("tps", [0, 4, 32, 64])
+@pytest.mark.parametrize("guess", [False, True])
+def test_systems_that_do_not_fit_beside_ones_that_do(bbs, handle, tps, guess):
+    """In one warp: systems scaled to the ends of FP64's range, one whose scaled
+    rows sum to more than the fixed-point matrix holds, one with a zero guess
+    among guesses of every size; each as the oracle solves it."""
+    n, B = 40, 16
+    rng = np.random.default_rng(3)
+    pat = W.stencil_pattern("1d3", n)
+    vals = W.stencil_values(pat, B, rng, 0.05, 0.5)
+    b = rng.uniform(-1, 1, (B, n))
+    rows = np.repeat(np.arange(n), np.diff(pat.row_ptrs))
+    vals[1] *= 2.0 ** 480          # the matrix beyond FP32's range
+    b[2] *= 2.0 ** 450             # the right-hand side beyond 2^400
+    b[5] *= 2.0 ** -450
+    r = np.where(np.arange(n) % 2, 64.0, 1.0)
+    vals[9] *= r[rows]             # neighbouring rows scaled 64 : 1
+    b[9] *= r
+    b[12] *= 2.0 ** 390            # inside the range, at both ends
+    b[13] *= 2.0 ** -390
+    x0 = None
+    if guess:
+        D = W.to_dense(pat, vals).reshape(-1, n, n)
+        x0 = np.linalg.solve(D, b[..., None])[..., 0] * (1 + 1e-3 * rng.uniform(-1, 1, (B, n)))
+        x0[4] = 0.0
+        x0[6] *= 1e6               # far from the solution
+    check(bbs, handle, pat, vals, b, "csr", x0, threads_per_system=tps)
