@@ -71,10 +71,7 @@ TRAFFIC = {("bicgstab_packed_kernel", "stencil2d5_12x12"): (135.11e6, 16384),
            ("cg_packed_kernel", "sym_stencil2d5_12x12_cg+jacobi"): (133.00e6, 16384),
            ("gmres_packed_kernel", "stencil2d5_12x12_gmres+jacobi"): (147.83e6, 16384),
            ("bicgstab_ilu_packed_kernel", "stencil2d5_12x12_bicgstab+ilu0"): (134.60e6, 16384),
-           ("refine_kernel", "stencil2d9_32x32"): (396.44e6, 4096),
-           ("varsize_kernel", "uneven_n16-1024"): (333.05e6, 20000),
-           ("varsize_kernel+varpacked_kernel", "uneven_n16-1024"): (336.46e6, 20000),
-           ("varsize_kernel+varpacked_kernel+varwide_kernel", "uneven_n16-1024"): (332.21e6, 20000)}
+           ("refine_kernel", "stencil2d9_32x32"): (396.44e6, 4096)}
 
 
 # mixed refinement of the 32x32 9-point batch: the inner FP32 tolerance from a
@@ -349,12 +346,13 @@ class Uneven:
         self.desc = self.plan.describe()
         self.log = bbs.Log.empty(vb.num_batch, device=dev)
         self.num_batch = vb.num_batch
-        # one graph: the persistent team launch (with its counter reset), one
-        # launch per packed class of small systems and per wide-team class
+        # one graph: the persistent team launches (with their counters' reset;
+        # counted as one), one launch per packed class of small systems and per
+        # wide-team class
         d = self.desc
         persistent = 1 if d["persistent_grid"] else 0
-        self.kernel = "+".join(k for k, c in (("varsize_kernel", persistent), ("varpacked_kernel", d["packed_launches"]),
-                                              ("varwide_kernel", d["wide_launches"])) if c)
+        self.kernel = "+".join(k for k, c in (("varteam_kernel", persistent + d["wide_launches"]),
+                                              ("varpacked_kernel", d["packed_launches"])) if c)
         self.launches_per_step = persistent + d["packed_launches"] + d["wide_launches"]
         self.mixed = False
 

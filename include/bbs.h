@@ -311,10 +311,13 @@ typedef struct {
  * (wide[b], BiCGSTAB with Jacobi only, a bit set: 1 = systems whose rows hold
  * at most 4 stored values on average, 2 = the others, 3 = both, 0 = none. Such
  * a system, if it needs more than 8 rows per thread on the fewest warps that
- * hold it in at most 16 rows per thread (1, 2 or 4 warps), is solved by that
- * many warps, one block per system, values staged, in a launch of its own,
- * where such blocks still leave an SM 8 warps; the others run in the
- * persistent launch). block_warps is 8 (up to 8 rows per thread) or 16 (up to 4 rows per
+ * hold it in at most 16 rows per thread (1, 2 or 4 warps), is solved by a
+ * block of its own, values staged, in a launch of its own, where blocks of that
+ * many warps still leave an SM 8 warps; the others run in the persistent
+ * launches). With BiCGSTAB and Jacobi a system that one block can stage takes
+ * the fewest warps, a power of two, that leave 8 rows per thread (2 where its
+ * rows hold more than 24 values on average), whatever team_warps and
+ * stage_values say. block_warps is 8 (up to 8 rows per thread) or 16 (up to 4 rows per
  * thread). The planner lowers a bucket's warps to those of the next larger
  * bucket if they exceed them and raises them to the minimum its rows need. */
 typedef struct {
@@ -344,8 +347,10 @@ bbs_status bbs_var_default_tuning(int32_t max_n, bbs_var_tuning *tuning);
  * pointers that do not ascend within [0, nnz]) and builds an ELL column table
  * of each such pattern on the device. The other systems are ordered longest
  * first and grouped in segments of equal team size for one persistent launch
- * whose grid fills every SM. The CUDA graph holds "reset the work counters ->
- * the persistent launch" and, beside it, the packed and wide launches. Allocates the
+ * whose grid fills every SM; with BiCGSTAB and Jacobi those of them that one
+ * block each can stage go by (warps, rows per thread) instead, one persistent
+ * launch for each such group. The CUDA graph holds "reset the work counters ->
+ * the persistent launches" and, beside them, the packed and wide launches. Allocates the
  * plan's own device buffers (system order, counters, tables). The patterns
  * must not change while the plan lives (values, b and x may). tuning NULL =
  * default tuning. */
@@ -359,8 +364,8 @@ bbs_status bbs_var_plan_create(bbs_handle *handle, const bbs_var_batch *batch,
 bbs_status bbs_var_solve(bbs_var_plan *plan, const double *b, double *x, const bbs_log *log,
                          void *stream);
 
-/* What a plan runs: systems solved by teams in the persistent launch, systems
- * solved packed and the number of packed launches, the persistent grid (0 when
+/* What a plan runs: systems solved by teams in the persistent launches, systems
+ * solved packed and the number of packed launches, the blocks of the persistent launches (0 when
  * every system runs packed or wide), and systems solved by wide teams and the
  * number of wide launches. Host only. */
 typedef struct {

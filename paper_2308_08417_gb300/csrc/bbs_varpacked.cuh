@@ -6,7 +6,8 @@
 // rows whose group fits the shared-memory rule into a class (L, R): the
 // narrowest L of 4, 8, 16 that covers its n in R <= kMaxPackedR rows per lane.
 // Each class is one launch of varpacked_kernel<SOLVER, L, R> over the class's
-// systems (one warp per block, 32 / L systems per warp, in lockstep), and the
+// systems (32 / L systems per warp, in lockstep; one or kPackedWarps warps per
+// block), and the
 // plan's CUDA graph holds these launches beside the persistent team kernel.
 // Each pattern of a packed system has an ELL column table built once when
 // the plan is made; the values are gathered through it into shared memory in
@@ -54,11 +55,13 @@ struct VarPackedParams {
 
 // SOLVER: 0 = BiCGSTAB, 1 = CG (the uneven path's two solvers).
 template <int SOLVER, int L, int R>
-__global__ void __launch_bounds__(32, packed_min_blocks(R)) varpacked_kernel(const __grid_constant__ VarPackedParams P) {
+__global__ void __launch_bounds__(32 * kPackedWarps, packed_min_blocks(R) / kPackedWarps)
+    varpacked_kernel(const __grid_constant__ VarPackedParams P) {
     extern __shared__ __align__(16) unsigned char raw[];
     constexpr int G = 32 / L;
     const int lane = threadIdx.x & 31, g = lane / L;
-    const int item = blockIdx.x * G + g;
+    const int warp = threadIdx.x >> 5;
+    const int item = (blockIdx.x * (blockDim.x >> 5) + warp) * G + g;
     // groups past the end of the class solve its last system and never write
     const bool valid = item < P.count;
     const int sys = ldg(P.order + (valid ? item : P.count - 1));
@@ -74,7 +77,7 @@ __global__ void __launch_bounds__(32, packed_min_blocks(R)) varpacked_kernel(con
     tm.nwarps = 1;
     tm.bar = 0;
     const int n_pad = (n + 1) & ~1;
-    unsigned char* slice = raw + (size_t)g * P.slice;
+    unsigned char* slice = raw + (size_t)(warp * G + g) * P.slice;
     TeamSmem sm;
     sm.red = nullptr;
     sm.xa = reinterpret_cast<double*>(slice);

@@ -1,12 +1,14 @@
 // Uneven batches, host side: plan, autotuner and the CUDA graph of the
-// persistent team launch (kernel in bbs_varsize.cuh) and of the packed
-// small-system launches (bbs_varpacked.cuh).
+// persistent team launches (kernels in bbs_varteam.cuh and, for CG and
+// unpreconditioned systems, bbs_varsize.cuh) and of the packed small-system
+// launches (bbs_varpacked.cuh).
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <numeric>
 #include <vector>
 
@@ -16,31 +18,34 @@
 #include "bbs_internal.h"
 #include "bbs_kernels.h"
 #include "bbs_varpacked.cuh"
-#include "bbs_varwide.cuh"
+#include "bbs_varteam.cuh"
 #include "bbs_varsize.cuh"
 
 namespace bbs {
 const void* varpacked_fn(int solver, int L, int R) {
     return L == 4 ? varpacked_fn_l4(solver, R) : L == 8 ? varpacked_fn_l8(solver, R) : varpacked_fn_l16(solver, R);
 }
-const void* varwide_fn(int R) { return R <= 12 ? varwide_fn_lo(R) : varwide_fn_hi(R); }
+const void* varteam_fn(int R) { return R <= 5 ? varteam_fn_lo(R) : varteam_fn_hi(R); }
 }  // namespace bbs
 
 // ------------------------------------------------------------------ host
 
 struct PackedClass {
-    int L = 0, R = 0, grid = 0;
+    int L = 0, R = 0, warps = 1, grid = 0;
     size_t smem = 0;
     const void* fn = nullptr;
     bbs::VarPackedParams P{};
     cudaGraphNode_t node = nullptr;
 };
 
-struct WideClass {
-    int warps = 0, R = 0;
+// Systems of one (warps, rows per thread), one block per system: wide teams, or
+// the team systems of a persistent launch.
+struct BlockClass {
+    int warps = 0, R = 0, grid = 0;
+    bool wide = false;
     size_t smem = 0;
     const void* fn = nullptr;
-    bbs::VarWideParams P{};
+    bbs::VarTeamParams P{};
     cudaGraphNode_t node = nullptr;
 };
 
@@ -51,12 +56,13 @@ struct bbs_var_plan {
     size_t smem = 0;
     const void* fn = nullptr;
     bbs::VarParams P{};
-    int team_count = 0;  // systems of the persistent launch
-    bool has_team = false;
+    int team_count = 0;  // systems of the persistent launches
+    int team_grid = 0;   // blocks of the persistent launches of one block per system
+    bool has_team = false;  // the persistent launch of warp teams is in the graph
     int packed_count = 0;
     std::vector<PackedClass> classes;
-    int wide_count = 0;
-    std::vector<WideClass> wides;
+    int wide_count = 0, wide_launches = 0;
+    std::vector<BlockClass> blocks;
     int32_t* d_order = nullptr;
     int32_t* d_counters = nullptr;
     int32_t* d_tables = nullptr;  // flag [4] | xcols | xsrc of the packed patterns
@@ -88,6 +94,18 @@ int pow2_at_least(int v) {
     int p = 1;
     while (p < v) p <<= 1;
     return p;
+}
+
+// Lets fn use smem bytes of dynamic shared memory. The limit belongs to the
+// function, which the plan's other classes and other plans use too: it is only
+// ever raised.
+cudaError_t allow_smem(const void* fn, size_t smem) {
+    static std::mutex mutex;
+    std::lock_guard<std::mutex> lock(mutex);
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, fn);
+    if (e != cudaSuccess || (size_t)a.maxDynamicSharedSizeBytes >= smem) return e;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
 bool is_pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
@@ -150,6 +168,7 @@ struct PlanInputs {
 // chosen by the rule of the uniform packed kernels: the narrowest group of 4,
 // 8 or 16 lanes that covers n in at most kMaxPackedR rows per lane and leaves
 // at least kVarPackedMinWarps one-warp blocks resident per SM.
+constexpr int kVarWideMinR = 9, kVarWideMaxR = 16;  // rows per thread that make a team wide
 constexpr int kVarPackMaxN = 16 * bbs::kMaxPackedR;
 constexpr int kVarPackedMinWarps = 8;
 
@@ -283,10 +302,10 @@ bbs_status build_plan(bbs_handle* h, const PlanInputs& in, bbs_var_plan** out) {
         // wide bit 1: rows of at most 4 stored values on average; bit 2: denser
         const int density_bit = in.host->pat_nnz[p] <= 4 * n ? 1 : 2;
         if (wide_ok && (t.wide[bucket[i]] & density_bit)) {
-            const int w = pow2_at_least((n + 32 * bbs::kVarWideMaxR - 1) / (32 * bbs::kVarWideMaxR));
+            const int w = pow2_at_least((n + 32 * kVarWideMaxR - 1) / (32 * kVarWideMaxR));
             const int R = (n + 32 * w - 1) / (32 * w);
-            const size_t smem = bbs::varwide_smem(n, in.host->pat_nnz[p]);
-            if (w <= 4 && R >= bbs::kVarWideMinR && smem <= (size_t)optin && wide_resident_warps(smem, w) >= 8) {
+            const size_t smem = bbs::varteam_smem(n, in.host->pat_nnz[p]) - 16;
+            if (w <= 4 && R >= kVarWideMinR && smem <= (size_t)optin && wide_resident_warps(smem, w) >= 8) {
                 wide_w[i] = w;
                 wide_r[i] = R;
                 continue;
@@ -326,17 +345,16 @@ bbs_status build_plan(bbs_handle* h, const PlanInputs& in, bbs_var_plan** out) {
     std::vector<int32_t> order;
     order.reserve(nb);
     std::vector<int> seg_nmax, seg_nnzmax;
-    for (int k = 0; k < (int)idx.size(); ++k) {
-        const int i = idx[k];
+    const auto segments = [&](const std::vector<int>& systems) {
+      P.num_segments = 0;
+      for (int k = 0; k < (int)systems.size(); ++k) {
+        const int i = systems[k];
         order.push_back(sys[i]);
         const int w = W[bucket[i]], st = t.stage_values[bucket[i]];
         const int p = in.host->sys_pattern[sys[i]];
         if (P.num_segments == 0 || P.seg_warps[P.num_segments - 1] != w ||
             P.seg_stage[P.num_segments - 1] != st) {
-            if (P.num_segments == bbs::kMaxSeg) {
-                delete pl;
-                return errf(BBS_ERR_UNSUPPORTED, "more than %d segments", bbs::kMaxSeg);
-            }
+            if (P.num_segments == bbs::kMaxSeg) return false;
             P.seg_begin[P.num_segments] = k;
             P.seg_count[P.num_segments] = 0;
             P.seg_warps[P.num_segments] = w;
@@ -349,6 +367,12 @@ bbs_status build_plan(bbs_handle* h, const PlanInputs& in, bbs_var_plan** out) {
         ++P.seg_count[s];
         seg_nmax[s] = std::max(seg_nmax[s], in.host->pat_n[p]);
         seg_nnzmax[s] = std::max(seg_nnzmax[s], in.host->pat_nnz[p]);
+      }
+      return true;
+    };
+    if (!segments(idx)) {
+        delete pl;
+        return errf(BBS_ERR_UNSUPPORTED, "more than %d segments", bbs::kMaxSeg);
     }
     pl->team_count = (int)idx.size();
 
@@ -375,34 +399,65 @@ bbs_status build_plan(bbs_handle* h, const PlanInputs& in, bbs_var_plan** out) {
         c.P.count = (int)m.size();
         c.P.slice = (int)group_slice(raw, c.L);
         c.smem = (size_t)c.P.slice * (size_t)(32 / c.L);
-        c.grid = (c.P.count + 32 / c.L - 1) / (32 / c.L);
+        // blocks of several warps in step, as bbs_solve launches full batches
+        const int warps = (c.P.count + 32 / c.L - 1) / (32 / c.L);
+        if (in.o->solver == BBS_SOLVER_BICGSTAB && warps > bbs::kPackedWarps * sms &&
+            c.smem * bbs::kPackedWarps <= (size_t)optin)
+            c.warps = bbs::kPackedWarps;
+        c.smem *= (size_t)c.warps;
+        c.grid = (warps + c.warps - 1) / c.warps;
         c.fn = bbs::varpacked_fn(in.o->solver == BBS_SOLVER_CG ? 1 : 0, c.L, c.R);
         pl->packed_count += c.P.count;
         pl->classes.push_back(c);
     }
-    // wide classes, each ordered by estimated cost (longest first)
-    std::map<std::pair<int, int>, std::vector<int>> wcls;
+    // wide teams, and the team systems where one block each can stage them
+    // (BiCGSTAB with Jacobi): by (warps, rows per thread), the largest classes
+    // first, each ordered by estimated cost (longest first)
+    std::map<std::pair<int, int>, std::vector<int>> wcls, tcls;
+    const auto block_shape = [&](int i) {
+        const int p = in.host->sys_pattern[sys[i]];
+        const int n = in.host->pat_n[p];
+        int w = pow2_at_least((n + 32 * bbs::kMaxR - 1) / (32 * bbs::kMaxR));
+        if (in.host->pat_nnz[p] > 24 * n)  // long rows: two to a thread, as bbs_solve
+            while (w < 8 && n > 64 * w) w *= 2;
+        return std::make_pair(w, (n + 32 * w - 1) / (32 * w));
+    };
+    std::vector<int> left;  // to the persistent launch of warp teams
     for (int i = 0; i < nb; ++i)
-        if (wide_w[i] > 0) wcls[{wide_w[i], wide_r[i]}].push_back(i);
-    std::vector<int> wide_begin;
-    for (auto& kv : wcls) {
-        std::vector<int>& m = kv.second;
-        std::stable_sort(m.begin(), m.end(), [&](int a, int c) { return cost[a] > cost[c]; });
-        wide_begin.push_back((int)order.size());
-        WideClass c;
-        c.warps = kv.first.first;
-        c.R = kv.first.second;
-        for (int i : m) {
-            order.push_back(sys[i]);
-            const int p = in.host->sys_pattern[sys[i]];
-            c.smem = std::max(c.smem, bbs::varwide_smem(in.host->pat_n[p], in.host->pat_nnz[p]));
-        }
-        c.P.count = (int)m.size();
-        c.fn = bbs::varwide_fn(c.R);
-        pl->wide_count += c.P.count;
-        pl->wides.push_back(c);
+        if (wide_w[i] > 0) wcls[block_shape(i)].push_back(i);
+    for (int i : idx) {
+        const int p = in.host->sys_pattern[sys[i]];
+        if (wide_ok && bbs::varteam_smem(in.host->pat_n[p], in.host->pat_nnz[p]) <= (size_t)optin)
+            tcls[block_shape(i)].push_back(i);
+        else
+            left.push_back(i);
     }
-    pl->has_team = pl->team_count > 0 || (pl->classes.empty() && pl->wides.empty());
+    std::vector<int> block_begin;
+    for (const bool wide : {true, false}) {
+        auto& classes = wide ? wcls : tcls;
+        for (auto kv = classes.rbegin(); kv != classes.rend(); ++kv) {
+            std::vector<int>& m = kv->second;
+            std::stable_sort(m.begin(), m.end(), [&](int a, int c) { return cost[a] > cost[c]; });
+            block_begin.push_back((int)order.size());
+            BlockClass c;
+            c.wide = wide;
+            c.warps = kv->first.first;
+            c.R = kv->first.second;
+            for (int i : m) {
+                order.push_back(sys[i]);
+                const int p = in.host->sys_pattern[sys[i]];
+                c.smem = std::max(c.smem, bbs::varteam_smem(in.host->pat_n[p], in.host->pat_nnz[p]));
+            }
+            c.P.count = (int)m.size();
+            c.fn = bbs::varteam_fn(c.R);
+            if (wide) {
+                pl->wide_count += c.P.count;
+                ++pl->wide_launches;
+            }
+            pl->blocks.push_back(c);
+        }
+    }
+    pl->has_team = pl->team_count > 0 || (pl->classes.empty() && pl->blocks.empty());
 
     cudaError_t e;
     if (pl->has_team) {
@@ -425,8 +480,7 @@ bbs_status build_plan(bbs_handle* h, const PlanInputs& in, bbs_var_plan** out) {
                         pl->smem, optin);
         }
         pl->fn = rmax == 8 ? bbs::varsize_kernel8_fn() : bbs::varsize_kernel4_fn();
-        if ((e = cudaFuncSetAttribute(pl->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl->smem)) !=
-            cudaSuccess) {
+        if ((e = allow_smem(pl->fn, pl->smem)) != cudaSuccess) {
             delete pl;
             return cuda_err(e, "cudaFuncSetAttribute");
         }
@@ -440,14 +494,29 @@ bbs_status build_plan(bbs_handle* h, const PlanInputs& in, bbs_var_plan** out) {
         }
         pl->grid = per_sm * sms;
     }
+    // The checks above hold for every team system; the launch of warp teams is
+    // made only for those that no block takes.
+    size_t left_begin = 0;
+    if (!tcls.empty()) {
+        left_begin = order.size();
+        segments(left);
+        if (left.empty()) pl->has_team = false;
+    }
     for (auto& c : pl->classes)
-        if ((e = cudaFuncSetAttribute(c.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem)) !=
-            cudaSuccess)
-            return plan_fail(pl, cuda_err(e, "cudaFuncSetAttribute (packed)"));
-    for (auto& c : pl->wides)
-        if ((e = cudaFuncSetAttribute(c.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem)) !=
-            cudaSuccess)
-            return plan_fail(pl, cuda_err(e, "cudaFuncSetAttribute (wide)"));
+        if ((e = allow_smem(c.fn, c.smem)) != cudaSuccess)
+            return plan_fail(pl, cuda_err(e, "shared memory limit (packed)"));
+    for (auto& c : pl->blocks) {
+        if ((e = allow_smem(c.fn, c.smem)) != cudaSuccess)
+            return plan_fail(pl, cuda_err(e, "shared memory limit (one block per system)"));
+        c.grid = c.P.count;
+        if (!c.wide) {
+            int per_sm = 0;
+            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, c.fn, 32 * c.warps, c.smem)) != cudaSuccess)
+                return plan_fail(pl, cuda_err(e, "occupancy query"));
+            c.grid = std::min(c.P.count, std::max(1, per_sm) * sms);
+            pl->team_grid += c.grid;
+        }
+    }
 
     P.pat_n = vb->pat_n;
     P.pat_nnz = vb->pat_nnz;
@@ -469,16 +538,16 @@ bbs_status build_plan(bbs_handle* h, const PlanInputs& in, bbs_var_plan** out) {
     P.cfg.inner_tol = 0.0;
     P.cfg.ws = nullptr;
 
-    if ((e = cudaMalloc(&pl->d_order, sizeof(int32_t) * std::max(nb, 1))) != cudaSuccess ||
-        (e = cudaMalloc(&pl->d_counters, sizeof(int32_t) * bbs::kMaxSeg)) != cudaSuccess)
+    if ((e = cudaMalloc(&pl->d_order, sizeof(int32_t) * std::max<size_t>(order.size(), 1))) != cudaSuccess ||
+        (e = cudaMalloc(&pl->d_counters, sizeof(int32_t) * (bbs::kMaxSeg + pl->blocks.size()))) != cudaSuccess)
         return plan_fail(pl, errf(BBS_ERR_NO_MEMORY, "plan buffers: %s", cudaGetErrorString(e)));
-    if (nb > 0 && (e = cudaMemcpy(pl->d_order, order.data(), sizeof(int32_t) * nb, cudaMemcpyHostToDevice)) !=
-                      cudaSuccess)
+    if (!order.empty() && (e = cudaMemcpy(pl->d_order, order.data(), sizeof(int32_t) * order.size(),
+                                          cudaMemcpyHostToDevice)) != cudaSuccess)
         return plan_fail(pl, cuda_err(e, "order upload"));
-    P.order = pl->d_order;
+    P.order = pl->d_order + left_begin;
     P.counters = pl->d_counters;
-    for (size_t c = 0; c < pl->wides.size(); ++c) {
-        bbs::VarWideParams& Q = pl->wides[c].P;
+    for (size_t c = 0; c < pl->blocks.size(); ++c) {
+        bbs::VarTeamParams& Q = pl->blocks[c].P;
         Q.pat_n = vb->pat_n;
         Q.pat_nnz = vb->pat_nnz;
         Q.rp_off = vb->pat_rp_off;
@@ -489,7 +558,8 @@ bbs_status build_plan(bbs_handle* h, const PlanInputs& in, bbs_var_plan** out) {
         Q.val_off = vb->val_off;
         Q.vec_off = vb->vec_off;
         Q.values = vb->values;
-        Q.order = pl->d_order + wide_begin[c];
+        Q.order = pl->d_order + block_begin[c];
+        Q.counter = pl->blocks[c].wide ? nullptr : pl->d_counters + bbs::kMaxSeg + c;
         Q.cfg = P.cfg;
     }
 
@@ -549,20 +619,22 @@ bbs_status build_plan(bbs_handle* h, const PlanInputs& in, bbs_var_plan** out) {
         }
     }
 
-    // graph: [reset the work counters -> the persistent launch] beside one
+    // graph: [reset the work counters -> the persistent launches] beside one
     // launch per packed class and per wide class (no order among them)
     if ((e = cudaGraphCreate(&pl->graph, 0)) != cudaSuccess) return plan_fail(pl, cuda_err(e, "graph create"));
-    if (pl->has_team) {
+    cudaGraphNode_t mset = nullptr;
+    if (pl->has_team || pl->team_grid > 0) {
         cudaMemsetParams mp{};
         mp.dst = pl->d_counters;
         mp.elementSize = sizeof(int32_t);
-        mp.width = bbs::kMaxSeg;
+        mp.width = bbs::kMaxSeg + pl->blocks.size();
         mp.height = 1;
         mp.value = 0;
         mp.pitch = 0;
-        cudaGraphNode_t mset = nullptr;
         if ((e = cudaGraphAddMemsetNode(&mset, pl->graph, nullptr, 0, &mp)) != cudaSuccess)
             return plan_fail(pl, cuda_err(e, "graph memset node"));
+    }
+    if (pl->has_team) {
         void* args[] = {&P};
         cudaKernelNodeParams kp{};
         kp.func = const_cast<void*>(pl->fn);
@@ -578,22 +650,22 @@ bbs_status build_plan(bbs_handle* h, const PlanInputs& in, bbs_var_plan** out) {
         cudaKernelNodeParams kp{};
         kp.func = const_cast<void*>(c.fn);
         kp.gridDim = dim3(c.grid);
-        kp.blockDim = dim3(32);
+        kp.blockDim = dim3(32 * c.warps);
         kp.sharedMemBytes = (unsigned)c.smem;
         kp.kernelParams = args;
         if ((e = cudaGraphAddKernelNode(&c.node, pl->graph, nullptr, 0, &kp)) != cudaSuccess)
             return plan_fail(pl, cuda_err(e, "graph packed node"));
     }
-    for (auto& c : pl->wides) {
+    for (auto& c : pl->blocks) {
         void* args[] = {&c.P};
         cudaKernelNodeParams kp{};
         kp.func = const_cast<void*>(c.fn);
-        kp.gridDim = dim3(c.P.count);
+        kp.gridDim = dim3(c.grid);
         kp.blockDim = dim3(32 * c.warps);
         kp.sharedMemBytes = (unsigned)c.smem;
         kp.kernelParams = args;
-        if ((e = cudaGraphAddKernelNode(&c.node, pl->graph, nullptr, 0, &kp)) != cudaSuccess)
-            return plan_fail(pl, cuda_err(e, "graph wide node"));
+        if ((e = cudaGraphAddKernelNode(&c.node, pl->graph, c.wide ? nullptr : &mset, c.wide ? 0 : 1, &kp)) != cudaSuccess)
+            return plan_fail(pl, cuda_err(e, "graph block node"));
     }
     if ((e = cudaGraphInstantiate(&pl->exec, pl->graph, 0)) != cudaSuccess)
         return plan_fail(pl, cuda_err(e, "graph instantiate"));
@@ -681,13 +753,13 @@ bbs_status bbs_var_solve(bbs_var_plan* pl, const double* b, double* x, const bbs
         cudaKernelNodeParams kp{};
         kp.func = const_cast<void*>(c.fn);
         kp.gridDim = dim3(c.grid);
-        kp.blockDim = dim3(32);
+        kp.blockDim = dim3(32 * c.warps);
         kp.sharedMemBytes = (unsigned)c.smem;
         kp.kernelParams = args;
         if ((e = cudaGraphExecKernelNodeSetParams(pl->exec, c.node, &kp)) != cudaSuccess)
             return cuda_err(e, "graph parameter update (packed)");
     }
-    for (auto& c : pl->wides) {
+    for (auto& c : pl->blocks) {
         c.P.b = b;
         c.P.x = x;
         c.P.iters = log->iters;
@@ -696,12 +768,12 @@ bbs_status bbs_var_solve(bbs_var_plan* pl, const double* b, double* x, const bbs
         void* args[] = {&c.P};
         cudaKernelNodeParams kp{};
         kp.func = const_cast<void*>(c.fn);
-        kp.gridDim = dim3(c.P.count);
+        kp.gridDim = dim3(c.grid);
         kp.blockDim = dim3(32 * c.warps);
         kp.sharedMemBytes = (unsigned)c.smem;
         kp.kernelParams = args;
         if ((e = cudaGraphExecKernelNodeSetParams(pl->exec, c.node, &kp)) != cudaSuccess)
-            return cuda_err(e, "graph parameter update (wide)");
+            return cuda_err(e, "graph parameter update (one block per system)");
     }
     if ((e = cudaGraphLaunch(pl->exec, reinterpret_cast<cudaStream_t>(stream))) != cudaSuccess)
         return cuda_err(e, "graph launch");
@@ -714,8 +786,8 @@ bbs_status bbs_var_plan_describe(const bbs_var_plan* pl, bbs_var_plan_desc* d) {
     d->packed_systems = pl->packed_count;
     d->packed_launches = (int32_t)pl->classes.size();
     d->wide_systems = pl->wide_count;
-    d->wide_launches = (int32_t)pl->wides.size();
-    d->persistent_grid = pl->has_team ? pl->grid : 0;
+    d->wide_launches = pl->wide_launches;
+    d->persistent_grid = (pl->has_team ? pl->grid : 0) + pl->team_grid;
     return BBS_OK;
 }
 
