@@ -226,7 +226,7 @@ bbs_status make_plan(const bbs_handle* h, const bbs_batch_matrix* A, const bbs_o
             p->lanes = L;
             p->R = R;
             const long long warps = ((long long)A->num_batch + 32 / L - 1) / (32 / L);
-            if (o->solver == BBS_SOLVER_BICGSTAB && !ilu && smem * bbs::kPackedWarps <= (size_t)h->max_smem_optin &&
+            if (!gmres && !ilu && smem * bbs::kPackedWarps <= (size_t)h->max_smem_optin &&
                 warps > (long long)bbs::kPackedWarps * h->sms)
                 p->warps = bbs::kPackedWarps;
             p->threads = 32;
@@ -296,18 +296,20 @@ bbs_status make_plan(const bbs_handle* h, const bbs_batch_matrix* A, const bbs_o
                                    ? align_up((size_t)p->R * (size_t)A->ell_k * (size_t)p->threads * 6, 16)
                                    : align_up(vps * (mixed ? 4 : 8), 16);
     const size_t limit = (size_t)h->max_smem_optin;
+    // block fixed point (bbs_fixed.cuh): FP64 BiCGSTAB and CG with Jacobi
+    const bool fixed = !mixed && o->precond == BBS_PREC_JACOBI &&
+                       (o->solver == BBS_SOLVER_BICGSTAB || o->solver == BBS_SOLVER_CG);
     bool stage = false;
     if (o->values_in_smem == 1)
         stage = base + stage_bytes <= limit;
     else if (o->values_in_smem == 0)
-        // (the fixed-point BiCGSTAB needs staged values: 1,000 systems of n = 2,025,
+        // (the fixed-point solvers need staged values: BiCGSTAB, 1,000 systems of n = 2,025,
         // 9-point: staged, one block on an SM, 3.26 ms, streamed FP64 4.73 ms)
-        stage = base + stage_bytes <= (o->solver == BBS_SOLVER_BICGSTAB && o->precond == BBS_PREC_JACOBI && !mixed
-                                           ? limit : kAutoStageBytes);
+        stage = base + stage_bytes <= (fixed ? limit : kAutoStageBytes);
     if (base > limit) return fail(BBS_ERR_UNSUPPORTED, "shared memory need %zu exceeds %zu", base, limit);
-    if (stage && tps == 0 && !mixed && o->solver == BBS_SOLVER_BICGSTAB && o->precond == BBS_PREC_JACOBI) {
-        // The fixed-point kernel is bound by latency, not by a pipe: its warps
-        // spread evenly over the SM's four schedulers in powers of two (n = 625,
+    if (stage && tps == 0 && fixed) {
+        // The fixed-point kernels are bound by latency, not by a pipe: its warps
+        // spread evenly over the SM's four schedulers in powers of two (BiCGSTAB, n = 625,
         // 5-point, 6,400 systems: 3 warps 4.97 ms, 4 warps 3.51 ms; n = 1,600: 7
         // warps 4.60 ms, 8 warps 4.22 ms), and long rows leave few blocks on an
         // SM, where two rows per thread fill it (n = 144, 43 values a row, 16,384

@@ -342,8 +342,8 @@ struct Lanes {
         return v;
     }
     // out[j] = the sum of p[j], its vectors' exponents adding up to e[j]; o or-ed
-    template <int ND>
-    __device__ __forceinline__ void sums(const Part (&p)[ND], const int (&e)[ND], Sc (&out)[ND], unsigned& o) {
+    template <int ND, typename O>
+    __device__ __forceinline__ void sums(const Part (&p)[ND], const int (&e)[ND], Sc (&out)[ND], O& o) {
 #pragma unroll
         for (int s = L / 2; s; s >>= 1) o |= shfl_xor(o, s);
         const Part k = lane_sums<L, ND>(p, lane);
@@ -377,6 +377,10 @@ struct Warps {
         parity ^= 1;
         return r;
     }
+    __device__ __forceinline__ static unsigned or_all(unsigned o) { return __reduce_or_sync(kFull, o); }
+    __device__ __forceinline__ static unsigned long long or_all(unsigned long long o) {
+        return (unsigned long long)or_all((unsigned)(o >> 32)) << 32 | or_all((unsigned)o);
+    }
     __device__ __forceinline__ int max_int(int v) {
         v = __reduce_max_sync(kFull, v);
         if (tm.nwarps == 1) return v;
@@ -386,9 +390,9 @@ struct Warps {
         for (int w = 0; w < tm.nwarps; ++w) v = max(v, r[w]);
         return v;
     }
-    template <int ND>
-    __device__ __forceinline__ void sums(const Part (&p)[ND], const int (&e)[ND], Sc (&out)[ND], unsigned& o) {
-        o = __reduce_or_sync(kFull, o);
+    template <int ND, typename O>
+    __device__ __forceinline__ void sums(const Part (&p)[ND], const int (&e)[ND], Sc (&out)[ND], O& o) {
+        o = or_all(o);
         const Part k = lane_sums<32, ND>(p, tm.lane);
         const int w = which<32, ND>(tm.lane);
         if (tm.nwarps == 1) {
@@ -400,13 +404,13 @@ struct Warps {
             for (int j = 0; j < ND; ++j) out[j] = Sc{shfl(d.m, home<32, ND>(j)), shfl(d.e, home<32, ND>(j))};
             return;
         }
-        // slot of a warp: hi[3] (24 bytes) | lo[3] | mask, padded to 48
+        // slot of a warp: hi[3] (24 bytes) | lo[3] | 4 unused | mask (4 or 8 bytes), 48 in all
         unsigned char* r = half();
         if (w < ND && tm.lane == home<32, ND>(w)) {
             unsigned char* slot = r + tm.warp * 48;
             reinterpret_cast<long long*>(slot)[w] = k.hi;
             reinterpret_cast<int*>(slot + 24)[w] = k.lo;
-            if (w == 0) reinterpret_cast<unsigned*>(slot + 36)[0] = o;
+            if (w == 0) *reinterpret_cast<O*>(slot + 40) = o;
         }
         tm.sync();
         Part t[ND];
@@ -419,7 +423,7 @@ struct Warps {
                 t[j].hi += reinterpret_cast<const long long*>(slot)[j];
                 t[j].lo += reinterpret_cast<const int*>(slot + 24)[j];
             }
-            o |= reinterpret_cast<const unsigned*>(slot + 36)[0];
+            o |= *reinterpret_cast<const O*>(slot + 40);
         }
 #pragma unroll
         for (int j = 0; j < ND; ++j) out[j] = value(t[j], e[j]);
@@ -460,18 +464,18 @@ __device__ __forceinline__ void carry(Sum (&s)[R]) {
     }
 }
 
-// V = A Y for the caller's rows: `a` the staged digits, `y` the vector's
-// digits in shared memory. The result's exponent is y's plus sigma - 2, its
-// entries are below 2^59: sum |A hi| |Y hi| <= 2^31 2^28, and m holds 64 terms
-// of 2^57 between carries. The slots are the outer loop: R rows' loads are in
+// A Y for the caller's rows: `a` the staged digits, `y` the vector's digits in
+// shared memory. hh comes in units of y's exponent plus sigma - 2, below 2^59
+// (sum |A hi| |Y hi| <= 2^31 2^28), m as the 29 bits below it, rounded by
+// `round`. Between carries m holds kTerms terms of 2^57 (of 2^59 where |Y| goes
+// to 2^59, and hh to 2^61). The slots are the outer loop: R rows' loads are in
 // flight at once, and the loop's code stays within the instruction cache (all
 // rows' slots unrolled took 5 times the code and ran 8 times slower).
-template <int SF, int R>
-__device__ __forceinline__ void spmv_fixed(const Mat<double>& S, const int2* __restrict__ a,
-                                           const int2* __restrict__ y, Dig (&v)[R], const Team& tm) {
-    Sum s[R];
+template <int SF, int kTerms, int R>
+__device__ __forceinline__ void spmv_sums(const Mat<double>& S, const int2* __restrict__ a,
+                                          const int2* __restrict__ y, Sum (&s)[R], int round, const Team& tm) {
 #pragma unroll
-    for (int q = 0; q < R; ++q) s[q] = Sum{0, 1 << 28};  // rounds the last shift
+    for (int q = 0; q < R; ++q) s[q] = Sum{0, round};
     // Only the last row may lie past the end: such a lane repeats its first row
     // in its place (row 0 if it has none) and drops the result, so that the
     // loops need no branch.
@@ -491,8 +495,8 @@ __device__ __forceinline__ void spmv_fixed(const Mat<double>& S, const int2* __r
         }
         most = __reduce_max_sync(kFull, most);
 #pragma unroll 1
-        for (int j0 = 0; j0 < most; j0 += 64) {
-            const int j1 = min(most, j0 + 64);
+        for (int j0 = 0; j0 < most; j0 += kTerms) {
+            const int j1 = min(most, j0 + kTerms);
 #pragma unroll 1
             for (int j = j0; j < j1; ++j)
 #pragma unroll
@@ -504,8 +508,8 @@ __device__ __forceinline__ void spmv_fixed(const Mat<double>& S, const int2* __r
         const int32_t* c = S.cols + first;
         const int2* ar = a + first;
 #pragma unroll 1
-        for (int j0 = 0; j0 < S.k; j0 += 64) {
-            const int j1 = min(S.k, j0 + 64);
+        for (int j0 = 0; j0 < S.k; j0 += kTerms) {
+            const int j1 = min(S.k, j0 + kTerms);
 #pragma unroll 2
             for (int j = j0; j < j1; ++j) {
 #pragma unroll
@@ -520,8 +524,8 @@ __device__ __forceinline__ void spmv_fixed(const Mat<double>& S, const int2* __r
         const int rs = by_columns(S.n) ? 1 : S.n, cs = by_columns(S.n) ? S.n : 1;
         const int2* ar = a + first * rs;
 #pragma unroll 1
-        for (int j0 = 0; j0 < S.n; j0 += 64) {
-            const int j1 = min(S.n, j0 + 64);
+        for (int j0 = 0; j0 < S.n; j0 += kTerms) {
+            const int j1 = min(S.n, j0 + kTerms);
 #pragma unroll 2
             for (int j = j0; j < j1; ++j) {
                 const Dig yj = dig(y[j]);
@@ -533,12 +537,23 @@ __device__ __forceinline__ void spmv_fixed(const Mat<double>& S, const int2* __r
         }
     }
 #pragma unroll
-    for (int q = 0; q < R; ++q) v[q] = split(q + 1 < R || last ? s[q].hh : 0);
+    for (int q = 0; q < R; ++q)
+        if (q + 1 == R && !last) s[q] = Sum{0, 0};
+}
+
+// Their digits, rounded to units of y's exponent plus sigma - 2.
+template <int SF, int R>
+__device__ __forceinline__ void spmv_fixed(const Mat<double>& S, const int2* __restrict__ a,
+                                           const int2* __restrict__ y, Dig (&v)[R], const Team& tm) {
+    Sum s[R];
+    spmv_sums<SF, 64>(S, a, y, s, 1 << 28, tm);
+#pragma unroll
+    for (int q = 0; q < R; ++q) v[q] = split(s[q].hh);
 }
 
 // A residual b - A x, of which most leading bits have cancelled: shifts it so
 // that its largest entry has 56 bits (its exponent e follows), and returns its
-// squared norm. On entry the entries stay below 2^62.
+// squared norm.
 template <int R, class G>
 __device__ __forceinline__ Sc norm2_full(long long (&y)[R], int& e, G& g) {
     unsigned long long o = 0;
@@ -560,6 +575,59 @@ __device__ __forceinline__ Sc norm2_full(long long (&y)[R], int& e, G& g) {
     unsigned none = 0;
     g.sums(pt, pe, r, none);
     return r[0];
+}
+
+// ||b - A x||^2 (x through buf). A group with `take` set keeps b - A x in r,
+// and x with its units made finer.
+template <int SF, int R, class G>
+__device__ __forceinline__ Sc true_residual(const Mat<double>& S, const int2* as, int2* buf, const SysIO& io, int sigma,
+                                            long long (&X)[R], int& eX, int& bX, long long (&Rv)[R], int& eR, int& bR,
+                                            bool take, G& g, const Team& tm) {
+    const int n = io.n;
+    // x with 59 bits: shifted up exactly where it holds fewer (a guess far above
+    // the solution has left it coarse units), else rounded for the product
+    unsigned long long xo = 0;
+#pragma unroll
+    for (int q = 0; q < R; ++q) xo |= (unsigned long long)(X[q] ^ (X[q] >> 63));
+    const int k = 59 - g.max_int(64 - __clzll((long long)xo));
+    const int up = k > 0 && k < 59 ? k : 0, dx = max(-k, 0), ex4 = eX - up + dx;
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        const int row = tm.row(q);
+        const long long y = (long long)((unsigned long long)X[q] << up);
+        if (row < n) buf[row] = pack(split((y + ((1ll << dx) >> 1)) >> dx));
+        if (take) X[q] = y;
+    }
+    if (take) {  // (a system's bits do not depend on the warp's others)
+        eX -= up;
+        bX = 59 - min(k, 0);
+    }
+    g.sync();
+    Sum t[R];
+    spmv_sums<SF, 16>(S, as, buf, t, 1 << 27, tm);
+    int eb = 0;
+    double bq[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        const int row = tm.row(q);
+        bq[q] = row < n ? io.b[row] : 0.0;
+        eb = max(eb, (__double2hiint(bq[q]) >> 20) & 0x7ff);
+    }
+    eb = g.max_int(eb) - 1022 - 57;
+    // (b below 2^61 and A x below 2^62, in the finest unit that allows)
+    int eo = max(eb - 4, ex4 + sigma - 3);
+    long long w[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q)
+        w[q] = to_int(bq[q], -eo) - shr(t[q].hh + t[q].hh + (t[q].m >> 28), eo - ex4 - sigma + 3);
+    const Sc res = norm2_full(w, eo, g);
+    if (take) {
+#pragma unroll
+        for (int q = 0; q < R; ++q) Rv[q] = w[q];
+        eR = eo;
+        bR = 57;
+    }
+    return res;
 }
 
 // --------------------------------------------------------------- BiCGSTAB
@@ -670,29 +738,14 @@ __device__ __forceinline__ bool bicgstab_fixed(const Mat<double>& A, const Mat<d
         g.sums(pt, pe, r, none);
         nb2 = r[0];
         if (g.any(run && !xz)) {
-            const int ex0 = xz ? ebq : exm - 1022 - 57;
-#pragma unroll
-            for (int q = 0; q < R; ++q) {
-                const int row = tm.row(q);
-                if (row < n) {
-                    X[q] = to_int(diag_entry<FMT>(A, row) * io.x[row], -ex0);
-                    pb[row] = pack(split(X[q]));
-                }
-            }
-            g.sync();
-            Dig t[R];
-            spmv_fixed<SF, R>(S, as, pb, t, tm);
             if (!xz) {
-                // (b below 2^61 and A x~ below 2^59, in the finest unit that allows)
-                const int eo = max(ebq - 4, ex0 + sigma - 2);
+                eX = exm - 1022 - 57;
+                bX = 57;
 #pragma unroll
                 for (int q = 0; q < R; ++q)
-                    Rv[q] = (q + 1 < R || last ? to_int(io.b[tm.row(q)], -eo) : 0) -
-                            shr(join(t[q]), eo - ex0 - sigma + 2);
-                eR = eo;
-                eX = ex0;
-                bX = 57;
+                    if (q + 1 < R || last) X[q] = to_int(diag_entry<FMT>(A, tm.row(q)) * io.x[tm.row(q)], -eX);
             }
+            true_residual<SF>(S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, !xz, g, tm);
         }
     }
     const Sc tol2 = unpack(C.tol * C.tol), tau2 = C.tol_type == 1 ? mul(tol2, nb2) : tol2;
@@ -722,50 +775,8 @@ __device__ __forceinline__ bool bicgstab_fixed(const Mat<double>& A, const Mat<d
         if (row < n) pa[row] = make_int2(0, 0);  // p = 0
     }
 
-    // b - A x~ (x~ through pb), for the groups that take it in r; ||.||^2
     const auto residual = [&](bool take) -> Sc {
-        // x~ with 56 bits: shifted up exactly where it holds fewer (a guess far above
-        // the solution has left it coarse units), else rounded for the product
-        unsigned long long xo = 0;
-#pragma unroll
-        for (int q = 0; q < R; ++q) xo |= (unsigned long long)(X[q] ^ (X[q] >> 63));
-        const int k = 56 - g.max_int(64 - __clzll((long long)xo));
-        const int up = k > 0 && k < 56 ? k : 0, dx = max(-k, 0), ex4 = eX - up + dx;
-#pragma unroll
-        for (int q = 0; q < R; ++q) {
-            const int row = tm.row(q);
-            const long long y = (long long)((unsigned long long)X[q] << up);
-            if (row < n) pb[row] = pack(split((y + ((1ll << dx) >> 1)) >> dx));
-            if (take) X[q] = y;
-        }
-        if (take) {  // (a system's bits do not depend on the warp's others)
-            eX -= up;
-            bX = 56 - min(k, 0);
-        }
-        g.sync();
-        Dig t[R];
-        spmv_fixed<SF, R>(S, as, pb, t, tm);
-        int eb = 0;
-        double bq[R];
-#pragma unroll
-        for (int q = 0; q < R; ++q) {
-            const int row = tm.row(q);
-            bq[q] = row < n ? io.b[row] : 0.0;
-            eb = max(eb, (__double2hiint(bq[q]) >> 20) & 0x7ff);
-        }
-        eb = g.max_int(eb) - 1022 - 57;
-        int eo = max(eb - 4, ex4 + sigma - 2);
-        long long w[R];
-#pragma unroll
-        for (int q = 0; q < R; ++q) w[q] = to_int(bq[q], -eo) - shr(join(t[q]), eo - ex4 - sigma + 2);
-        const Sc res = norm2_full(w, eo, g);
-        if (take) {
-#pragma unroll
-            for (int q = 0; q < R; ++q) Rv[q] = w[q];
-            eR = eo;
-            bR = 57;
-        }
-        return res;
+        return true_residual<SF>(S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, take, g, tm);
     };
 
     for (int it = 1; it <= C.max_iters; ++it) {

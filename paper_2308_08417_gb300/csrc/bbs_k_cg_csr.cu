@@ -1,6 +1,6 @@
 // cg kernel instantiated for the CSR format, R = 1..kMaxR rows per thread.
 #include "bbs_kernels.h"
-#include "bbs_solvers.cuh"
+#include "bbs_fixed_cg.cuh"
 
 namespace bbs {
 const void* cg_fn_csr(int R) {

@@ -26,6 +26,7 @@
 #pragma once
 
 #include "bbs_fixed.cuh"
+#include "bbs_fixed_cg.cuh"
 #include "bbs_solvers.cuh"
 
 namespace bbs {
@@ -529,6 +530,27 @@ __device__ __forceinline__ void cg_packed_system(const PackedOp<FMT, R>& op, con
     write_result(io, x, status, iters, sqrt(res2 / nb2), 0, tm);
 }
 
+// CG of a warp's groups: with Jacobi in block fixed point, as BiCGSTAB above.
+template <int FMT, int L, int R>
+__device__ __noinline__ void cg_packed_fp64(const PackedOp<FMT, R> op, const SysIO io, bool valid, const SolveCfg C,
+                                            const TeamSmem sm, const Team tm) {
+    cg_packed_system<FMT, L, R>(op, io, valid, C, sm, tm);
+}
+
+template <int FMT, int L, int R>
+__device__ __forceinline__ void cg_packed_any(const PackedOp<FMT, R>& op, const SysIO& io, bool valid,
+                                              const SolveCfg& C, const TeamSmem& sm, const Team& tm) {
+    bool left = valid;
+    if (C.precond == 1) {  // every lane takes part, those without a system too
+        const bool done = fx::cg_fixed<staged_fmt<FMT>(), R>(op.A, op.S, io, valid, C, sm, fx::Lanes<L>{tm.lane}, tm);
+        left = valid && !done;
+    }
+    if (__any_sync(kFull, left)) {
+        __syncwarp();
+        cg_packed_fp64<FMT, L, R>(op, io, left, C, sm, tm);
+    }
+}
+
 // ----------------------------------------------------------------- GMRES
 
 // Right-preconditioned GMRES(m) with Jacobi folded into the staged values
@@ -909,11 +931,11 @@ __global__ void __launch_bounds__(32, packed_cg_min_blocks(R)) gmres_packed_kern
 }
 
 template <int FMT, int L, int R>
-__global__ void __launch_bounds__(32, packed_cg_min_blocks(R)) cg_packed_kernel(const SolveParams P) {
+__global__ void __launch_bounds__(32 * kPackedWarps, packed_cg_min_blocks(R) / kPackedWarps) cg_packed_kernel(const SolveParams P) {
     extern __shared__ __align__(16) unsigned char raw[];
     const PackedGroup<FMT, L, R> G(P, raw, blockIdx.x);
     if (packed_reject(P, G)) return;
-    cg_packed_system<FMT, L, R>(G.op, sys_io(P, G.sys), G.valid, solve_cfg(P, G.sys), G.sm, G.tm);
+    cg_packed_any<FMT, L, R>(G.op, sys_io(P, G.sys), G.valid, solve_cfg(P, G.sys), G.sm, G.tm);
 }
 
 }  // namespace bbs

@@ -854,7 +854,6 @@ __device__ __forceinline__ void gmres_system(const Op<FMT, R, double, double>& o
     }
 
 BBS_UNIFORM_KERNEL(bicgstab_kernel, bicgstab_system)
-BBS_UNIFORM_KERNEL(cg_kernel, cg_system)
 BBS_UNIFORM_KERNEL(gmres_kernel, gmres_system)
 #undef BBS_UNIFORM_KERNEL
 

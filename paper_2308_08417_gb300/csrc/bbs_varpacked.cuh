@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(32 * kPackedWarps, packed_min_blocks(R) / kPac
     io.inner = nullptr;
     io.n = n;
     if constexpr (SOLVER == 1)
-        cg_packed_system<FMT_CSR, L, R>(op, io, valid, P.cfg, sm, tm);
+        cg_packed_any<FMT_CSR, L, R>(op, io, valid, P.cfg, sm, tm);
     else
         bicgstab_packed_any<FMT_CSR, L, R>(op, io, valid, P.cfg, sm, tm);
 }

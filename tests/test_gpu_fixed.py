@@ -1,4 +1,4 @@
-"""The block fixed-point BiCGSTAB at the edges of its layouts and ranges, against the CPU oracle."""
+"""The block fixed-point BiCGSTAB and CG at the edges of its layouts and ranges, against the CPU oracle."""
 
 import numpy as np
 import pytest
@@ -27,7 +27,7 @@ def handle(bbs):
 def check(bbs, handle, pat, vals, b, fmt, x0=None, label="", **opts):
     A = W.make_batch(pat, vals, fmt)
     g = gpu_solve(bbs, handle, A, b, x0, **opts)
-    r = oracle.solve_batch(A, b, x0)
+    r = oracle.solve_batch(A, b, x0, solver=opts.get("solver", "bicgstab"))
     D = W.to_dense(pat, vals).reshape(-1, pat.n, pat.n)
     fails = compare(*g[:4], r[0], r[1], r[3], rel_host=host_rel_residual(D, g[0], b), label=f"{label} {fmt} {opts}")
     assert not fails, "\n".join(fails)
@@ -86,3 +86,42 @@ def test_systems_that_do_not_fit_beside_ones_that_do(bbs, handle, tps, guess):
         x0[4] = 0.0
         x0[6] *= 1e6               # far from the solution
     check(bbs, handle, pat, vals, b, "csr", x0, threads_per_system=tps)
+
+
+@pytest.mark.parametrize("fmt,tps", [("csr", 0), ("ell", 8), ("dense", 16), ("csr", 32), ("dense", 64), ("ell", 96)])
+def test_cg_edges(bbs, handle, fmt, tps):
+    """CG: 3 rows on many lanes, full rows longer than one carry, blocks of four
+    warps with a ragged end, guesses, and in one batch systems that do not fit
+    (a symmetric scaling of 64 : 1 between neighbours, both ends of the range)
+    beside ones that do."""
+    rng = np.random.default_rng(5)
+    for n, B in ((3, 9), (20, 6001), (72, 5)):
+        if tps and tps < 32 and -(-n // tps) > 10:
+            continue
+        if n == 72:  # a symmetric full matrix
+            pat = W.random_pattern(n, n * n, rng)
+            low = np.tril(rng.uniform(-1.0, 0.0, (B, n, n)), -1)
+            full = low + low.transpose(0, 2, 1)
+            i = np.arange(n)
+            full[:, i, i] = np.abs(full).sum(2) * (1 + rng.uniform(0.05, 0.5, (B, n)))
+            vals = full.reshape(B, -1)
+        else:
+            pat = W.stencil_pattern("1d3", n)
+            vals = W.stencil_values(pat, B, rng, 0.05, 0.5, symmetric=True)
+        check(bbs, handle, pat, vals, rng.uniform(-1, 1, (B, n)), fmt, solver="cg", threads_per_system=tps)
+    n, B = 40, 12
+    if tps == 0 or -(-n // tps) <= 10:
+        pat = W.stencil_pattern("1d3", n)
+        vals = W.stencil_values(pat, B, rng, 0.3, 0.9, symmetric=True)
+        b = rng.uniform(-1, 1, (B, n))
+        rows = np.repeat(np.arange(n), np.diff(pat.row_ptrs))
+        r = np.where(np.arange(n) % 2, 64.0, 1.0)
+        vals[3] *= r[rows] * r[pat.col_idxs]
+        b[3] *= r
+        vals[5] *= 2.0 ** 480
+        b[6] *= 2.0 ** -450
+        vals[8] *= 2.0 ** 90
+        D = W.to_dense(pat, vals).reshape(-1, n, n)
+        x0 = np.linalg.solve(D, b[..., None])[..., 0] * (1 + 1e-3 * rng.uniform(-1, 1, (B, n)))
+        x0[4] = 0.0
+        check(bbs, handle, pat, vals, b, fmt, x0, solver="cg", threads_per_system=tps)
