@@ -630,6 +630,151 @@ __device__ __forceinline__ Sc true_residual(const Mat<double>& S, const int2* as
     return res;
 }
 
+// The set-up of a solve with Jacobi folded in: whether the system fits (`run`;
+// false is returned, and nothing has been overwritten, where no group's does),
+// the staged matrix as digits of A D^-1, x~ = D x0, r = b - A x~ and ||b||^2.
+template <int FMT, int SF, int R, class G>
+__device__ __forceinline__ bool folded_setup(const Mat<double>& A, const Mat<double>& S, const SysIO& io, bool valid,
+                                             const TeamSmem& sm, G& g, const Team& tm, long long (&X)[R], int& eX,
+                                             int& bX, long long (&Rv)[R], int& eR, int& bR, int& sigma, bool& run,
+                                             Sc& nb2) {
+    const int n = io.n;
+    int2* as = in_shared<int2>(S.vals);
+    int2* pa = in_shared<int2>(sm.xa);
+    int2* pb = in_shared<int2>(sm.xb);
+    const bool last = tm.row(R - 1) < n;
+    eX = kNone;
+    bX = 0;
+    // (loops over the caller's rows stay rolled here: this runs once)
+    long long* dm = in_shared<long long>(sm.xb);  // 1 / a_ii: its digits,
+    int2* de = pa;                                // its exponent and FP32 value
+    int bad = 0, eb = 0, exm = 0;
+#pragma unroll 1
+    for (int row = tm.tid; row < n; row += tm.nt) {
+        double d = 0.0;
+        each_entry<SF>(S, row, [&](int e, int col) {
+            if (col == row) d = S.vals[e];
+        });
+        bad |= normal64(d) ? 0 : 1;
+        const Sc di = rcp(unpack(d));
+        dm[row] = di.m;
+        de[row] = make_int2(di.e, __float_as_int(fabsf(__frcp_rn((float)d))));
+        const double xt = d * io.x[row];
+        eb = max(eb, (__double2hiint(io.b[row]) >> 20) & 0x7ff);
+        exm = max(exm, zero64(xt) ? 0 : max(1, (__double2hiint(xt) >> 20) & 0x7ff));
+    }
+    g.sync();
+    int top = 0;  // largest row sum (as the bits of a non-negative FP32, NaN on top)
+#pragma unroll 1
+    for (int row = tm.tid; row < n; row += tm.nt) {
+        float t = 0.0f;
+        each_entry<SF>(S, row, [&](int e, int col) {
+            if (col >= 0) t = fmaf(fabsf((float)S.vals[e]), __int_as_float(de[col].y), t);
+        });
+        top = max(top, __float_as_int(t * 1.0001f) & 0x7fffffff);
+    }
+    top = g.max_int(bad ? 0x7fffffff : top);
+    eb = g.max_int(eb);
+    exm = g.max_int(exm);
+    const bool xz = exm == 0;  // the guess is zero
+    run = valid && top < __float_as_int(kRowSumMax) && eb > 623 && eb < 1423 && (xz || (exm > 623 && exm < 1423));
+    if (!g.any(run)) return false;
+    sigma = max(1, (top >> 23) - 126);  // row sums < 2^sigma
+    const int ebq = eb - 1022 - 57;
+    // --- the matrix as digits: A D^-1 2^(60 - sigma), unit diagonal, the
+    // quotients to the last bit or two
+    const auto digits = [&](double v, int row, int col) {
+        long long a = 0;
+        if (col == row) {
+            a = 1ll << (60 - sigma);
+        } else if (col >= 0) {
+            const Sc u = unpack(v);
+            a = round_shr(mul62(u.m, dm[col]), sigma - 122 - u.e - de[col].x);
+        }
+        return pack(split(a));
+    };
+#pragma unroll 1
+    for (int row = run ? tm.tid : n; row < n; row += tm.nt) {
+        if (SF == FMT_DENSE && by_columns(n)) {  // (read again from global memory: not in place)
+#pragma unroll 2
+            for (int j = 0; j < n; ++j) as[j * n + row] = digits(ldg(A.vals + (size_t)row * n + j), row, j);
+        } else {
+            each_entry<SF>(S, row, [&](int e, int col) { as[e] = digits(S.vals[e], row, col); });
+        }
+    }
+    g.sync();
+    // --- r = b - A x~
+    eR = ebq;
+    Dot d;
+    d.clear();
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        const int row = tm.row(q);
+        Rv[q] = row < n ? to_int(io.b[row], -ebq) : 0;
+        X[q] = 0;
+        d.square(split(Rv[q]));
+    }
+    const Part pt[1] = {part(d)};
+    const int pe[1] = {2 * ebq};
+    Sc r[1];
+    unsigned none = 0;
+    g.sums(pt, pe, r, none);
+    nb2 = r[0];
+    if (g.any(run && !xz)) {
+        if (!xz) {
+            eX = exm - 1022 - 57;
+            bX = 57;
+#pragma unroll
+            for (int q = 0; q < R; ++q)
+                if (q + 1 < R || last) X[q] = to_int(diag_entry<FMT>(A, tm.row(q)) * io.x[tm.row(q)], -eX);
+        }
+        true_residual<SF>(S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, !xz, g, tm);
+    }
+    return true;
+}
+
+// The end of such a solve: x = D^-1 x~ and the log, for the groups that ran.
+template <int FMT, int SF, int R, class G>
+__device__ __forceinline__ void folded_finish(const Mat<double>& A, const Mat<double>& S, const int2* as, int2* pb,
+                                              const SysIO& io, int sigma, long long (&X)[R], int& eX, int& bX,
+                                              long long (&Rv)[R], int& eR, int& bR, bool run, int iters, int status,
+                                              Sc res2, Sc nb2, const TeamSmem& sm, G& g, const Team& tm) {
+    const int n = io.n;
+    const bool last = tm.row(R - 1) < n;
+    // x = D^-1 x~, rounded to FP64
+    long long* xw = in_shared<long long>(sm.xa);
+    const bool moved = run && iters > 0;
+#pragma unroll
+    for (int q = 0; q < R; ++q)
+        if (q + 1 < R || last) xw[tm.row(q)] = X[q];
+#pragma unroll 1
+    for (int row = moved ? tm.tid : n; row < n; row += tm.nt) {
+        const Sc d = unpack(diag_entry<FMT>(A, row));
+        const double x = to_double(mul(normal(xw[row], eX), rcp(d)));
+        io.x[row] = x;
+        const Sc xr = unpack(x);
+        xw[row] = round_shr(mul62(xr.m, d.m), eX - xr.e - d.e - 62);
+    }
+    // where that rounding weighs in the residual (below 4e-12), the log takes
+    // the residual of the rounded x
+    const bool close = moved && le(res2, Sc{nb2.m, nb2.e - 76});
+    if (g.any(close)) {
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+            if (q + 1 < R || last) X[q] = xw[tm.row(q)];
+        const Sc res = true_residual<SF>(S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, false, g, tm);
+        if (close) res2 = res;
+    }
+    if (run) {
+        if (tm.tid == 0) {
+            *io.iters = iters;
+            *io.rel_res = sqrt(to_double(res2) / to_double(nb2));
+            *io.status = status;
+            if (io.inner != nullptr) *io.inner = 0;
+        }
+    }
+}
+
 // --------------------------------------------------------------- BiCGSTAB
 
 // BiCGSTAB with Jacobi folded into the staged matrix, as
@@ -650,104 +795,18 @@ __device__ __forceinline__ bool bicgstab_fixed(const Mat<double>& A, const Mat<d
     int2* pa = in_shared<int2>(sm.xa);  // p
     int2* pb = in_shared<int2>(sm.xb);  // s, and x~ for true residuals
 
-    // --- does the system fit? (FP32 is enough for the bound of the row sums)
     long long X[R], Rv[R];  // x~ = D x, r (then s)
     Dig rh[R], v[R];
     int eX = kNone, bX = 0, eR, bR, sigma;
     bool run;
     Sc nb2;
-    const bool last = tm.row(R - 1) < n;  // only a lane's last row may lie past the end
-    {
-        // (loops over the caller's rows stay rolled here: this runs once)
-        long long* dm = in_shared<long long>(sm.xb);  // 1 / a_ii: its digits,
-        int2* de = pa;                                // its exponent and FP32 value
-        int bad = 0, eb = 0, exm = 0;
-#pragma unroll 1
-        for (int row = tm.tid; row < n; row += tm.nt) {
-            double d = 0.0;
-            each_entry<SF>(S, row, [&](int e, int col) {
-                if (col == row) d = S.vals[e];
-            });
-            bad |= normal64(d) ? 0 : 1;
-            const Sc di = rcp(unpack(d));
-            dm[row] = di.m;
-            de[row] = make_int2(di.e, __float_as_int(fabsf(__frcp_rn((float)d))));
-            const double xt = d * io.x[row];
-            eb = max(eb, (__double2hiint(io.b[row]) >> 20) & 0x7ff);
-            exm = max(exm, zero64(xt) ? 0 : max(1, (__double2hiint(xt) >> 20) & 0x7ff));
+    if (!folded_setup<FMT, SF>(A, S, io, valid, sm, g, tm, X, eX, bX, Rv, eR, bR, sigma, run, nb2)) {
+        // (the block's other warps count on this one at their barriers)
+        for (int it = 1; it <= C.max_iters && g.live(false); ++it) {
         }
-        g.sync();
-        int top = 0;  // largest row sum (as the bits of a non-negative FP32, NaN on top)
-#pragma unroll 1
-        for (int row = tm.tid; row < n; row += tm.nt) {
-            float t = 0.0f;
-            each_entry<SF>(S, row, [&](int e, int col) {
-                if (col >= 0) t = fmaf(fabsf((float)S.vals[e]), __int_as_float(de[col].y), t);
-            });
-            top = max(top, __float_as_int(t * 1.0001f) & 0x7fffffff);
-        }
-        top = g.max_int(bad ? 0x7fffffff : top);
-        eb = g.max_int(eb);
-        exm = g.max_int(exm);
-        const bool xz = exm == 0;  // the guess is zero
-        run = valid && top < __float_as_int(kRowSumMax) && eb > 623 && eb < 1423 && (xz || (exm > 623 && exm < 1423));
-        if (!g.any(run)) {  // (the block's other warps count on this one at their barriers)
-            for (int it = 1; it <= C.max_iters && g.live(false); ++it) {
-            }
-            return false;
-        }
-        sigma = max(1, (top >> 23) - 126);  // row sums < 2^sigma
-        const int ebq = eb - 1022 - 57;
-        // --- the matrix as digits: A D^-1 2^(60 - sigma), unit diagonal, the
-        // quotients to the last bit or two
-        const auto digits = [&](double v, int row, int col) {
-            long long a = 0;
-            if (col == row) {
-                a = 1ll << (60 - sigma);
-            } else if (col >= 0) {
-                const Sc u = unpack(v);
-                a = round_shr(mul62(u.m, dm[col]), sigma - 122 - u.e - de[col].x);
-            }
-            return pack(split(a));
-        };
-#pragma unroll 1
-        for (int row = run ? tm.tid : n; row < n; row += tm.nt) {
-            if (SF == FMT_DENSE && by_columns(n)) {  // (read again from global memory: not in place)
-#pragma unroll 2
-                for (int j = 0; j < n; ++j) as[j * n + row] = digits(ldg(A.vals + (size_t)row * n + j), row, j);
-            } else {
-                each_entry<SF>(S, row, [&](int e, int col) { as[e] = digits(S.vals[e], row, col); });
-            }
-        }
-        g.sync();
-        // --- r = b - A x~
-        eR = ebq;
-        Dot d;
-        d.clear();
-#pragma unroll
-        for (int q = 0; q < R; ++q) {
-            const int row = tm.row(q);
-            Rv[q] = row < n ? to_int(io.b[row], -ebq) : 0;
-            X[q] = 0;
-            d.square(split(Rv[q]));
-        }
-        const Part pt[1] = {part(d)};
-        const int pe[1] = {2 * ebq};
-        Sc r[1];
-        unsigned none = 0;
-        g.sums(pt, pe, r, none);
-        nb2 = r[0];
-        if (g.any(run && !xz)) {
-            if (!xz) {
-                eX = exm - 1022 - 57;
-                bX = 57;
-#pragma unroll
-                for (int q = 0; q < R; ++q)
-                    if (q + 1 < R || last) X[q] = to_int(diag_entry<FMT>(A, tm.row(q)) * io.x[tm.row(q)], -eX);
-            }
-            true_residual<SF>(S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, !xz, g, tm);
-        }
+        return false;
     }
+    const bool last = tm.row(R - 1) < n;  // only a lane's last row may lie past the end
     const Sc tol2 = unpack(C.tol * C.tol), tau2 = C.tol_type == 1 ? mul(tol2, nb2) : tol2;
     Sc rr = norm2_full(Rv, eR, g);
     bR = 57;
@@ -1013,38 +1072,7 @@ __device__ __forceinline__ bool bicgstab_fixed(const Mat<double>& A, const Mat<d
         const Sc res = residual(false);
         if (need) res2 = res;
     }
-    // x = D^-1 x~, rounded to FP64
-    long long* xw = in_shared<long long>(sm.xa);
-    const bool moved = run && iters > 0;
-#pragma unroll
-    for (int q = 0; q < R; ++q)
-        if (q + 1 < R || last) xw[tm.row(q)] = X[q];
-#pragma unroll 1
-    for (int row = moved ? tm.tid : n; row < n; row += tm.nt) {
-        const Sc d = unpack(diag_entry<FMT>(A, row));
-        const double x = to_double(mul(normal(xw[row], eX), rcp(d)));
-        io.x[row] = x;
-        const Sc xr = unpack(x);
-        xw[row] = round_shr(mul62(xr.m, d.m), eX - xr.e - d.e - 62);
-    }
-    // where that rounding weighs in the residual (below 4e-12), the log takes
-    // the residual of the rounded x
-    const bool close = moved && le(res2, Sc{nb2.m, nb2.e - 76});
-    if (g.any(close)) {
-#pragma unroll
-        for (int q = 0; q < R; ++q)
-            if (q + 1 < R || last) X[q] = xw[tm.row(q)];
-        const Sc res = residual(false);
-        if (close) res2 = res;
-    }
-    if (run) {
-        if (tm.tid == 0) {
-            *io.iters = iters;
-            *io.rel_res = sqrt(to_double(res2) / to_double(nb2));
-            *io.status = status;
-            if (io.inner != nullptr) *io.inner = 0;
-        }
-    }
+    folded_finish<FMT, SF>(A, S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, run, iters, status, res2, nb2, sm, g, tm);
     return run;
 }
 

@@ -27,6 +27,7 @@
 
 #include "bbs_fixed.cuh"
 #include "bbs_fixed_cg.cuh"
+#include "bbs_fixed_gmres.cuh"
 #include "bbs_solvers.cuh"
 
 namespace bbs {
@@ -827,6 +828,12 @@ __device__ __forceinline__ void gmres_packed_system(const PackedOp<FMT, R>& op, 
     }
 }
 
+template <int FMT, int L, int R>
+__device__ __noinline__ void gmres_packed_fp64(const PackedOp<FMT, R> op, const SysIO io, bool valid, const SolveCfg C,
+                                               double* xa, double* ext, const Team tm) {
+    gmres_packed_system<FMT, L, R>(op, io, valid, C, xa, ext, tm);
+}
+
 // ------------------------------------------------------------- kernels
 
 // Resident blocks an SM must hold, which sets the register cap (registers
@@ -927,7 +934,17 @@ __global__ void __launch_bounds__(32, packed_cg_min_blocks(R)) gmres_packed_kern
     const size_t count = FMT == FMT_CSR ? (size_t)P.xk * P.n : P.vps;
     unsigned char* slice = raw + (size_t)((threadIdx.x & 31) / L) * P.slice;
     double* ext = reinterpret_cast<double*>(slice + P.stage_off + ((count * 8 + 15) & ~(size_t)15));
-    gmres_packed_system<FMT, L, R>(G.op, sys_io(P, G.sys), G.valid, solve_cfg(P, G.sys), G.sm.xa, ext, G.tm);
+    bool left = G.valid;
+    if (P.precond == 1) {  // block fixed point; every lane takes part, those without a system too
+        const bool done = fx::gmres_fixed<FMT, staged_fmt<FMT>(), R>(G.op.A, G.op.S, sys_io(P, G.sys), G.valid,
+                                                                     solve_cfg(P, G.sys), G.sm, ext,
+                                                                     fx::Lanes<L>{G.tm.lane}, G.tm);
+        left = G.valid && !done;
+    }
+    if (__any_sync(kFull, left)) {
+        __syncwarp();
+        gmres_packed_fp64<FMT, L, R>(G.op, sys_io(P, G.sys), left, solve_cfg(P, G.sys), G.sm.xa, ext, G.tm);
+    }
 }
 
 template <int FMT, int L, int R>

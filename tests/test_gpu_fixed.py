@@ -1,4 +1,4 @@
-"""The block fixed-point BiCGSTAB and CG at the edges of its layouts and ranges, against the CPU oracle."""
+"""The block fixed-point BiCGSTAB, CG and GMRES at the edges of its layouts and ranges, against the CPU oracle."""
 
 import numpy as np
 import pytest
@@ -27,7 +27,7 @@ def handle(bbs):
 def check(bbs, handle, pat, vals, b, fmt, x0=None, label="", **opts):
     A = W.make_batch(pat, vals, fmt)
     g = gpu_solve(bbs, handle, A, b, x0, **opts)
-    r = oracle.solve_batch(A, b, x0, solver=opts.get("solver", "bicgstab"))
+    r = oracle.solve_batch(A, b, x0, solver=opts.get("solver", "bicgstab"), restart=opts.get("gmres_restart", 10))
     D = W.to_dense(pat, vals).reshape(-1, pat.n, pat.n)
     fails = compare(*g[:4], r[0], r[1], r[3], rel_host=host_rel_residual(D, g[0], b), label=f"{label} {fmt} {opts}")
     assert not fails, "\n".join(fails)
@@ -125,3 +125,31 @@ def test_cg_edges(bbs, handle, fmt, tps):
         x0 = np.linalg.solve(D, b[..., None])[..., 0] * (1 + 1e-3 * rng.uniform(-1, 1, (B, n)))
         x0[4] = 0.0
         check(bbs, handle, pat, vals, b, fmt, x0, solver="cg", threads_per_system=tps)
+
+
+@pytest.mark.parametrize("fmt,tps", [("csr", 0), ("ell", 4), ("dense", 8), ("csr", 16)])
+@pytest.mark.parametrize("restart", [1, 10, 32])
+def test_gmres_edges(bbs, handle, fmt, tps, restart):
+    """GMRES: fewer rows than lanes, a heavy column (products above the rows' own
+    bound), guesses, and systems that do not fit beside ones that do."""
+    rng = np.random.default_rng(restart)
+    pat = W.stencil_pattern("1d3", 3)
+    check(bbs, handle, pat, W.stencil_values(pat, 9, rng, 0.3, 0.5), rng.uniform(-1, 1, (9, 3)), fmt, solver="gmres",
+          threads_per_system=tps, gmres_restart=restart)
+    n, B = 30, 13
+    pat = W.random_pattern(n, n * n, rng)
+    vals = W.general_values(pat, B, rng, 0.3, 0.9).reshape(B, n, n)
+    vals[2, :, 4] = np.where(np.arange(n) == 4, vals[2, :, 4], 20.0 * vals[2, 4, 4])  # 29 entries of 20 a_jj
+    vals = vals.reshape(B, -1)
+    b = rng.uniform(-1, 1, (B, n))
+    vals[5] *= 2.0 ** 480
+    b[6] *= 2.0 ** -450
+    vals[8] *= 2.0 ** 90
+    D = W.to_dense(pat, vals).reshape(-1, n, n)
+    x0 = np.linalg.solve(D, b[..., None])[..., 0] * (1 + 1e-3 * rng.uniform(-1, 1, (B, n)))
+    x0[3] = 0.0
+    A = W.make_batch(pat, vals, fmt)
+    g = gpu_solve(bbs, handle, A, b, x0, threads_per_system=tps, solver="gmres", gmres_restart=restart, max_iters=400)
+    r = oracle.solve_batch(A, b, x0, solver="gmres", restart=restart, max_iters=400)
+    fails = compare(*g[:4], r[0], r[1], r[3], rel_host=host_rel_residual(D, g[0], b), label=f"gmres {fmt} {tps}")
+    assert not fails, "\n".join(fails)
