@@ -2,31 +2,36 @@
 // layers for a tile of 128 systems, with the activations in shared memory and
 // the accumulator in tensor memory between the layers.
 //
-// Per block (10 warps):
-//   * warps 0-7 (256 threads) assemble the tile's standardised BF16 features
+// Per block (18 warps):
+//   * warps 0-15 (512 threads) assemble the tile's standardised BF16 features
 //     [diag(A), b, x_prev] with coalesced loads straight into the K-major
 //     no-swizzle core-matrix layout the MMAs read (8 rows x 16 bytes per core
 //     matrix, 16-byte K chunks 128 * 16 bytes apart), then run every
-//     epilogue: thread (warp w,
-//     lane l) owns TMEM lane / tile row 32 (w % 4) + l and every other
+//     epilogue: thread (warp w, lane l) owns TMEM lane / tile row 32 (w % 4) + l and every fourth
 //     16-column chunk (w / 4 picks which). Hidden layers: bias + GELU, BF16,
 //     written back over the layer's own input (its MMAs have completed).
 //     Output layer: bias, staged as FP32 in shared memory, then a coalesced
 //     pass writes x0 = x_prev + gamma (out * sigma + mu), or accumulates the
 //     gate statistics sum c.d and sum c.c (c = out * sigma + mu, d = x_next -
 //     x_prev) into acc.
-//   * warp 8, one lane: streams every layer's weights through a ring of
+//   * warp 16, one lane: streams every layer's weights through a ring of
 //     kInferStages stages, each a 64-wide K tile of W_l [N_l, K_l] copied by
 //     TMA (eight 16-byte-wide column boxes) with an mbarrier armed by bytes.
-//   * warp 9 allocates the tensor memory; one lane issues the MMAs: per K
+//   * warp 17 allocates the tensor memory; one lane issues the MMAs: per K
 //     tile four tcgen05.mma kind::f16 (M = 128, N = N_l, K = 16) into the
 //     FP32 accumulator, a commit that frees the stage, and after each layer a
 //     commit to "accumulator ready".
-// Handshakes: act_ready (256 arrivals: the layer's BF16 input is in shared
+// Handshakes: act_ready (512 arrivals: the layer's BF16 input is in shared
 // memory, fenced to the async proxy) and acc_ready (one commit per layer).
 // Every wait is bounded; a wait that runs out sets *err, the role stops, and
 // the block still waits (bounded) for its copies and MMAs before it frees the
 // tensor memory.
+//
+// A block's phases follow one another, and what takes the time is the latency
+// of the feature loads (four of them in flight per thread and a division per
+// entry, with 8 warps) and of the epilogues' GELU chains, not the bytes (133
+// MB, 20 us at the copy rate) or the MMAs. Sixteen warps and no divisions:
+// 16,384 systems, n = 144, hidden 256, 119.6 -> 79.2 us, the same bits.
 #pragma once
 
 #include <cstdint>
@@ -42,7 +47,9 @@ namespace mlp {
 
 constexpr int kInferRows = 128;
 constexpr int kInferStages = 3;
-constexpr int kInferEpiWarps = 8;
+constexpr int kInferEpiWarps = 16;
+constexpr int kInferEpi = kInferEpiWarps * 32;       // their threads
+constexpr int kInferColGroups = kInferEpiWarps / 4;  // 16-column chunks they take at a time
 constexpr int kInferThreads = (kInferEpiWarps + 2) * 32;
 
 struct InferParams {
@@ -226,7 +233,7 @@ __global__ void __launch_bounds__(kInferThreads, 1)
             umma_commit(saddr(done));  // arrives once every MMA issued above has completed
         }
     } else {  // epilogue warps
-        const int q = warp & 3, half = warp >> 2;
+        const int q = warp & 3, group = warp >> 2;
         const int r = q * 32 + lane;
         const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
         // the tile's features: the 256 threads walk the tile's rows of b and
@@ -235,15 +242,17 @@ __global__ void __launch_bounds__(kInferThreads, 1)
         // values into the core-matrix layout; padding columns get zeros
         {
             const int rows = min(kInferRows, p.num_batch - row0);
-            const int et = tid;  // 0..255
+            const int et = tid;  // 0..511
             unsigned char* actb = act;
             const auto put = [&](int rr, int f, float v) {
                 *reinterpret_cast<__nv_bfloat16*>(actb + (size_t)(f >> 3) * kLboA + (size_t)rr * 16 + (f & 7) * 2) =
                     __float2bfloat16_rn(v);
             };
+            // (rr, f) of the thread's entries without a division each
+            int rr = et / n, f = et - rr * n;
+            const int dr = kInferEpi / n, df = kInferEpi - dr * n;
 #pragma unroll 4
-            for (int idx = et; idx < kInferRows * n; idx += kInferEpiWarps * 32) {
-                const int rr = idx / n, f = idx - rr * n;
+            for (int idx = et; idx < kInferRows * n; idx += kInferEpi) {
                 float vd = 0.0f, vb = 0.0f, vx = 0.0f;
                 if (rr < rows) {  // standardised in FP32 (the FP64 pipe is scarce; BF16 follows)
                     const size_t sysr = (size_t)(row0 + rr);
@@ -256,6 +265,12 @@ __global__ void __launch_bounds__(kInferThreads, 1)
                 put(rr, f, vd);
                 put(rr, n + f, vb);
                 put(rr, 2 * n + f, vx);
+                rr += dr;
+                f += df;
+                if (f >= n) {
+                    f -= n;
+                    ++rr;
+                }
             }
             const int padw = p.in_pad - 3 * n;
             for (int idx = et; idx < kInferRows * padw; idx += kInferEpiWarps * 32)
@@ -270,7 +285,7 @@ __global__ void __launch_bounds__(kInferThreads, 1)
             }
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             const float* bias = sbias + l * p.hidden;
-            for (int c0 = half * 16; c0 < p.hidden; c0 += 32) {
+            for (int c0 = group * 16; c0 < p.hidden; c0 += 16 * kInferColGroups) {
                 uint32_t v[16];
                 tmem_ld16(lane_addr + (uint32_t)c0, v);
                 uint32_t w[8];
@@ -292,7 +307,7 @@ __global__ void __launch_bounds__(kInferThreads, 1)
         if (ok) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             const float* bias = sbias + 3 * p.hidden;
-            for (int c0 = half * 16; c0 < p.n_mma; c0 += 32) {
+            for (int c0 = group * 16; c0 < p.n_mma; c0 += 16 * kInferColGroups) {
                 uint32_t v[16];
                 tmem_ld16(lane_addr + (uint32_t)c0, v);
 #pragma unroll
@@ -307,9 +322,10 @@ __global__ void __launch_bounds__(kInferThreads, 1)
         if (ok) {
             const double g = GATE ? 0.0 : *p.gamma;
             double cd = 0.0, cc = 0.0;
+            int rr = tid / n, j = tid - rr * n;
+            const int dr = kInferEpi / n, dj = kInferEpi - dr * n;
 #pragma unroll 4
-            for (int idx = tid; idx < rows * n; idx += kInferEpiWarps * 32) {
-                const int rr = idx / n, j = idx - rr * n;
+            for (int idx = tid; idx < rows * n; idx += kInferEpi) {
                 const size_t gi = (size_t)(row0 + rr) * n + j;
                 // the de-standardised change in FP32, added to x_prev in FP64
                 const float c = fmaf(out[(size_t)rr * (n + 1) + j], p.stdv[3 * n + j], p.mean[3 * n + j]);
@@ -318,6 +334,12 @@ __global__ void __launch_bounds__(kInferThreads, 1)
                     cc = fma((double)c, (double)c, cc);
                 } else {
                     p.x0[gi] = fma(g, (double)c, p.xp[gi]);
+                }
+                rr += dr;
+                j += dj;
+                if (j >= n) {
+                    j -= n;
+                    ++rr;
                 }
             }
             if constexpr (GATE) {
