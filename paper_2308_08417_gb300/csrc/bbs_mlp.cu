@@ -53,25 +53,27 @@ __device__ __forceinline__ float gelu_grad(float z) {
 
 // ---------------------------------------------------------- epilogues
 
-enum EpiMode { EPI_F32 = 0, EPI_BIAS_GELU = 1, EPI_BIAS = 2, EPI_GELU_BWD = 3 };
+enum EpiMode { EPI_F32 = 0, EPI_BIAS_GELU = 1, EPI_BIAS = 2, EPI_GELU_BWD = 3, EPI_LOSS = 4 };
 
 struct Epi {
     int mode;
     float* c;                 // EPI_F32 / EPI_BIAS: output; EPI_BIAS_GELU: pre-activation store
     int ldc;
-    size_t zstride;           // EPI_F32: split-K part blockIdx.z goes to c + blockIdx.z * zstride
+    size_t zstride;           // EPI_F32: split-K part z goes to c + z * zstride
     const float* bias;        // EPI_BIAS_GELU / EPI_BIAS
     __nv_bfloat16* y;         // BF16 row-major output (EPI_BIAS_GELU, EPI_GELU_BWD)
     int ldy;
     __nv_bfloat16* yt;        // BF16 transposed output, may be null
     int ldyt;
-    const float* z;           // EPI_GELU_BWD: pre-activation of the layer below
+    const float* z;           // EPI_GELU_BWD: pre-activation of the layer below; EPI_LOSS: targets
     int ldz;
+    float* loss;              // EPI_LOSS: the mean squared error is added here
 
+    // One element; the mma.sync GEMM calls it (no split, no EPI_LOSS).
     __device__ __forceinline__ void operator()(int m, int n, float v) const {
         switch (mode) {
             case EPI_F32:
-                c[(size_t)blockIdx.z * zstride + (size_t)m * ldc + n] = v;
+                c[(size_t)m * ldc + n] = v;
                 break;
             case EPI_BIAS:
                 c[(size_t)m * ldc + n] = v + bias[n];
@@ -92,6 +94,90 @@ struct Epi {
             }
         }
     }
+
+    // Rows warp, warp + 8, ... of one column of the tile (lanes are
+    // neighbouring columns), eight rows' loads in flight at a time. With yt
+    // the BF16 result takes the accumulator's place in the tile.
+    template <int MODE>
+    __device__ __forceinline__ float column(float* t, int ld, int r0, int c0, int m0, int n0, int M, int bz) const {
+        constexpr int kWarps = umma::kThreads / 32, kU = 8;
+        const int n = n0 + c0;
+        const float bn = MODE == EPI_F32 || MODE == EPI_GELU_BWD ? 0.0f : bias[n];
+        const float scale = MODE == EPI_LOSS ? 2.0f / ((float)M * (float)ldc) : 0.0f;
+        float acc = 0.0f;
+        for (int i = r0; i < umma::kBM; i += kU * kWarps) {
+            float in[kU];
+            if (MODE == EPI_GELU_BWD || MODE == EPI_LOSS) {
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    const int m = m0 + i + u * kWarps;
+                    in[u] = m < M ? __ldg(z + (size_t)m * ldz + n) : 0.0f;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int r = i + u * kWarps, m = m0 + r;
+                if (m >= M) continue;
+                float* at = t + r * ld + c0;
+                float v = *at + bn;
+                if (MODE == EPI_F32) {
+                    c[(size_t)bz * zstride + (size_t)m * ldc + n] = v;
+                } else if (MODE == EPI_BIAS) {
+                    c[(size_t)m * ldc + n] = v;
+                } else {
+                    if (MODE == EPI_BIAS_GELU) {
+                        c[(size_t)m * ldc + n] = v;
+                        v = gelu(v);
+                    } else if (MODE == EPI_GELU_BWD) {
+                        v *= gelu_grad(in[u]);
+                    } else {
+                        const float diff = v - in[u];
+                        acc += diff * diff;
+                        v = diff * scale;
+                    }
+                    const __nv_bfloat16 h = __float2bfloat16_rn(v);
+                    y[(size_t)m * ldy + n] = h;
+                    if (yt) *reinterpret_cast<__nv_bfloat16*>(at) = h;
+                }
+            }
+        }
+        return acc;
+    }
+
+    // The epilogue of a whole 128 x BN tile t (row stride BN + 1), by all
+    // threads of the block.
+    __device__ __forceinline__ void tile(float* t, int BN, int m0, int n0, int M, int N, int bz) const {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ld = BN + 1;
+        float acc = 0.0f;
+        for (int c0 = lane; c0 < BN && n0 + c0 < N; c0 += 32) {
+            switch (mode) {
+                case EPI_F32: column<EPI_F32>(t, ld, warp, c0, m0, n0, M, bz); break;
+                case EPI_BIAS: column<EPI_BIAS>(t, ld, warp, c0, m0, n0, M, bz); break;
+                case EPI_BIAS_GELU: column<EPI_BIAS_GELU>(t, ld, warp, c0, m0, n0, M, bz); break;
+                case EPI_GELU_BWD: column<EPI_GELU_BWD>(t, ld, warp, c0, m0, n0, M, bz); break;
+                default: acc += column<EPI_LOSS>(t, ld, warp, c0, m0, n0, M, bz); break;
+            }
+        }
+        if (mode == EPI_LOSS) {
+            for (int k = 16; k; k >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, k);
+            if (lane == 0) atomicAdd(loss, acc / ((float)M * (float)ldc));
+        }
+        if (yt == nullptr) return;  // the same for every thread
+        __syncthreads();
+        const int wide = (ldyt & 1) == 0;  // pairs of rows are then 4-byte aligned (m0 and r are even)
+        for (int j = warp; j < BN && n0 + j < N; j += umma::kThreads / 32)
+            for (int r = 2 * lane; r < umma::kBM && m0 + r < M; r += 64) {
+                const __nv_bfloat16 lo = *reinterpret_cast<const __nv_bfloat16*>(t + r * ld + j);
+                const __nv_bfloat16 hi = *reinterpret_cast<const __nv_bfloat16*>(t + (r + 1) * ld + j);
+                __nv_bfloat16* to = yt + (size_t)(n0 + j) * ldyt + m0 + r;
+                if (wide && m0 + r + 1 < M) {
+                    *reinterpret_cast<__nv_bfloat162*>(to) = __nv_bfloat162(lo, hi);
+                } else {
+                    to[0] = lo;
+                    if (m0 + r + 1 < M) to[1] = hi;
+                }
+            }
+    }
 };
 
 __global__ void __launch_bounds__(256) gemm_kernel(const __nv_bfloat16* __restrict__ A, int lda,
@@ -100,11 +186,38 @@ __global__ void __launch_bounds__(256) gemm_kernel(const __nv_bfloat16* __restri
     gemm_tn_mma<Epi>(A, lda, B, ldb, M, N, K, epi);
 }
 
-__global__ void __launch_bounds__(128, 1) gemm_umma_kernel(const __grid_constant__ CUtensorMap ta,
-                                                           const __grid_constant__ CUtensorMap tb, int M, int N,
-                                                           int K, int BN, int ktiles_per_split, Epi epi,
-                                                           int* err) {
-    umma::gemm_tn_tma<Epi>(&ta, &tb, M, N, K, BN, ktiles_per_split, epi, err);
+// [4096 x 256] from K = 256 with GELU: 36 -> 12 us; with the GELU gradient
+// 28 -> 14 us (one launch from cold caches). What is left is latency: launch,
+// copies, one wave of 128 blocks' epilogues.
+__global__ void __launch_bounds__(umma::kThreads, 2) gemm_umma_kernel(const __grid_constant__ CUtensorMap ta,
+                                                                      const __grid_constant__ CUtensorMap tb, int M,
+                                                                      int N, int K, int BN, int ktiles_per_split,
+                                                                      Epi epi, int* err) {
+    umma::gemm_tn_tma<Epi>(&ta, &tb, M, N, K, BN, blockIdx.x, blockIdx.y, blockIdx.z, ktiles_per_split, epi, err);
+}
+
+// The weight gradients of all layers, C_l = A_l B_l^T over the same K (the
+// minibatch), in one launch: each alone is 8 to 14 tiles and was split 16-fold
+// only to fill the chip for 11 to 20 us a layer. They wait for nothing but the
+// output gradients, which are all there by the end of the backward chain.
+// The splits are those of the single GEMM, so the sums are the same. 57 us of
+// GEMMs and 24 us of sums -> 17 and 12 us.
+struct WeightGrads {
+    CUtensorMap a[kLayers], b[kLayers];
+    int M[kLayers], N[kLayers], BN[kLayers], kps[kLayers], nt[kLayers], mt[kLayers];
+    int first[kLayers + 1];  // first block of each
+    Epi epi[kLayers];
+};
+
+__global__ void __launch_bounds__(umma::kThreads, 2) weight_grads_kernel(const __grid_constant__ WeightGrads w, int K,
+                                                                         int* err) {
+    int l = 0;
+    while (l + 1 < kLayers && (int)blockIdx.x >= w.first[l + 1]) ++l;
+    int t = blockIdx.x - w.first[l];
+    const int bx = t % w.nt[l];
+    t /= w.nt[l];
+    umma::gemm_tn_tma<Epi>(&w.a[l], &w.b[l], w.M[l], w.N[l], K, w.BN[l], bx, t % w.mt[l], t / w.mt[l], w.kps[l],
+                           w.epi[l], err);
 }
 
 // c[m][n] = sum over the splits of part[z][m][n] (split-K, fixed order).
@@ -116,6 +229,63 @@ __global__ void splitk_reduce_kernel(int M, int N, int splits, const float* __re
         for (int z = 0; z < splits; ++z) s += part[(size_t)z * total + i];
         c[(i / N) * ldc + i % N] = s;
     }
+}
+
+// What is left of all layers' gradients, in one launch: the split-K sums
+// (blocks below first[0]; splits <= 1 leaves a layer's as they are) and, one
+// block per output, the bias gradients db[j] = sum of row j of dT [N, M].
+// One warp a row with 2-byte loads took 10 us a layer, most of it waiting;
+// a block reads the row in one or two 16-byte loads per thread (M is a
+// multiple of 64) and adds in a tree, so its chains are shorter too.
+struct GradSums {
+    const float* part[kLayers];
+    float* c[kLayers];
+    size_t total[kLayers];
+    int splits[kLayers];
+    const __nv_bfloat16* dT[kLayers];
+    float* db[kLayers];
+    int first[kLayers + 1];  // first bias block of each layer
+};
+
+__global__ void __launch_bounds__(256) grad_sums_kernel(const __grid_constant__ GradSums g, int M) {
+    if ((int)blockIdx.x < g.first[0]) {
+        for (int l = 0; l < kLayers; ++l) {
+            const int splits = g.splits[l];
+            if (splits <= 1) continue;
+            const size_t total = g.total[l];
+            const float* __restrict__ part = g.part[l];
+            for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
+                 i += (size_t)g.first[0] * blockDim.x) {
+                float s = 0.0f;
+#pragma unroll 8
+                for (int z = 0; z < splits; ++z) s += __ldg(part + (size_t)z * total + i);
+                g.c[l][i] = s;
+            }
+        }
+        return;
+    }
+    int l = 0;
+    while (l + 1 < kLayers && (int)blockIdx.x >= g.first[l + 1]) ++l;
+    const int j = blockIdx.x - g.first[l];
+    const uint4* row = reinterpret_cast<const uint4*>(g.dT[l] + (size_t)j * M);
+    float s = 0.0f;
+    for (int i = threadIdx.x; i < M / 8; i += blockDim.x) {
+        const uint4 q = __ldg(row + i);
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+        float p[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float2 f = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162&>(w[k]));
+            p[k] = f.x + f.y;
+        }
+        s += (p[0] + p[1]) + (p[2] + p[3]);
+    }
+    for (int k = 16; k; k >>= 1) s += __shfl_xor_sync(0xffffffffu, s, k);
+    __shared__ float ws[8];
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        g.db[l][j] = ((ws[0] + ws[1]) + (ws[2] + ws[3])) + ((ws[4] + ws[5]) + (ws[6] + ws[7]));
 }
 
 // ---------------------------------------------------- small kernels
@@ -200,22 +370,45 @@ __global__ void samples_kernel(int num_batch, int n, int in_pad, const int32_t* 
 }
 
 // Minibatch gather: rows idx[r] of the sample store into X [M, in_pad] and
-// X^T [in_pad, M], targets into T [M, n].
-__global__ void gather_kernel(int M, int in_pad, int n, const int32_t* __restrict__ idx,
-                              const __nv_bfloat16* __restrict__ feats, const float* __restrict__ targets,
-                              __nv_bfloat16* __restrict__ X, __nv_bfloat16* __restrict__ XT,
-                              float* __restrict__ T) {
-    const int r = blockIdx.x;
-    const size_t src = (size_t)idx[r];
-    for (int f = threadIdx.x; f < in_pad; f += blockDim.x) {
-        const __nv_bfloat16 v = feats[src * in_pad + f];
-        X[(size_t)r * in_pad + f] = v;
-        XT[(size_t)f * M + r] = v;
+// X^T [in_pad, M], targets into T [M, n]; clears the loss. One block moves 64
+// rows by 64 features through shared memory (M and in_pad are multiples of
+// 64), so that both copies are written in whole lines: a block per row wrote
+// X^T two bytes a line, 21 us for 4096 x 448 (now 8). The store is the
+// caller's; `wide` says that it is 16-byte aligned.
+__global__ void __launch_bounds__(256) gather_kernel(int M, int in_pad, int n, const int32_t* __restrict__ idx,
+                                                     const __nv_bfloat16* __restrict__ feats,
+                                                     const float* __restrict__ targets, bool wide,
+                                                     __nv_bfloat16* __restrict__ X, __nv_bfloat16* __restrict__ XT,
+                                                     float* __restrict__ T, float* __restrict__ loss) {
+    __shared__ __nv_bfloat16 t[64][66];
+    const int tid = threadIdx.x, f0 = blockIdx.x * 64, r0 = blockIdx.y * 64;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *loss = 0.0f;
+    const int c = (tid & 7) * 8;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int r = h * 32 + (tid >> 3);
+        const __nv_bfloat16* from = feats + (size_t)idx[r0 + r] * in_pad + f0 + c;
+        alignas(16) __nv_bfloat16 v[8];
+        if (wide) {
+            *reinterpret_cast<uint4*>(v) = __ldg(reinterpret_cast<const uint4*>(from));
+        } else {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = from[k];
+        }
+        *reinterpret_cast<uint4*>(X + (size_t)(r0 + r) * in_pad + f0 + c) = *reinterpret_cast<uint4*>(v);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) t[r][c + k] = v[k];
     }
-    for (int k = threadIdx.x; k < n; k += blockDim.x) T[(size_t)r * n + k] = targets[src * n + k];
+    for (int i = blockIdx.x * 256 + tid; i < 64 * n; i += gridDim.x * 256)
+        T[(size_t)r0 * n + i] = targets[(size_t)idx[r0 + i / n] * n + i % n];
+    __syncthreads();
+    const int r = (tid & 31) * 2;
+    for (int f = tid >> 5; f < 64; f += 8)
+        *reinterpret_cast<__nv_bfloat162*>(XT + (size_t)(f0 + f) * M + r0 + r) = __nv_bfloat162(t[r][f], t[r + 1][f]);
 }
 
 // dOut = 2 (out - t) / (M n) as BF16 [M, n_pad] and [n_pad, M]; loss sum.
+// For the mma.sync GEMM; the tcgen05 one has it in its epilogue (EPI_LOSS).
 __global__ void loss_kernel(int M, int n, int n_pad, const float* __restrict__ out,
                             const float* __restrict__ t, __nv_bfloat16* __restrict__ d,
                             __nv_bfloat16* __restrict__ dT, float* __restrict__ loss) {
@@ -244,19 +437,16 @@ __global__ void loss_kernel(int M, int n, int n_pad, const float* __restrict__ o
     }
 }
 
-// db[j] = sum over the row j of dT [N, M] (BF16), one warp per row.
-__global__ void bias_grad_kernel(int N, int M, const __nv_bfloat16* __restrict__ dT, float* __restrict__ db) {
-    const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (j >= N) return;
-    float s = 0.0f;
-    for (int m = threadIdx.x & 31; m < M; m += 32) s += __bfloat162float(dT[(size_t)j * M + m]);
-    for (int k = 16; k; k >>= 1) s += __shfl_xor_sync(0xffffffffu, s, k);
-    if ((threadIdx.x & 31) == 0) db[j] = s;
-}
+// Adam, and the BF16 copies of the new weights (pads stay zero): the four
+// packing launches that followed took 4 us each, next to nothing of it work.
+struct Layers {
+    int off_W[kLayers], out[kLayers], in[kLayers], in_pad[kLayers], out_pad[kLayers];
+    __nv_bfloat16 *Wb[kLayers], *WTb[kLayers];
+};
 
 __global__ void adam_kernel(size_t count, float* __restrict__ p, const float* __restrict__ g,
                             float* __restrict__ m, float* __restrict__ v, float lr, float b1, float b2,
-                            float eps, float c1, float c2) {
+                            float eps, float c1, float c2, const __grid_constant__ Layers w) {
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (size_t)gridDim.x * blockDim.x) {
         const float gi = g[i];
@@ -264,7 +454,16 @@ __global__ void adam_kernel(size_t count, float* __restrict__ p, const float* __
         const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
         m[i] = mi;
         v[i] = vi;
-        p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+        const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+        p[i] = pi;
+        int l = 0;
+        while (l + 1 < kLayers && (int)i >= w.off_W[l + 1]) ++l;
+        const int e = (int)i - w.off_W[l], r = e / w.in[l], k = e - r * w.in[l];
+        if (r < w.out[l]) {  // past the weights: the layer's biases
+            const __nv_bfloat16 h = __float2bfloat16_rn(pi);
+            w.Wb[l][(size_t)r * w.in_pad[l] + k] = h;
+            w.WTb[l][(size_t)k * w.out_pad[l] + r] = h;
+        }
     }
 }
 
@@ -382,11 +581,10 @@ struct bbs_mlp {
     __nv_bfloat16 *D = nullptr, *DT = nullptr;
     __nv_bfloat16* DZ[3] = {};
     __nv_bfloat16* DZT[3] = {};
-    int32_t* idx = nullptr;
     int* err = nullptr;     // set by a tensor-core GEMM whose waits ran out
     double* gate = nullptr;  // [gamma, sum c.d, sum c.c] (see bbs_mlp_gate_observe)
     float* part = nullptr;  // split-K partial sums of the weight-gradient GEMMs
-    size_t part_cap = 0;    // floats
+    size_t part_cap = 0;    // floats one layer may take of it
     int sms = 0;
     int gemm_kind = BBS_GEMM_TCGEN05;  // or BBS_GEMM_MMA_SYNC
     // fused inference (bbs_mlp_infer.cuh): TMA maps of the BF16 weights, the
@@ -438,70 +636,98 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 }
 
 // TMA map of a K-major BF16 operand [rows, K] (row stride ld elements) read
-// in boxes of 8 K-elements (16 bytes) by box_rows rows; rows past the end
-// read as zeros.
-bool make_operand_map(CUtensorMap* map, const __nv_bfloat16* ptr, int rows, int K, int ld, int box_rows) {
+// in boxes of box_k K-elements by box_rows rows: 8 (16 bytes) without a
+// swizzle, or 64 (128 bytes) in the 128-byte swizzle. Rows past the end read
+// as zeros.
+bool make_operand_map(CUtensorMap* map, const __nv_bfloat16* ptr, int rows, int K, int ld, int box_rows,
+                      int box_k = 8) {
     PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     if (enc == nullptr) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    const cuuint32_t box[2] = {8, (cuuint32_t)box_rows};
+    const cuuint32_t box[2] = {(cuuint32_t)box_k, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<__nv_bfloat16*>(ptr), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, box_k == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Tiles and splits of a tcgen05 GEMM: 128 rows x BN columns, BN <= 64 so that
+// the layer GEMMs over thousands of samples launch hundreds of blocks. An
+// FP32-output GEMM with few tiles and a long K (the weight gradients, K =
+// samples) is split over K when part_cap floats have room: each split writes
+// its partial tile, which are then added in a fixed order.
+struct Tiles {
+    int BN, mt, nt, splits, kps;
+};
+
+// Grows with the number of k-tiles nk; 1 where the tiles fill the chip.
+int max_splits(const Tiles& t, int nk, size_t total, size_t part_cap, int sms) {
+    const int want = 2 * sms, tiles = t.mt * t.nt;  // two blocks per SM fit (96 KB of stages each)
+    if (tiles >= want || nk < 8 || total == 0) return 1;
+    const size_t s = std::min<size_t>((size_t)std::min((want + tiles - 1) / tiles, nk / 4), part_cap / total);
+    return (int)std::max<size_t>(s, 1);
+}
+
+Tiles gemm_tiles(int M, int N, int K, bool split, size_t part_cap, int sms) {
+    Tiles t;
+    const int ntile = (N + 63) / 64;
+    t.BN = std::max(16, round_up((N + ntile - 1) / ntile, 16));
+    t.mt = (M + bbs::umma::kBM - 1) / bbs::umma::kBM;
+    t.nt = (N + t.BN - 1) / t.BN;
+    const int nk = K / bbs::umma::kBK;
+    t.splits = 1, t.kps = nk;
+    if (split) {
+        t.splits = max_splits(t, nk, (size_t)M * N, part_cap, sms);
+        if (t.splits > 1) {
+            t.kps = (nk + t.splits - 1) / t.splits;
+            t.splits = (nk + t.kps - 1) / t.kps;  // every split has k-tiles
+        }
+    }
+    return t;
+}
+
+bool gemm_maps(CUtensorMap* ta, CUtensorMap* tb, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb,
+               int M, int N, int K, int BN) {
+    return make_operand_map(ta, A, M, K, lda, bbs::umma::kBM, bbs::umma::kBK) &&
+           make_operand_map(tb, B, N, K, ldb, BN, bbs::umma::kBK);
+}
+
+template <class Kernel>
+cudaError_t gemm_attr(Kernel k) {
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bbs::umma::smem_bytes(64));
 }
 
 // C = A B^T through the chosen tensor-core path (kind 1: tcgen05 with the
 // accumulator in tensor memory, K a multiple of 64; kind 0: mma.sync).
-// tcgen05 tiles: 128 rows x BN columns, BN <= 64 so that the layer GEMMs
-// over thousands of samples launch hundreds of blocks. An FP32-output GEMM
-// with few tiles and a long K (the weight gradients, K = samples) is split
-// over K when `part` has room: each split writes its partial tile, and
-// splitk_reduce_kernel adds them in a fixed order.
 cudaError_t gemm_any(int kind, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M, int N,
                      int K, const Epi& e, int* err, cudaStream_t st, float* part = nullptr, size_t part_cap = 0,
                      int sms = 152) {
     if (kind == BBS_GEMM_TCGEN05) {
-        const int ntile = (N + 63) / 64;
-        const int BN = std::max(16, round_up((N + ntile - 1) / ntile, 16));
-        const int mt = (M + bbs::umma::kBM - 1) / bbs::umma::kBM, nt = (N + BN - 1) / BN;
-        const int nk = K / bbs::umma::kBK;
-        int splits = 1, kps = nk;
-        const int want = 2 * sms;  // two blocks per SM fit (96 KB of stages each)
-        if (e.mode == bbs::mlp::EPI_F32 && part != nullptr && mt * nt < want && nk >= 8) {
-            splits = std::min((want + mt * nt - 1) / (mt * nt), nk / 4);
-            while (splits > 1 && (size_t)splits * M * N > part_cap) --splits;
-            if (splits > 1) {
-                kps = (nk + splits - 1) / splits;
-                splits = (nk + kps - 1) / kps;  // every split has k-tiles
-            }
-        }
+        const Tiles t = gemm_tiles(M, N, K, e.mode == bbs::mlp::EPI_F32 && part != nullptr, part_cap, sms);
         CUtensorMap ta, tb;
-        if (!make_operand_map(&ta, A, M, K, lda, bbs::umma::kBM) || !make_operand_map(&tb, B, N, K, ldb, BN))
-            return cudaErrorInvalidValue;
-        const size_t smem = bbs::umma::smem_bytes(BN);
+        if (!gemm_maps(&ta, &tb, A, lda, B, ldb, M, N, K, t.BN)) return cudaErrorInvalidValue;
         static bool attr_set = false;
         if (!attr_set) {
-            cudaError_t a = cudaFuncSetAttribute(bbs::mlp::gemm_umma_kernel,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)bbs::umma::smem_bytes(64));
+            cudaError_t a = gemm_attr(bbs::mlp::gemm_umma_kernel);
             if (a != cudaSuccess) return a;
             attr_set = true;
         }
-        dim3 grid(nt, mt, splits);
-        if (splits == 1) {
-            bbs::mlp::gemm_umma_kernel<<<grid, 128, smem, st>>>(ta, tb, M, N, K, BN, kps, e, err);
+        dim3 grid(t.nt, t.mt, t.splits);
+        const size_t smem = bbs::umma::smem_bytes(t.BN);
+        if (t.splits == 1) {
+            bbs::mlp::gemm_umma_kernel<<<grid, bbs::umma::kThreads, smem, st>>>(ta, tb, M, N, K, t.BN, t.kps, e, err);
             return cudaGetLastError();
         }
         Epi pe = e;
         pe.c = part;
         pe.ldc = N;
         pe.zstride = (size_t)M * N;
-        bbs::mlp::gemm_umma_kernel<<<grid, 128, smem, st>>>(ta, tb, M, N, K, BN, kps, pe, err);
+        bbs::mlp::gemm_umma_kernel<<<grid, bbs::umma::kThreads, smem, st>>>(ta, tb, M, N, K, t.BN, t.kps, pe, err);
         const size_t total = (size_t)M * N;
         const int blocks = (int)std::min<size_t>((total + 255) / 256, (size_t)sms * 8);
-        bbs::mlp::splitk_reduce_kernel<<<blocks, 256, 0, st>>>(M, N, splits, part, e.c, e.ldc);
+        bbs::mlp::splitk_reduce_kernel<<<blocks, 256, 0, st>>>(M, N, t.splits, part, e.c, e.ldc);
         return cudaGetLastError();
     }
     dim3 grid((N + bbs::mlp::kBN - 1) / bbs::mlp::kBN, (M + bbs::mlp::kBM - 1) / bbs::mlp::kBM);
@@ -511,7 +737,7 @@ cudaError_t gemm_any(int kind, const __nv_bfloat16* A, int lda, const __nv_bfloa
 
 cudaError_t gemm(bbs_mlp* m, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M, int N,
                  int K, const Epi& e, cudaStream_t st) {
-    return gemm_any(m->gemm_kind, A, lda, B, ldb, M, N, K, e, m->err, st, m->part, m->part_cap, m->sms);
+    return gemm_any(m->gemm_kind, A, lda, B, ldb, M, N, K, e, m->err, st);
 }
 
 Epi epi_f32(float* c, int ldc) {
@@ -532,7 +758,10 @@ void pack_all(bbs_mlp* m, cudaStream_t st) {
 }
 
 // Forward pass of M rows of X [M, in_pad]; activations kept for backward.
-cudaError_t forward(bbs_mlp* m, const __nv_bfloat16* X, int M, bool keep_transposed, cudaStream_t st) {
+// With a loss (tcgen05 only) the last layer writes the output gradient D and
+// D^T and adds the mean squared error instead of storing its output.
+cudaError_t forward(bbs_mlp* m, const __nv_bfloat16* X, int M, bool keep_transposed, cudaStream_t st,
+                    float* loss = nullptr) {
     const __nv_bfloat16* h = X;
     int ldh = m->in_pad;
     cudaError_t e = cudaSuccess;
@@ -556,26 +785,32 @@ cudaError_t forward(bbs_mlp* m, const __nv_bfloat16* X, int M, bool keep_transpo
     ep.c = m->out;
     ep.ldc = m->n;
     ep.bias = m->p + m->off_b[3];
+    if (loss != nullptr) {
+        ep.mode = bbs::mlp::EPI_LOSS;
+        ep.z = m->T;
+        ep.ldz = m->n;
+        ep.y = m->D;  // its pad columns stay zero
+        ep.ldy = m->n_pad;
+        ep.yt = m->DT;
+        ep.ldyt = M;
+        ep.loss = loss;
+    }
     return gemm(m, h, ldh, m->Wb[3], m->pad_in[3], M, m->n, m->pad_in[3], ep, st);
 }
 
-// Loss and gradients of the minibatch in X/XT/T (M rows) into m->g.
+// Loss (cleared by the caller) and gradients of the minibatch in X/XT/T (M
+// rows) into m->g: forward, then the chain of the layers' output gradients,
+// then every weight gradient, which only reads them.
 cudaError_t backward(bbs_mlp* m, int M, float* loss, cudaStream_t st) {
     using namespace bbs::mlp;
-    cudaError_t e = forward(m, m->X, M, true, st);
+    const bool tc = m->gemm_kind == BBS_GEMM_TCGEN05;
+    cudaError_t e = forward(m, m->X, M, true, st, tc ? loss : nullptr);
     if (e != cudaSuccess) return e;
-    loss_kernel<<<M, 160, 0, st>>>(M, m->n, m->n_pad, m->out, m->T, m->D, m->DT, loss);
-    // layer 4
-    const __nv_bfloat16* dT = m->DT;  // [out_pad, M]
-    const __nv_bfloat16* d = m->D;    // [M, out_pad]
+    if (!tc) loss_kernel<<<M, 160, 0, st>>>(M, m->n, m->n_pad, m->out, m->T, m->D, m->DT, loss);
+    const __nv_bfloat16 *dT[kLayers], *d = m->D;  // [out, M] and [M, out_pad]
     int ld_d = m->n_pad;
-    for (int l = 3; l >= 0; --l) {
-        const int out = m->dims_out[l], in = m->dims_in[l];
-        // dW_l = d^T [out, M] . h_{l-1}^T [in, M]^T  -> [out, in]
-        const __nv_bfloat16* hT = (l == 0) ? m->XT : m->YT[l - 1];
-        if ((e = gemm(m, dT, M, hT, M, out, in, M, epi_f32(m->g + m->off_W[l], in), st)) != cudaSuccess) return e;
-        bias_grad_kernel<<<(out + 7) / 8, 256, 0, st>>>(out, M, dT, m->g + m->off_b[l]);
-        if (l == 0) break;
+    dT[kLayers - 1] = m->DT;
+    for (int l = kLayers - 1; l > 0; --l) {
         // d_{l-1} = (d . W_l) * gelu'(z_{l-1}):  [M, in] = d [M, out_pad] . W_l^T [in, out_pad]^T
         Epi ep{};
         ep.mode = EPI_GELU_BWD;
@@ -585,11 +820,55 @@ cudaError_t backward(bbs_mlp* m, int M, float* loss, cudaStream_t st) {
         ep.ldy = m->hidden;
         ep.yt = m->DZT[l - 1];
         ep.ldyt = M;
-        if ((e = gemm(m, d, ld_d, m->WTb[l], m->pad_out[l], M, in, m->pad_out[l], ep, st)) != cudaSuccess) return e;
+        if ((e = gemm(m, d, ld_d, m->WTb[l], m->pad_out[l], M, m->dims_in[l], m->pad_out[l], ep, st)) != cudaSuccess)
+            return e;
         d = m->DZ[l - 1];
-        dT = m->DZT[l - 1];
+        dT[l - 1] = m->DZT[l - 1];
         ld_d = m->hidden;
     }
+    // dW_l = d_l^T [out, M] . h_{l-1}^T [in, M]^T, the partial sums of the
+    // layers one after the other in m->part
+    WeightGrads w{};
+    GradSums g{};
+    size_t used = 0, reduce = 0;
+    for (int l = 0; l < kLayers; ++l) {
+        const int out = m->dims_out[l], in = m->dims_in[l];
+        const __nv_bfloat16* hT = l == 0 ? m->XT : m->YT[l - 1];
+        g.c[l] = m->g + m->off_W[l];
+        g.total[l] = (size_t)out * in;
+        g.splits[l] = 1;
+        g.dT[l] = dT[l];
+        g.db[l] = m->g + m->off_b[l];
+        g.first[l + 1] = g.first[l] + out;
+        if (!tc) {
+            if ((e = gemm(m, dT[l], M, hT, M, out, in, M, epi_f32(g.c[l], in), st)) != cudaSuccess) return e;
+            continue;
+        }
+        const Tiles t = gemm_tiles(out, in, M, true, m->part_cap, m->sms);
+        if (!gemm_maps(&w.a[l], &w.b[l], dT[l], M, hT, M, out, in, M, t.BN)) return cudaErrorInvalidValue;
+        w.M[l] = out, w.N[l] = in, w.BN[l] = t.BN, w.kps[l] = t.kps, w.nt[l] = t.nt, w.mt[l] = t.mt;
+        w.first[l + 1] = w.first[l] + t.nt * t.mt * t.splits;
+        w.epi[l] = epi_f32(g.c[l], in);
+        g.splits[l] = t.splits;
+        if (t.splits > 1) {
+            w.epi[l].c = m->part + used;
+            w.epi[l].zstride = g.total[l];
+            g.part[l] = m->part + used;
+            used += (size_t)t.splits * g.total[l];
+            reduce = std::max(reduce, g.total[l]);
+        }
+    }
+    if (tc) {
+        static bool attr_set = false;
+        if (!attr_set) {
+            if ((e = gemm_attr(weight_grads_kernel)) != cudaSuccess) return e;
+            attr_set = true;
+        }
+        weight_grads_kernel<<<w.first[kLayers], bbs::umma::kThreads, bbs::umma::smem_bytes(64), st>>>(w, M, m->err);
+    }
+    const int rb = (int)std::min<size_t>((reduce + 255) / 256, (size_t)m->sms * 8);
+    for (int l = 0; l <= kLayers; ++l) g.first[l] += rb;
+    grad_sums_kernel<<<g.first[kLayers], 256, 0, st>>>(g, M);
     return cudaGetLastError();
 }
 
@@ -639,18 +918,26 @@ bbs_status bbs_mlp_create(bbs_handle* h, int32_t n, int32_t hidden, uint64_t see
     ok = ok && dev_alloc(m, &m->X, MB * m->in_pad) && dev_alloc(m, &m->XT, MB * m->in_pad) &&
          dev_alloc(m, &m->T, MB * n) && dev_alloc(m, &m->out, MB * n) &&
          dev_alloc(m, &m->D, MB * m->n_pad) && dev_alloc(m, &m->DT, MB * m->n_pad) &&
-         dev_alloc(m, &m->idx, MB) && dev_alloc(m, &m->err, 1) && dev_alloc(m, &m->gate, 3);
+         dev_alloc(m, &m->err, 1) && dev_alloc(m, &m->gate, 3);
     for (int l = 0; l < 3 && ok; ++l)
         ok = dev_alloc(m, &m->Z[l], MB * hidden) && dev_alloc(m, &m->Y[l], MB * hidden) &&
              dev_alloc(m, &m->YT[l], MB * hidden) && dev_alloc(m, &m->DZ[l], MB * hidden) &&
              dev_alloc(m, &m->DZT[l], MB * hidden);
-    // split-K partials of the weight gradients: up to 32 splits of the largest [out, in]
+    // split-K partials of the weight gradients: a layer takes up to 32 splits of the largest [out, in]
     size_t wmax = 0;
     for (int l = 0; l < 4; ++l) wmax = std::max(wmax, (size_t)outs[l] * ins[l]);
     m->part_cap = 32 * wmax;
-    ok = ok && dev_alloc(m, &m->part, m->part_cap);
     cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, m->device);
     if (m->sms <= 0) m->sms = 152;
+    // all layers' at a time; a smaller minibatch is never split further
+    size_t psum = 0;
+    for (int l = 0; l < 4; ++l) {
+        const size_t total = (size_t)outs[l] * ins[l];
+        psum += max_splits(gemm_tiles(outs[l], ins[l], 0, false, 0, m->sms), max_batch / bbs::umma::kBK, total,
+                           m->part_cap, m->sms) *
+                total;
+    }
+    ok = ok && dev_alloc(m, &m->part, psum);
     if (!ok) {
         bbs_mlp_destroy(m);
         return errf(BBS_ERR_NO_MEMORY, "MLP buffers");
@@ -778,11 +1065,9 @@ bbs_status bbs_mlp_gradients(bbs_mlp* m, const uint16_t* feats, const float* tar
     if (M < 64 || M > m->max_batch || M % 64 != 0)
         return errf(BBS_ERR_INVALID_ARG, "minibatch must be a multiple of 64 up to %d", m->max_batch);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    cudaMemcpyAsync(m->idx, rows, sizeof(int32_t) * M, cudaMemcpyDeviceToDevice, st);
-    bbs::mlp::gather_kernel<<<M, 128, 0, st>>>(M, m->in_pad, m->n, m->idx,
-                                               reinterpret_cast<const __nv_bfloat16*>(feats), targets, m->X,
-                                               m->XT, m->T);
-    cudaMemsetAsync(loss, 0, sizeof(float), st);
+    bbs::mlp::gather_kernel<<<dim3(m->in_pad / 64, M / 64), 256, 0, st>>>(
+        M, m->in_pad, m->n, rows, reinterpret_cast<const __nv_bfloat16*>(feats), targets,
+        reinterpret_cast<uintptr_t>(feats) % 16 == 0, m->X, m->XT, m->T, loss);
     cudaError_t e = backward(m, M, loss, st);
     return e == cudaSuccess ? BBS_OK : errf(BBS_ERR_CUDA, "%s", cudaGetErrorString(e));
 }
@@ -794,9 +1079,13 @@ bbs_status bbs_mlp_train_step(bbs_mlp* m, const uint16_t* feats, const float* ta
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     m->adam_t += 1;
     const float c1 = 1.0f - powf(0.9f, (float)m->adam_t), c2 = 1.0f - powf(0.999f, (float)m->adam_t);
+    bbs::mlp::Layers w;
+    for (int l = 0; l < bbs::mlp::kLayers; ++l) {
+        w.off_W[l] = (int)m->off_W[l], w.out[l] = m->dims_out[l], w.in[l] = m->dims_in[l];
+        w.in_pad[l] = m->pad_in[l], w.out_pad[l] = m->pad_out[l], w.Wb[l] = m->Wb[l], w.WTb[l] = m->WTb[l];
+    }
     bbs::mlp::adam_kernel<<<(unsigned)std::min<size_t>((m->count + 255) / 256, 2048), 256, 0, st>>>(
-        m->count, m->p, m->g, m->m, m->v, lr, 0.9f, 0.999f, 1e-8f, c1, c2);
-    pack_all(m, st);
+        m->count, m->p, m->g, m->m, m->v, lr, 0.9f, 0.999f, 1e-8f, c1, c2, w);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? BBS_OK : errf(BBS_ERR_CUDA, "%s", cudaGetErrorString(e));
 }

@@ -3,20 +3,25 @@
 //   C[m][n] = sum_k A[m*lda + k] * B[n*ldb + k]     (both operands K-major)
 // K must be a multiple of 64 and the row strides multiples of 8 elements.
 //
-// One block of 4 warps computes a 128 x BN tile (BN a multiple of 16, <= 256)
-// over the k-tiles [kt0, kt1) of its split (blockIdx.z):
+// One block of 8 warps computes a 128 x BN tile (BN a multiple of 16, <= 256)
+// over the k-tiles [kt0, kt1) of its split:
 //   * thread 0 of warp 0 is the producer: for each 64-wide k-tile it issues
-//     TMA copies (cp.async.bulk.tensor.2d) of eight 16-byte-wide column boxes
-//     of A (128 rows) and of B (BN rows) into one of kStages stages, laid out
-//     as the no-swizzle K-major "core matrix" canonical form (8 rows x 16
-//     bytes per 128-byte core matrix; 8-row groups 128 bytes apart, 16-byte
-//     K chunks 16 * rows bytes apart), and arms the stage's "full" mbarrier
-//     with the byte count;
+//     one TMA copy (cp.async.bulk.tensor.2d) of A (128 rows x 128 bytes) and
+//     one of B (BN rows) into one of kStages stages in the 128-byte swizzle,
+//     and arms the stage's "full" mbarrier with the byte count;
 //   * thread 0 of warp 1 issues four tcgen05.mma (M = 128, N = BN, K = 16)
 //     per k-tile once the stage is full, and tcgen05.commit frees the stage
 //     through its "empty" mbarrier; a last commit signals "done";
-//   * then every warp reads its 32 accumulator lanes (rows) with tcgen05.ld
-//     and runs the epilogue functor epi(m, n, value).
+//   * then the warps move the accumulator from tensor memory into the stages'
+//     shared memory (FP32, one word of padding per row) and the epilogue
+//     walks the tile from there, along rows for row-major operands and along
+//     columns for the transposed copy.
+// The GEMMs here are small (thousands of rows by a few hundred), so what a
+// tile costs around its MMAs decides. With a thread's accumulator row written
+// straight to memory each store touched 32 rows, and with 16-byte boxes each
+// k-tile took 16 copies of 16-byte lines: 36 us for [4096 x 256] from K = 256
+// with bias, GELU, pre-activation and both BF16 copies, against the 3 us that
+// its bytes take; see gemm_umma_kernel for what it takes now.
 // Rows past M and N are zero-filled by TMA. Every mbarrier wait is bounded;
 // a wait that runs out sets *err, the block stops issuing, waits (bounded)
 // for the copies and MMAs it already issued, and still frees its tensor
@@ -32,7 +37,7 @@
 namespace bbs {
 namespace umma {
 
-constexpr int kBM = 128, kBK = 64, kStages = 4;
+constexpr int kBM = 128, kBK = 64, kStages = 4, kThreads = 256;
 constexpr int kWaitIters = 1 << 22;
 
 __device__ __forceinline__ uint32_t saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -47,6 +52,13 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
     d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
     d |= (uint64_t)1 << 46;
     return d;
+}
+
+// The same for the 128-byte swizzle: rows of 128 bytes (64 BF16 of K) in
+// atoms of 8 rows, 1,024 bytes apart; a step of 16 in K adds 32 bytes to the
+// start address. The leading offset is not used.
+__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
+    return smem_desc(addr, 16, 1024) | (uint64_t)2 << 61;
 }
 
 // Instruction descriptor, kind::f16: D = F32, A = B = BF16, both K-major.
@@ -117,15 +129,16 @@ __host__ __device__ constexpr size_t smem_bytes(int BN) { return kStages * stage
 
 template <class Epi>
 __device__ __forceinline__ void gemm_tn_tma(const CUtensorMap* ta, const CUtensorMap* tb, int M, int N, int K,
-                                            int BN, int ktiles_per_split, const Epi& epi, int* err) {
+                                            int BN, int bx, int by, int bz, int ktiles_per_split, const Epi& epi,
+                                            int* err) {
     extern __shared__ unsigned char smem_raw[];
     // TMA destinations and MMA operands: 1024-byte aligned base
     unsigned char* smem = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.y * kBM, n0 = blockIdx.x * BN;
+    const int m0 = by * kBM, n0 = bx * BN;
     const int nk = K / kBK;
-    const int kt0 = blockIdx.z * ktiles_per_split;
+    const int kt0 = bz * ktiles_per_split;
     const int kt1 = min(nk, kt0 + ktiles_per_split);
     const uint32_t a_bytes = kBM * kBK * 2, b_bytes = (uint32_t)BN * kBK * 2;
     const uint32_t sbytes = a_bytes + b_bytes;
@@ -135,8 +148,6 @@ __device__ __forceinline__ void gemm_tn_tma(const CUtensorMap* ta, const CUtenso
     uint64_t* done = bars + 2 * kStages;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
     const uint32_t tmem_cols = BN <= 32 ? 32u : BN <= 64 ? 64u : BN <= 128 ? 128u : 256u;
-    // K-major no-swizzle layout written by the column boxes
-    const uint32_t lbo_a = kBM * 16, lbo_b = (uint32_t)BN * 16, sbo = 128;
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(saddr(tmem_slot)),
@@ -171,11 +182,8 @@ __device__ __forceinline__ void gemm_tn_tma(const CUtensorMap* ta, const CUtenso
             const uint32_t a = base + s * sbytes, b = a + a_bytes, fb = saddr(&full[s]);
             mbar_expect_tx(fb, sbytes);
             const int k0 = kt * kBK;
-#pragma unroll
-            for (int kc = 0; kc < kBK / 8; ++kc) {
-                tma_load_2d(a + kc * lbo_a, ta, k0 + 8 * kc, m0, fb);
-                tma_load_2d(b + kc * lbo_b, tb, k0 + 8 * kc, n0, fb);
-            }
+            tma_load_2d(a, ta, k0, m0, fb);
+            tma_load_2d(b, tb, k0, n0, fb);
         }
         // the copies of the last (up to kStages) stages land before the block
         // ends, whether or not the MMA side consumed them
@@ -193,8 +201,8 @@ __device__ __forceinline__ void gemm_tn_tma(const CUtensorMap* ta, const CUtenso
             const uint32_t a = base + s * sbytes, b = a + a_bytes;
 #pragma unroll
             for (int ks = 0; ks < kBK / 16; ++ks)
-                umma_bf16(tmem, smem_desc(a + ks * 2 * lbo_a, lbo_a, sbo), smem_desc(b + ks * 2 * lbo_b, lbo_b, sbo),
-                          idesc, (i > 0 || ks > 0) ? 1u : 0u);
+                umma_bf16(tmem, smem_desc_sw128(a + ks * 32), smem_desc_sw128(b + ks * 32), idesc,
+                          (i > 0 || ks > 0) ? 1u : 0u);
             umma_commit(saddr(&empty[s]));
         }
         umma_commit(saddr(done));  // arrives once every MMA issued above has completed
@@ -203,18 +211,18 @@ __device__ __forceinline__ void gemm_tn_tma(const CUtensorMap* ta, const CUtenso
     ok = __syncthreads_and(ok ? 1 : 0) != 0;  // the tensor-memory loads below are warp-collective
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     if (ok && kt1 > kt0) {
-        const int m = m0 + warp * 32 + lane;
-        for (int c0 = 0; c0 < BN; c0 += 16) {
+        // every copy has landed and every MMA has read its operands: the
+        // stages are free for the tile
+        float* tile = reinterpret_cast<float*>(smem);
+        const int q = warp & 3, row = q * 32 + lane;
+        for (int c0 = (warp >> 2) * 16; c0 < BN; c0 += 32) {
             uint32_t v[16];
-            tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-            if (m < M) {
+            tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int n = n0 + c0 + j;
-                    if (n < N && c0 + j < BN) epi(m, n, __uint_as_float(v[j]));
-                }
-            }
+            for (int j = 0; j < 16; ++j) tile[row * (BN + 1) + c0 + j] = __uint_as_float(v[j]);
         }
+        __syncthreads();
+        epi.tile(tile, BN, m0, n0, M, N, bz);
     } else if (!ok && tid == 0) {
         atomicExch(err, 1);
     }
