@@ -51,6 +51,15 @@ __device__ __forceinline__ float gelu_grad(float z) {
     return 0.5f * (1.0f + t) + 0.5f * z * (1.0f - t * t) * du;
 }
 
+// Sum over a block of 256 threads, in a tree; thread 0 has it.
+__device__ __forceinline__ float block_tree_sum(float s) {
+    for (int k = 16; k; k >>= 1) s += __shfl_xor_sync(0xffffffffu, s, k);
+    __shared__ float ws[8];
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
+    __syncthreads();
+    return ((ws[0] + ws[1]) + (ws[2] + ws[3])) + ((ws[4] + ws[5]) + (ws[6] + ws[7]));
+}
+
 // ---------------------------------------------------------- epilogues
 
 enum EpiMode { EPI_F32 = 0, EPI_BIAS_GELU = 1, EPI_BIAS = 2, EPI_GELU_BWD = 3, EPI_LOSS = 4 };
@@ -67,7 +76,7 @@ struct Epi {
     int ldyt;
     const float* z;           // EPI_GELU_BWD: pre-activation of the layer below; EPI_LOSS: targets
     int ldz;
-    float* loss;              // EPI_LOSS: the mean squared error is added here
+    float* loss;              // EPI_LOSS: the tile's sum of squared errors, one per block
 
     // One element; the mma.sync GEMM calls it (no split, no EPI_LOSS).
     __device__ __forceinline__ void operator()(int m, int n, float v) const {
@@ -95,28 +104,29 @@ struct Epi {
         }
     }
 
-    // Rows warp, warp + 8, ... of one column of the tile (lanes are
+    // Rows r0, r0 + step, ... of one column of the tile (lanes are
     // neighbouring columns), eight rows' loads in flight at a time. With yt
     // the BF16 result takes the accumulator's place in the tile.
     template <int MODE>
-    __device__ __forceinline__ float column(float* t, int ld, int r0, int c0, int m0, int n0, int M, int bz) const {
-        constexpr int kWarps = umma::kThreads / 32, kU = 8;
+    __device__ __forceinline__ float column(float* t, int ld, int r0, int step, int c0, int m0, int n0, int M,
+                                            int bz) const {
+        constexpr int kU = 8;
         const int n = n0 + c0;
         const float bn = MODE == EPI_F32 || MODE == EPI_GELU_BWD ? 0.0f : bias[n];
         const float scale = MODE == EPI_LOSS ? 2.0f / ((float)M * (float)ldc) : 0.0f;
         float acc = 0.0f;
-        for (int i = r0; i < umma::kBM; i += kU * kWarps) {
+        for (int i = r0; i < umma::kBM; i += kU * step) {
             float in[kU];
             if (MODE == EPI_GELU_BWD || MODE == EPI_LOSS) {
 #pragma unroll
                 for (int u = 0; u < kU; ++u) {
-                    const int m = m0 + i + u * kWarps;
+                    const int m = m0 + i + u * step;
                     in[u] = m < M ? __ldg(z + (size_t)m * ldz + n) : 0.0f;
                 }
             }
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
-                const int r = i + u * kWarps, m = m0 + r;
+                const int r = i + u * step, m = m0 + r;
                 if (m >= M) continue;
                 float* at = t + r * ld + c0;
                 float v = *at + bn;
@@ -149,18 +159,20 @@ struct Epi {
     __device__ __forceinline__ void tile(float* t, int BN, int m0, int n0, int M, int N, int bz) const {
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ld = BN + 1;
         float acc = 0.0f;
-        for (int c0 = lane; c0 < BN && n0 + c0 < N; c0 += 32) {
+        const bool pair = BN == 16;  // a warp then takes two rows at a time
+        const int r0 = pair ? 2 * warp + (lane >> 4) : warp, step = (pair ? 2 : 1) * (umma::kThreads / 32);
+        for (int c0 = pair ? lane & 15 : lane; c0 < BN && n0 + c0 < N; c0 += 32) {
             switch (mode) {
-                case EPI_F32: column<EPI_F32>(t, ld, warp, c0, m0, n0, M, bz); break;
-                case EPI_BIAS: column<EPI_BIAS>(t, ld, warp, c0, m0, n0, M, bz); break;
-                case EPI_BIAS_GELU: column<EPI_BIAS_GELU>(t, ld, warp, c0, m0, n0, M, bz); break;
-                case EPI_GELU_BWD: column<EPI_GELU_BWD>(t, ld, warp, c0, m0, n0, M, bz); break;
-                default: acc += column<EPI_LOSS>(t, ld, warp, c0, m0, n0, M, bz); break;
+                case EPI_F32: column<EPI_F32>(t, ld, r0, step, c0, m0, n0, M, bz); break;
+                case EPI_BIAS: column<EPI_BIAS>(t, ld, r0, step, c0, m0, n0, M, bz); break;
+                case EPI_BIAS_GELU: column<EPI_BIAS_GELU>(t, ld, r0, step, c0, m0, n0, M, bz); break;
+                case EPI_GELU_BWD: column<EPI_GELU_BWD>(t, ld, r0, step, c0, m0, n0, M, bz); break;
+                default: acc += column<EPI_LOSS>(t, ld, r0, step, c0, m0, n0, M, bz); break;
             }
         }
         if (mode == EPI_LOSS) {
-            for (int k = 16; k; k >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, k);
-            if (lane == 0) atomicAdd(loss, acc / ((float)M * (float)ldc));
+            acc = block_tree_sum(acc);
+            if (threadIdx.x == 0) loss[blockIdx.y * gridDim.x + blockIdx.x] = acc;
         }
         if (yt == nullptr) return;  // the same for every thread
         __syncthreads();
@@ -186,9 +198,11 @@ __global__ void __launch_bounds__(256) gemm_kernel(const __nv_bfloat16* __restri
     gemm_tn_mma<Epi>(A, lda, B, ldb, M, N, K, epi);
 }
 
-// [4096 x 256] from K = 256 with GELU: 36 -> 12 us; with the GELU gradient
-// 28 -> 14 us (one launch from cold caches). What is left is latency: launch,
-// copies, one wave of 128 blocks' epilogues.
+// [4096 x 256] from K = 256 with GELU: 36 -> 10 us; with the GELU gradient
+// 28 -> 11 us (one launch from cold caches). What is left is latency: launch,
+// copies, one wave of 256 blocks' epilogues. Launches overlap in a step (the
+// next kernel sets up while this one runs): 138 -> 103 us with the narrower
+// tiles and the sums below.
 __global__ void __launch_bounds__(umma::kThreads, 2) gemm_umma_kernel(const __grid_constant__ CUtensorMap ta,
                                                                       const __grid_constant__ CUtensorMap tb, int M,
                                                                       int N, int K, int BN, int ktiles_per_split,
@@ -231,37 +245,87 @@ __global__ void splitk_reduce_kernel(int M, int N, int splits, const float* __re
     }
 }
 
-// What is left of all layers' gradients, in one launch: the split-K sums
-// (blocks below first[0]; splits <= 1 leaves a layer's as they are) and, one
-// block per output, the bias gradients db[j] = sum of row j of dT [N, M].
-// One warp a row with 2-byte loads took 10 us a layer, most of it waiting;
-// a block reads the row in one or two 16-byte loads per thread (M is a
-// multiple of 64) and adds in a tree, so its chains are shorter too.
-struct GradSums {
-    const float* part[kLayers];
-    float* c[kLayers];
-    size_t total[kLayers];
-    int splits[kLayers];
-    const __nv_bfloat16* dT[kLayers];
-    float* db[kLayers];
-    int first[kLayers + 1];  // first bias block of each layer
+struct Layers {
+    int off_W[kLayers], off_b[kLayers], out[kLayers], in[kLayers], in_pad[kLayers], out_pad[kLayers];
+    __nv_bfloat16 *Wb[kLayers], *WTb[kLayers];
 };
 
-__global__ void __launch_bounds__(256) grad_sums_kernel(const __grid_constant__ GradSums g, int M) {
+struct Adam {
+    float *p, *m, *v;
+    float lr, b1, b2, eps, c1, c2;
+};
+
+// One parameter's step and, of a weight, the BF16 copies of what it becomes
+// (their pads stay zero). Element e of layer l, parameter i in all.
+__device__ __forceinline__ void adam_update(const Adam& a, const Layers& w, int l, int e, int i, float gi) {
+    const float mi = a.b1 * a.m[i] + (1.0f - a.b1) * gi;
+    const float vi = a.b2 * a.v[i] + (1.0f - a.b2) * gi * gi;
+    a.m[i] = mi;
+    a.v[i] = vi;
+    const float pi = a.p[i] - a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
+    a.p[i] = pi;
+    if (i < w.off_b[l]) {
+        const int r = e / w.in[l], k = e - r * w.in[l];
+        const __nv_bfloat16 h = __float2bfloat16_rn(pi);
+        w.Wb[l][(size_t)r * w.in_pad[l] + k] = h;
+        w.WTb[l][(size_t)k * w.out_pad[l] + r] = h;
+    }
+}
+
+// What is left of all layers' gradients, in one launch, and with ADAM the
+// step that they are for:
+//   * blocks below first[0]: one thread per weight adds its split-K parts
+//     (splits <= 1: the GEMM has left the gradient in g);
+//   * then one block per output: the bias gradient db[j] = sum of row j of dT
+//     [N, M]. One warp a row with 2-byte loads took 10 us a layer, most of it
+//     waiting; a block reads the row in one or two 16-byte loads per thread
+//     (M is a multiple of 64) and adds in a tree, so its chains are shorter;
+//   * with loss_parts, a last block that adds the tiles' losses, in a tree too
+//     (an atomic per row into one FP32 sum was less exact, and its last bits
+//     changed from run to run).
+// As eight launches of sums, one of Adam and four that packed the BF16 weights
+// this took 81 us a step of n = 144, hidden 256, M = 4096, nearly all of it
+// launches and latency: 12 us now, from cold caches.
+struct GradSums {
+    Layers w;
+    float* g;
+    int count;
+    const float* part[kLayers];
+    int splits[kLayers];
+    const __nv_bfloat16* dT[kLayers];
+    int first[kLayers + 1];  // first bias block of each layer
+    const float* loss_part;
+    int loss_parts;
+    float* loss;
+};
+
+template <bool ADAM>
+__global__ void __launch_bounds__(256) grad_sums_kernel(const __grid_constant__ GradSums g, int M, Adam a) {
+    umma::grid_wait();
     if ((int)blockIdx.x < g.first[0]) {
-        for (int l = 0; l < kLayers; ++l) {
-            const int splits = g.splits[l];
-            if (splits <= 1) continue;
-            const size_t total = g.total[l];
-            const float* __restrict__ part = g.part[l];
-            for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-                 i += (size_t)g.first[0] * blockDim.x) {
-                float s = 0.0f;
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.count; i += g.first[0] * blockDim.x) {
+            int l = 0;
+            while (l + 1 < kLayers && i >= g.w.off_W[l + 1]) ++l;
+            if (i >= g.w.off_b[l]) continue;
+            const int e = i - g.w.off_W[l], total = g.w.off_b[l] - g.w.off_W[l], splits = g.splits[l];
+            float s = 0.0f;
+            if (splits > 1) {
+                const float* __restrict__ part = g.part[l] + e;
 #pragma unroll 8
-                for (int z = 0; z < splits; ++z) s += __ldg(part + (size_t)z * total + i);
-                g.c[l][i] = s;
+                for (int z = 0; z < splits; ++z) s += __ldg(part + (size_t)z * total);
+                g.g[i] = s;
+            } else if (ADAM) {
+                s = g.g[i];
             }
+            if (ADAM) adam_update(a, g.w, l, e, i, s);
         }
+        return;
+    }
+    if ((int)blockIdx.x >= g.first[kLayers]) {
+        float s = 0.0f;
+        for (int i = threadIdx.x; i < g.loss_parts; i += blockDim.x) s += g.loss_part[i];
+        s = block_tree_sum(s);
+        if (threadIdx.x == 0) *g.loss = s / ((float)M * (float)g.w.out[kLayers - 1]);
         return;
     }
     int l = 0;
@@ -280,12 +344,12 @@ __global__ void __launch_bounds__(256) grad_sums_kernel(const __grid_constant__ 
         }
         s += (p[0] + p[1]) + (p[2] + p[3]);
     }
-    for (int k = 16; k; k >>= 1) s += __shfl_xor_sync(0xffffffffu, s, k);
-    __shared__ float ws[8];
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0)
-        g.db[l][j] = ((ws[0] + ws[1]) + (ws[2] + ws[3])) + ((ws[4] + ws[5]) + (ws[6] + ws[7]));
+    s = block_tree_sum(s);
+    if (threadIdx.x == 0) {
+        const int i = g.w.off_b[l] + j;
+        g.g[i] = s;
+        if (ADAM) adam_update(a, g.w, l, 0, i, s);
+    }
 }
 
 // ---------------------------------------------------- small kernels
@@ -381,6 +445,7 @@ __global__ void __launch_bounds__(256) gather_kernel(int M, int in_pad, int n, c
                                                      __nv_bfloat16* __restrict__ X, __nv_bfloat16* __restrict__ XT,
                                                      float* __restrict__ T, float* __restrict__ loss) {
     __shared__ __nv_bfloat16 t[64][66];
+    umma::grid_release();
     const int tid = threadIdx.x, f0 = blockIdx.x * 64, r0 = blockIdx.y * 64;
     if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *loss = 0.0f;
     const int c = (tid & 7) * 8;
@@ -434,36 +499,6 @@ __global__ void loss_kernel(int M, int n, int n_pad, const float* __restrict__ o
         float s = 0.0f;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += part[w];
         atomicAdd(loss, s / ((float)M * (float)n));
-    }
-}
-
-// Adam, and the BF16 copies of the new weights (pads stay zero): the four
-// packing launches that followed took 4 us each, next to nothing of it work.
-struct Layers {
-    int off_W[kLayers], out[kLayers], in[kLayers], in_pad[kLayers], out_pad[kLayers];
-    __nv_bfloat16 *Wb[kLayers], *WTb[kLayers];
-};
-
-__global__ void adam_kernel(size_t count, float* __restrict__ p, const float* __restrict__ g,
-                            float* __restrict__ m, float* __restrict__ v, float lr, float b1, float b2,
-                            float eps, float c1, float c2, const __grid_constant__ Layers w) {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.0f - b1) * gi;
-        const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-        p[i] = pi;
-        int l = 0;
-        while (l + 1 < kLayers && (int)i >= w.off_W[l + 1]) ++l;
-        const int e = (int)i - w.off_W[l], r = e / w.in[l], k = e - r * w.in[l];
-        if (r < w.out[l]) {  // past the weights: the layer's biases
-            const __nv_bfloat16 h = __float2bfloat16_rn(pi);
-            w.Wb[l][(size_t)r * w.in_pad[l] + k] = h;
-            w.WTb[l][(size_t)k * w.out_pad[l] + r] = h;
-        }
     }
 }
 
@@ -583,6 +618,7 @@ struct bbs_mlp {
     __nv_bfloat16* DZT[3] = {};
     int* err = nullptr;     // set by a tensor-core GEMM whose waits ran out
     double* gate = nullptr;  // [gamma, sum c.d, sum c.c] (see bbs_mlp_gate_observe)
+    float* loss_part = nullptr;  // one per tile of the output layer
     float* part = nullptr;  // split-K partial sums of the weight-gradient GEMMs
     size_t part_cap = 0;    // floats one layer may take of it
     int sms = 0;
@@ -654,7 +690,10 @@ bool make_operand_map(CUtensorMap* map, const __nv_bfloat16* ptr, int rows, int 
 }
 
 // Tiles and splits of a tcgen05 GEMM: 128 rows x BN columns, BN <= 64 so that
-// the layer GEMMs over thousands of samples launch hundreds of blocks. An
+// the layer GEMMs over thousands of samples launch hundreds of blocks, and
+// narrower while a GEMM that is not split leaves SMs without a block: its
+// epilogue is most of it, and halves with the tile (12 -> 10 us for [4096 x
+// 256] from K = 256, BN 64 -> 32). An
 // FP32-output GEMM with few tiles and a long K (the weight gradients, K =
 // samples) is split over K when part_cap floats have room: each split writes
 // its partial tile, which are then added in a fixed order.
@@ -678,6 +717,10 @@ Tiles gemm_tiles(int M, int N, int K, bool split, size_t part_cap, int sms) {
     t.nt = (N + t.BN - 1) / t.BN;
     const int nk = K / bbs::umma::kBK;
     t.splits = 1, t.kps = nk;
+    while (!split && t.BN > 16 && t.mt * t.nt < sms) {
+        t.BN = round_up(t.BN / 2, 16);
+        t.nt = (N + t.BN - 1) / t.BN;
+    }
     if (split) {
         t.splits = max_splits(t, nk, (size_t)M * N, part_cap, sms);
         if (t.splits > 1) {
@@ -686,6 +729,22 @@ Tiles gemm_tiles(int M, int N, int K, bool split, size_t part_cap, int sms) {
         }
     }
     return t;
+}
+
+// Launch that may begin before the stream's last kernel ends (umma::grid_wait).
+template <class... P, class... A>
+cudaError_t launch_early(void (*k)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, const A&... args) {
+    cudaLaunchConfig_t c{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.gridDim = grid;
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, k, args...);
 }
 
 bool gemm_maps(CUtensorMap* ta, CUtensorMap* tb, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb,
@@ -717,8 +776,8 @@ cudaError_t gemm_any(int kind, const __nv_bfloat16* A, int lda, const __nv_bfloa
         dim3 grid(t.nt, t.mt, t.splits);
         const size_t smem = bbs::umma::smem_bytes(t.BN);
         if (t.splits == 1) {
-            bbs::mlp::gemm_umma_kernel<<<grid, bbs::umma::kThreads, smem, st>>>(ta, tb, M, N, K, t.BN, t.kps, e, err);
-            return cudaGetLastError();
+            return launch_early(bbs::mlp::gemm_umma_kernel, grid, bbs::umma::kThreads, smem, st, ta, tb, M, N, K, t.BN,
+                                t.kps, e, err);
         }
         Epi pe = e;
         pe.c = part;
@@ -737,7 +796,7 @@ cudaError_t gemm_any(int kind, const __nv_bfloat16* A, int lda, const __nv_bfloa
 
 cudaError_t gemm(bbs_mlp* m, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M, int N,
                  int K, const Epi& e, cudaStream_t st) {
-    return gemm_any(m->gemm_kind, A, lda, B, ldb, M, N, K, e, m->err, st);
+    return gemm_any(m->gemm_kind, A, lda, B, ldb, M, N, K, e, m->err, st, nullptr, 0, m->sms);
 }
 
 Epi epi_f32(float* c, int ldc) {
@@ -758,8 +817,8 @@ void pack_all(bbs_mlp* m, cudaStream_t st) {
 }
 
 // Forward pass of M rows of X [M, in_pad]; activations kept for backward.
-// With a loss (tcgen05 only) the last layer writes the output gradient D and
-// D^T and adds the mean squared error instead of storing its output.
+// With loss parts (tcgen05 only) the last layer writes the output gradient D
+// and D^T and a sum of squared errors per tile instead of its output.
 cudaError_t forward(bbs_mlp* m, const __nv_bfloat16* X, int M, bool keep_transposed, cudaStream_t st,
                     float* loss = nullptr) {
     const __nv_bfloat16* h = X;
@@ -800,11 +859,12 @@ cudaError_t forward(bbs_mlp* m, const __nv_bfloat16* X, int M, bool keep_transpo
 
 // Loss (cleared by the caller) and gradients of the minibatch in X/XT/T (M
 // rows) into m->g: forward, then the chain of the layers' output gradients,
-// then every weight gradient, which only reads them.
-cudaError_t backward(bbs_mlp* m, int M, float* loss, cudaStream_t st) {
+// then every weight gradient, which only reads them, and the optimiser's step
+// if there is one.
+cudaError_t backward(bbs_mlp* m, int M, float* loss, const bbs::mlp::Adam* adam, cudaStream_t st) {
     using namespace bbs::mlp;
     const bool tc = m->gemm_kind == BBS_GEMM_TCGEN05;
-    cudaError_t e = forward(m, m->X, M, true, st, tc ? loss : nullptr);
+    cudaError_t e = forward(m, m->X, M, true, st, tc ? m->loss_part : nullptr);
     if (e != cudaSuccess) return e;
     if (!tc) loss_kernel<<<M, 160, 0, st>>>(M, m->n, m->n_pad, m->out, m->T, m->D, m->DT, loss);
     const __nv_bfloat16 *dT[kLayers], *d = m->D;  // [out, M] and [M, out_pad]
@@ -830,32 +890,43 @@ cudaError_t backward(bbs_mlp* m, int M, float* loss, cudaStream_t st) {
     // layers one after the other in m->part
     WeightGrads w{};
     GradSums g{};
-    size_t used = 0, reduce = 0;
+    g.g = m->g;
+    g.count = (int)m->count;
+    if (tc) {
+        const Tiles t = gemm_tiles(M, m->n, m->pad_in[kLayers - 1], false, 0, m->sms);  // the last layer's
+        g.loss_part = m->loss_part;
+        g.loss_parts = t.mt * t.nt;
+        g.loss = loss;
+    }
+    size_t used = 0;
+    bool walk = adam != nullptr;  // over the weights
     for (int l = 0; l < kLayers; ++l) {
         const int out = m->dims_out[l], in = m->dims_in[l];
+        const size_t total = (size_t)out * in;
+        float* dW = m->g + m->off_W[l];
         const __nv_bfloat16* hT = l == 0 ? m->XT : m->YT[l - 1];
-        g.c[l] = m->g + m->off_W[l];
-        g.total[l] = (size_t)out * in;
+        g.w.off_W[l] = (int)m->off_W[l], g.w.off_b[l] = (int)m->off_b[l];
+        g.w.out[l] = out, g.w.in[l] = in, g.w.in_pad[l] = m->pad_in[l], g.w.out_pad[l] = m->pad_out[l];
+        g.w.Wb[l] = m->Wb[l], g.w.WTb[l] = m->WTb[l];
         g.splits[l] = 1;
         g.dT[l] = dT[l];
-        g.db[l] = m->g + m->off_b[l];
         g.first[l + 1] = g.first[l] + out;
         if (!tc) {
-            if ((e = gemm(m, dT[l], M, hT, M, out, in, M, epi_f32(g.c[l], in), st)) != cudaSuccess) return e;
+            if ((e = gemm(m, dT[l], M, hT, M, out, in, M, epi_f32(dW, in), st)) != cudaSuccess) return e;
             continue;
         }
         const Tiles t = gemm_tiles(out, in, M, true, m->part_cap, m->sms);
         if (!gemm_maps(&w.a[l], &w.b[l], dT[l], M, hT, M, out, in, M, t.BN)) return cudaErrorInvalidValue;
         w.M[l] = out, w.N[l] = in, w.BN[l] = t.BN, w.kps[l] = t.kps, w.nt[l] = t.nt, w.mt[l] = t.mt;
         w.first[l + 1] = w.first[l] + t.nt * t.mt * t.splits;
-        w.epi[l] = epi_f32(g.c[l], in);
+        w.epi[l] = epi_f32(dW, in);
         g.splits[l] = t.splits;
         if (t.splits > 1) {
             w.epi[l].c = m->part + used;
-            w.epi[l].zstride = g.total[l];
+            w.epi[l].zstride = total;
             g.part[l] = m->part + used;
-            used += (size_t)t.splits * g.total[l];
-            reduce = std::max(reduce, g.total[l]);
+            used += (size_t)t.splits * total;
+            walk = true;
         }
     }
     if (tc) {
@@ -864,12 +935,14 @@ cudaError_t backward(bbs_mlp* m, int M, float* loss, cudaStream_t st) {
             if ((e = gemm_attr(weight_grads_kernel)) != cudaSuccess) return e;
             attr_set = true;
         }
-        weight_grads_kernel<<<w.first[kLayers], bbs::umma::kThreads, bbs::umma::smem_bytes(64), st>>>(w, M, m->err);
+        if ((e = launch_early(weight_grads_kernel, dim3(w.first[kLayers]), bbs::umma::kThreads,
+                              bbs::umma::smem_bytes(64), st, w, M, m->err)) != cudaSuccess)
+            return e;
     }
-    const int rb = (int)std::min<size_t>((reduce + 255) / 256, (size_t)m->sms * 8);
+    const int rb = walk ? (int)std::min<size_t>((m->count + 255) / 256, (size_t)m->sms * 16) : 0;
     for (int l = 0; l <= kLayers; ++l) g.first[l] += rb;
-    grad_sums_kernel<<<g.first[kLayers], 256, 0, st>>>(g, M);
-    return cudaGetLastError();
+    return launch_early(adam ? grad_sums_kernel<true> : grad_sums_kernel<false>, dim3(g.first[kLayers] + (tc ? 1 : 0)), 256, 0, st, g,
+                        M, adam ? *adam : Adam{});
 }
 
 }  // namespace
@@ -933,11 +1006,12 @@ bbs_status bbs_mlp_create(bbs_handle* h, int32_t n, int32_t hidden, uint64_t see
     size_t psum = 0;
     for (int l = 0; l < 4; ++l) {
         const size_t total = (size_t)outs[l] * ins[l];
-        psum += max_splits(gemm_tiles(outs[l], ins[l], 0, false, 0, m->sms), max_batch / bbs::umma::kBK, total,
+        psum += max_splits(gemm_tiles(outs[l], ins[l], 0, true, 0, m->sms), max_batch / bbs::umma::kBK, total,
                            m->part_cap, m->sms) *
                 total;
     }
     ok = ok && dev_alloc(m, &m->part, psum);
+    ok = ok && dev_alloc(m, &m->loss_part, (size_t)((max_batch + bbs::umma::kBM - 1) / bbs::umma::kBM) * ((n + 15) / 16));
     if (!ok) {
         bbs_mlp_destroy(m);
         return errf(BBS_ERR_NO_MEMORY, "MLP buffers");
@@ -1059,8 +1133,8 @@ bbs_status bbs_mlp_make_samples(bbs_mlp* m, const bbs_batch_matrix* A, const dou
     return e == cudaSuccess ? BBS_OK : errf(BBS_ERR_CUDA, "%s", cudaGetErrorString(e));
 }
 
-bbs_status bbs_mlp_gradients(bbs_mlp* m, const uint16_t* feats, const float* targets, const int32_t* rows,
-                             int32_t M, float* loss, void* stream) {
+static bbs_status gradients(bbs_mlp* m, const uint16_t* feats, const float* targets, const int32_t* rows, int32_t M,
+                            float* loss, const bbs::mlp::Adam* adam, void* stream) {
     if (m == nullptr || !feats || !targets || !rows || !loss) return errf(BBS_ERR_INVALID_ARG, "null argument");
     if (M < 64 || M > m->max_batch || M % 64 != 0)
         return errf(BBS_ERR_INVALID_ARG, "minibatch must be a multiple of 64 up to %d", m->max_batch);
@@ -1068,26 +1142,24 @@ bbs_status bbs_mlp_gradients(bbs_mlp* m, const uint16_t* feats, const float* tar
     bbs::mlp::gather_kernel<<<dim3(m->in_pad / 64, M / 64), 256, 0, st>>>(
         M, m->in_pad, m->n, rows, reinterpret_cast<const __nv_bfloat16*>(feats), targets,
         reinterpret_cast<uintptr_t>(feats) % 16 == 0, m->X, m->XT, m->T, loss);
-    cudaError_t e = backward(m, M, loss, st);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = backward(m, M, loss, adam, st);
     return e == cudaSuccess ? BBS_OK : errf(BBS_ERR_CUDA, "%s", cudaGetErrorString(e));
+}
+
+bbs_status bbs_mlp_gradients(bbs_mlp* m, const uint16_t* feats, const float* targets, const int32_t* rows,
+                             int32_t M, float* loss, void* stream) {
+    return gradients(m, feats, targets, rows, M, loss, nullptr, stream);
 }
 
 bbs_status bbs_mlp_train_step(bbs_mlp* m, const uint16_t* feats, const float* targets, const int32_t* rows,
                               int32_t M, float lr, float* loss, void* stream) {
-    bbs_status s = bbs_mlp_gradients(m, feats, targets, rows, M, loss, stream);
-    if (s != BBS_OK) return s;
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    m->adam_t += 1;
-    const float c1 = 1.0f - powf(0.9f, (float)m->adam_t), c2 = 1.0f - powf(0.999f, (float)m->adam_t);
-    bbs::mlp::Layers w;
-    for (int l = 0; l < bbs::mlp::kLayers; ++l) {
-        w.off_W[l] = (int)m->off_W[l], w.out[l] = m->dims_out[l], w.in[l] = m->dims_in[l];
-        w.in_pad[l] = m->pad_in[l], w.out_pad[l] = m->pad_out[l], w.Wb[l] = m->Wb[l], w.WTb[l] = m->WTb[l];
-    }
-    bbs::mlp::adam_kernel<<<(unsigned)std::min<size_t>((m->count + 255) / 256, 2048), 256, 0, st>>>(
-        m->count, m->p, m->g, m->m, m->v, lr, 0.9f, 0.999f, 1e-8f, c1, c2, w);
-    cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? BBS_OK : errf(BBS_ERR_CUDA, "%s", cudaGetErrorString(e));
+    if (m == nullptr) return errf(BBS_ERR_INVALID_ARG, "null argument");
+    const float t = (float)(m->adam_t + 1);
+    const bbs::mlp::Adam adam{m->p, m->m, m->v, lr, 0.9f, 0.999f, 1e-8f, 1.0f - powf(0.9f, t), 1.0f - powf(0.999f, t)};
+    bbs_status s = gradients(m, feats, targets, rows, M, loss, &adam, stream);
+    if (s == BBS_OK) m->adam_t += 1;
+    return s;
 }
 
 bbs_status bbs_mlp_set_gemm(bbs_mlp* m, int32_t kind) {

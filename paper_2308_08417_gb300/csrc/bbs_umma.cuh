@@ -122,6 +122,19 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 }
 
+// Programmatic dependent launch. A kernel launched with that attribute starts
+// while the one before it still runs; grid_wait() returns once that one has
+// completed and its writes are visible (at once in an ordinary launch), so
+// nothing in global memory is touched before it. grid_release() lets the next
+// kernel start. Every kernel of a chain waits before it ends, so waiting for
+// the last one means that all before it have completed too.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
+    asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+
 // Dynamic shared memory of a BN-wide tile: kStages stages of A and B, then
 // the barriers (full[kStages], empty[kStages], done) and the TMEM slot.
 __host__ __device__ constexpr size_t stage_bytes(int BN) { return (size_t)kBM * kBK * 2 + (size_t)BN * kBK * 2; }
@@ -156,6 +169,8 @@ __device__ __forceinline__ void gemm_tn_tma(const CUtensorMap* ta, const CUtenso
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
     if (tid == 32) {
+        prefetch_map(ta);
+        prefetch_map(tb);
         for (int s = 0; s < kStages; ++s) {
             mbar_init(saddr(&full[s]), 1);
             mbar_init(saddr(&empty[s]), 1);
@@ -163,6 +178,8 @@ __device__ __forceinline__ void gemm_tn_tma(const CUtensorMap* ta, const CUtenso
         mbar_init(saddr(done), 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
+    grid_release();
+    grid_wait();
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
