@@ -311,11 +311,18 @@ bbs_status make_plan(const bbs_handle* h, const bbs_batch_matrix* A, const bbs_o
         // The fixed-point kernels are bound by latency, not by a pipe: its warps
         // spread evenly over the SM's four schedulers in powers of two (BiCGSTAB, n = 625,
         // 5-point, 6,400 systems: 3 warps 4.97 ms, 4 warps 3.51 ms; n = 1,600: 7
-        // warps 4.60 ms, 8 warps 4.22 ms), and long rows leave few blocks on an
+        // warps 4.60 ms, 8 warps 4.22 ms). One warp is slower than two where it has
+        // long rows or eight of them per thread (BiCGSTAB, 4,000 and 117 systems: n = 169,
+        // 9-point, 851 us -> 834, 194 us -> 153; n = 256, 5-point, 961 us -> 916, 224 us ->
+        // 165; below the line n = 169, 5-point, 758 us -> 783, n = 200, 3-point, 832 us ->
+        // 943; CG there 797 us -> 766).
+        // The rule leaves the batch's size out: a system's bits depend on its group, and
+        // must not on how many others are solved with it. Long rows leave few blocks on an
         // SM, where two rows per thread fill it (n = 144, 43 values a row, 16,384
         // systems: 1 warp 19.9 ms, 2 warps 9.5 ms, 3 to 5 warps 8.4 ms).
         int t = 32;
         while (t < p->threads) t *= 2;
+        if (t == 32 && ((p->R > 4 && vps > 6 * (size_t)n) || p->R >= (o->solver == BBS_SOLVER_CG ? 7 : 8))) t = 64;
         if (vps > 24 * (size_t)n)
             while (t < 256 && n > 2 * t) t *= 2;
         // one block fills an SM's shared memory: 8 warps (n = 144, dense: 18.1 ms

@@ -30,7 +30,7 @@
 // What bounds it now: latency (fixed-latency dependences and instruction
 // fetch; 12 warps of 168 registers on an SM, 42 % of the issue slots used, FP64
 // unit 4 %). Measured, start (FP64 pipe 94 % of its rate) -> now:
-//   65,536 systems, n = 144, 5-point, CSR, 16 lanes   12.03 -> 5.6 ms
+//   65,536 systems, n = 144, 5-point, CSR, 16 lanes   12.03 -> 5.79 ms
 //   131,072 systems, n = 22, dense, 8 lanes            3.58 -> 1.46 ms
 //   16,384 systems, n = 144, 43 values a row          12.95 -> 8.6 ms
 //   4,096 systems, n = 1,024, 9-point, 4 warps        14.63 -> 6.5 ms
@@ -1095,13 +1095,12 @@ __device__ __forceinline__ void bicgstab_staged_jacobi(const Op<FMT, R, double, 
     bicgstab_scaled_system<FMT, R>(op, io, C, sm, tm);
 }
 
-// The folded BiCGSTAB keeps six vectors in registers; at 5-6 rows per thread
-// a cap of 128 registers holds them without spilling and doubles the systems
-// an SM keeps resident (the FP64 pipe needs many warps to stay busy).
-__host__ __device__ constexpr int folded_min_blocks(int R) { return (R == 5 || R == 6) ? 2 : 1; }
-
+// No cap on the registers beyond the block's own: at 128, which kept more FP64
+// warps resident at 5-6 rows per thread, the fixed-point code spills (BiCGSTAB,
+// n = 324, 9-point, 2 warps: 4,000 systems 2.02 -> 1.59 ms, 117 systems 376 ->
+// 217 us; the FP64 kernel took 2.51 ms and 368 us).
 template <int FMT, int R>
-__global__ void __launch_bounds__(max_threads_for(R), folded_min_blocks(R))
+__global__ void __launch_bounds__(max_threads_for(R), 1)
     bicgstab_folded_kernel(const SolveParams P) {
     extern __shared__ __align__(16) unsigned char raw[];
     const Team tm = Team::block();

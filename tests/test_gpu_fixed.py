@@ -153,3 +153,26 @@ def test_gmres_edges(bbs, handle, fmt, tps, restart):
     r = oracle.solve_batch(A, b, x0, solver="gmres", restart=restart, max_iters=400)
     fails = compare(*g[:4], r[0], r[1], r[3], rel_host=host_rel_residual(D, g[0], b), label=f"gmres {fmt} {tps}")
     assert not fails, "\n".join(fails)
+
+
+@pytest.mark.parametrize("solver,stencil,kx,ky,threads", [("bicgstab", "2d9", 13, 13, 64), ("bicgstab", "2d5", 16, 16, 64),
+                                                          ("bicgstab", "1d3", 200, 1, 32), ("cg", "1d3", 200, 1, 64),
+                                                          ("cg", "2d5", 13, 13, 32), ("bicgstab", "2d9", 18, 18, 64)])
+def test_warps_per_system_do_not_depend_on_the_batch(bbs, handle, solver, stencil, kx, ky, threads):
+    """The rule that gives long or many rows a second warp, on both sides of
+    its line, and a system's bits in a batch of one and of many."""
+    rng = np.random.default_rng(kx)
+    pat = W.stencil_pattern(stencil, kx, ky) if ky > 1 else W.stencil_pattern(stencil, kx)
+    sym = solver == "cg"
+    vals = W.stencil_values(pat, 700, rng, 0.05, 0.5, **({"symmetric": True} if sym else {}))
+    b = rng.uniform(-1, 1, (700, pat.n))
+    few = 9
+    check(bbs, handle, pat, vals[:few], b[:few], "csr", solver=solver)
+    got = []
+    for k in (few, 700):
+        A = W.make_batch(pat, vals[:k], "csr")
+        info = handle.describe(bbs.DeviceBatch.from_batch(A, "cuda"), bbs.bbs_default_options(solver=solver))
+        assert info["threads_per_system"] == threads
+        got.append(gpu_solve(bbs, handle, A, b[:k], solver=solver))
+    for x, y in zip(got[0][:4], got[1][:4]):
+        assert np.array_equal(x, y[:few])
