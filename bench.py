@@ -53,6 +53,12 @@ METRIC = "systems solved/s to rel. residual 1e-10"
 FP64_FLOP_PER_CLK_SM = 4.0
 # FP32 (non-tensor) FMA lanes: 128 per SM per clock = 256 FLOP/clk/SM.
 FP32_FLOP_PER_CLK_SM = 256.0
+# The Jacobi solvers work in 62-bit block fixed point on the integer pipe: 64
+# lanes of 32 x 32 + 64-bit multiply-add per SM per clock, up to four of them
+# per multiply-add of the algorithm = 32 FLOP/clk/SM.
+INT64_FLOP_PER_CLK_SM = 32.0
+FIXED_POINT_KERNELS = {"bicgstab_packed_kernel", "bicgstab_folded_kernel", "cg_packed_kernel", "cg_kernel",
+                       "gmres_packed_kernel", "varteam_kernel", "varpacked_kernel", "varteam_kernel+varpacked_kernel"}
 NUM_SMS = 152
 HBM_GBS = 6789.0  # measured copy bandwidth of the GB300s
 
@@ -62,14 +68,11 @@ HBM_GBS = 6789.0  # measured copy bandwidth of the GB300s
 # scales them to its own launch of the same shape by systems (traffic is the
 # compulsory bytes, which grow in proportion). A kernel run on a workload
 # without a capture reports null, and an entry is removed when its kernel
-# changes. The uneven batch's entries are captures of its first 20,000
-# systems (the persistent launch alone, and the graph of persistent, packed
-# and wide launches: the sum over its launches); per-system bytes vary with n,
-# so their scaling is approximate.
-TRAFFIC = {("bicgstab_packed_kernel", "stencil2d5_12x12"): (135.11e6, 16384),
-           ("bicgstab_folded_kernel", "stencil2d5_12x12"): (280.72e6, 32768),
-           ("cg_packed_kernel", "sym_stencil2d5_12x12_cg+jacobi"): (133.00e6, 16384),
-           ("gmres_packed_kernel", "stencil2d5_12x12_gmres+jacobi"): (147.83e6, 16384),
+# changes.
+TRAFFIC = {("bicgstab_packed_kernel", "stencil2d5_12x12"): (135.44e6, 16384),
+           ("bicgstab_folded_kernel", "stencil2d5_12x12"): (280.15e6, 32768),
+           ("cg_packed_kernel", "sym_stencil2d5_12x12_cg+jacobi"): (132.32e6, 16384),
+           ("gmres_packed_kernel", "stencil2d5_12x12_gmres+jacobi"): (149.97e6, 16384),
            ("bicgstab_ilu_packed_kernel", "stencil2d5_12x12_bicgstab+ilu0"): (134.60e6, 16384),
            ("refine_kernel", "stencil2d9_32x32"): (396.44e6, 4096)}
 
@@ -253,7 +256,8 @@ class Uniform:
             inner = self.log.inner_iters.cpu().numpy().astype(np.int64)
             return float(inner.sum()) * per_it, "fp32"
         it = self.log.iters.cpu().numpy().astype(np.int64)
-        return float(it.sum()) * per_it, "fp64"
+        fixed = o.precond == 1 and self.kernel in FIXED_POINT_KERNELS
+        return float(it.sum()) * per_it, "int64" if fixed else "fp64"
 
     def compulsory_bytes(self):
         B, A = self.num_batch, self.A
@@ -365,7 +369,7 @@ class Uneven:
     def work(self):
         it = self.log.iters.cpu().numpy().astype(np.int64)
         per_it = 4 * self.vb.sys_nnz().astype(np.int64) + 26 * self.vb.sys_n().astype(np.int64)
-        return float((it * per_it).sum()), "fp64"
+        return float((it * per_it).sum()), "int64" if self.kernel in FIXED_POINT_KERNELS else "fp64"
 
     def compulsory_bytes(self):
         return 8 * (self.vb.values.size + 3 * self.vb.b.size) + 16 * self.num_batch
@@ -670,7 +674,7 @@ def measured_peaks(bbs, h):
 def roofline(r, solve_ms, mhz, peaks=None):
     flops, arith = r.work()
     avg_s = statistics.mean(solve_ms) / 1e3
-    per_clk = FP64_FLOP_PER_CLK_SM if arith == "fp64" else FP32_FLOP_PER_CLK_SM
+    per_clk = {"fp64": FP64_FLOP_PER_CLK_SM, "int64": INT64_FLOP_PER_CLK_SM, "fp32": FP32_FLOP_PER_CLK_SM}[arith]
     peak = per_clk * NUM_SMS * mhz * 1e6 / 1e12
     achieved = flops / avg_s / 1e12
     out = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",

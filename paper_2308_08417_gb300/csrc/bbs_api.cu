@@ -172,9 +172,9 @@ int packed_warps_per_sm(size_t smem, int R) {
 
 // The library's packing: the narrowest group of 4, 8 or 16 lanes that covers
 // n in at most kMaxPackedR rows per lane and still leaves kPackedMinWarps
-// warps resident per SM (narrower groups put more systems on each FP64
-// instruction; fewer warps leave the FP64 pipe idle). Measured on GB300
-// (BiCGSTAB + Jacobi, 32,768 systems): 22 rows, 438 values: 8 lanes (14
+// warps resident per SM (narrower groups put more systems on each
+// instruction; fewer warps leave its latencies uncovered). Measured on GB300
+// with the FP64 kernels (BiCGSTAB, 32,768 systems): 22 rows, 438 values: 8 lanes (14
 // warps) 31.0 M systems/s, 4 lanes (7 warps) 28.5 M, one per warp 16.9 M;
 // 33 rows, 978 values (CSR): 16 lanes (13 warps) 13.4 M, 8 lanes (6 warps)
 // 12.7 M, one per warp 9.4 M; 54 rows, 2,560 values: 16 lanes (5 warps)

@@ -1,11 +1,10 @@
 // BiCGSTAB for small systems packed several to a warp (Sec. 3.2's one
 // system per work-group, with the work-group narrowed to L lanes).
 //
-// On GB300 an FP64 warp-instruction costs the same pipe time whether 32 or 1
-// of its lanes are active, and the FP64 pipe bounds these solvers. A system of
-// n rows on a whole warp wastes the lanes of its last row group (n = 144 on
-// 32 lanes: 160 slots) and pays the scalar work of every iteration (the
-// divisions for alpha, omega and beta, the reduction trees) once per system.
+// A warp-instruction costs the same issue and pipe time whether 32 or 1 of its
+// lanes are active. A system of n rows on a whole warp wastes the lanes of its
+// last row group (n = 144 on 32 lanes: 160 slots) and pays the scalar work of
+// every iteration (alpha, omega and beta, the reduction trees) once per system.
 // Here each aligned group of L lanes (L = 4, 8 or 16) owns one system, so one
 // warp advances 32 / L systems with each instruction:
 //   * lane l of group g owns rows l, l + L, ..., l + (R-1) L of system g;
@@ -18,11 +17,17 @@
 // computing discarded values until the warp's last system stops. Its x~ is
 // frozen by predication, and the rare per-system branches (the half-step
 // exit, the true-residual confirmation) run for the whole warp when any group
-// takes them, with only that group keeping the results. The method, its
-// stopping rules and its results are those of the one-system-per-team kernels
-// (bicgstab_scaled_system): Jacobi folded into the staged values, As = A D^-1
-// on x~ = D x, squared-norm tests on the integer pipe, true-residual
-// confirmation with at most kMaxRestarts restarts.
+// takes them, with only that group keeping the results.
+//
+// BiCGSTAB, CG and GMRES with Jacobi run in block fixed point on the integer
+// pipe (bbs_fixed.cuh and its CG and GMRES parts, where the figures stand).
+// What is here besides that: the staging, the FP64 versions of the same
+// methods for the systems that the fixed point does not take (no diagonal, a
+// wide spread, no preconditioner), whose bound is the FP64 pipe, and ILU(0).
+// Method, stopping rules and results of the FP64 versions are those of the
+// one-system-per-team kernels (bicgstab_scaled_system): Jacobi folded into the
+// staged values, As = A D^-1 on x~ = D x, squared-norm tests on the integer
+// pipe, true-residual confirmation with at most kMaxRestarts restarts.
 #pragma once
 
 #include "bbs_fixed.cuh"
