@@ -17,7 +17,7 @@
 // of its vector (block floating point), which is the measure the stopping
 // test ||b - A x|| <= tau uses.
 //   * Inner products keep all four partial products: exact up to a last
-//     rounding at 2^-69 of the full scale.
+//     rounding at 2^-100 of the full scale.
 //   * The matrix (Jacobi folded in, unit diagonal) is held as A 2^(60 - sigma)
 //     where 2^sigma bounds its row sums; a product drops only lo lo, below
 //     one unit of the result per stored entry.
@@ -48,6 +48,13 @@ namespace fx {
 
 constexpr int kNone = -1000000;  // exponent of a vector that is zero
 constexpr float kRowSumMax = 31.0f;
+// What became of a system: not begun (the staged values are intact), solved, or
+// given up (they are not).
+enum Fit { kUnfit, kDone, kLeft };
+// Statuses that end a solve here; of a system that stops in another way nothing is
+// written.
+constexpr int kStagnated = -2;
+__device__ __forceinline__ bool accepted(int status) { return status == ST_CONVERGED || status == ST_MAX_ITER; }
 constexpr int kMaxWarps = 16;  // warps of a team whose partial sums fit the reduction area
 
 struct Dig {
@@ -118,6 +125,30 @@ __device__ __forceinline__ long long shl31(long long y, int k) {
     return ((long long)(int)__funnelshift_l(lo, (unsigned)(y >> 32), k) << 32) | (unsigned)(lo << k);
 }
 
+// Shifts a residual of `bits` bits (44: or fewer, then its length is taken first)
+// up to 56, its exponent e following.
+template <int R, class G>
+__device__ __forceinline__ void fill_up(long long (&y)[R], int& e, int& bits, G& g) {
+    int k = max(0, 56 - bits);
+    if (g.any(bits <= 44)) {  // rare: it has fallen by 2^12 and more since it was last shifted
+        unsigned long long o = 0;
+#pragma unroll
+        for (int q = 0; q < R; ++q) o |= (unsigned long long)(y[q] ^ (y[q] >> 63));
+        const int length = g.max_int(64 - __clzll((long long)o));
+        if (bits <= 44) k = 56 - length;
+        const int far = max(0, k - 31);
+#pragma unroll
+        for (int q = 0; q < R; ++q) y[q] = (long long)((unsigned long long)y[q] << far);
+        k -= far;
+        e -= far;
+        bits = min(bits, 56 - k);
+    }
+    e -= k;
+    bits += k;
+#pragma unroll
+    for (int q = 0; q < R; ++q) y[q] = shl31(y[q], k);
+}
+
 // Sum of c y terms: hh in units of the result, m in units of 2^-29.
 struct Sum {
     long long hh, m;
@@ -164,19 +195,23 @@ __device__ __forceinline__ Dot dot_wide(const Dig (&a)[R], long long& carry) {
     return d;
 }
 
-// A partial sum on its way through the reduction: hi 2^21 + lo in units of
-// 2^47. Sums over 2048 rows of products of 2^118 stay below 2^63 in hi, and
-// 512 lanes' lo below 2^31.
+// A partial sum on its way through the reduction: hi 2^54 + lo in units of 2^14,
+// 0 <= lo < 2^54. Sums over 2048 rows of products of 2^118 stay below 2^63 in
+// hi, and 512 lanes' lo below 2^63. The bits below 2^14 are dropped: 2^-100 of
+// the full scale, so a vector whose entries have cancelled down to 2^40 units
+// still has a norm of 53 bits. (At 2^47, with 21 bits in lo, one of 2^32 units had
+// 17 bits, and one of 2^23 the norm 0: omega = 0 then stopped systems that FP64
+// solves, 28 of 300 with the matrix tridiag(-1, 2, -1), n = 128.)
 struct Part {
-    long long hi;
-    int lo;
+    long long hi, lo;
 };
 __device__ __forceinline__ Part part(const Dot& d, long long carry = 0) {
+    constexpr long long kLow = (1 << 29) - 1;
     const long long m = d.m + (d.ll >> 29);
     const long long h = d.hh + (m >> 29);
     Part p;
     p.hi = (h >> 10) + carry;
-    p.lo = ((int)(h & 1023) << 11) | (int)((unsigned)(m & ((1 << 29) - 1)) >> 18);
+    p.lo = (h & 1023) << 44 | (m & kLow) << 15 | (d.ll & kLow) >> 14;
     return p;
 }
 // A scalar m 2^e with 2^61 <= |m| < 2^62 (zero: m = 0, e = kNone). The
@@ -196,11 +231,11 @@ __device__ __forceinline__ Sc normal(long long v, int e) {
 }
 // The sum of vectors whose exponents add up to e.
 __device__ __forceinline__ Sc value(Part p, int e) {
-    const long long hi = p.hi + (p.lo >> 21);
-    const unsigned lo = (unsigned)p.lo & ((1u << 21) - 1);
-    const int z = min(__clzll(hi ^ (hi >> 63)) - 2, 41);
-    const long long v = (long long)(((unsigned long long)hi << z) + (((unsigned long long)lo << 41) >> (62 - z)));
-    return normal(v, 47 + 21 - z + e);
+    const long long hi = p.hi + (p.lo >> 54);
+    const long long lo = p.lo & ((1ll << 54) - 1);
+    const int z = min(__clzll(hi ^ (hi >> 63)) - 2, 54);
+    const long long v = (long long)((unsigned long long)hi << z) + (lo >> (54 - z));
+    return normal(v, 68 - z + e);
 }
 __device__ __forceinline__ Sc one() { return Sc{1ll << 61, -61}; }
 // c, exactly (zero below the normal range; infinities come out as 2^1024 and more)
@@ -237,11 +272,12 @@ __device__ __forceinline__ bool zero(Sc a) { return a.e < -1074 - 62; }
 // a <= b, both >= 0
 __device__ __forceinline__ bool le(Sc a, Sc b) { return a.e < b.e || (a.e == b.e && a.m <= b.m); }
 
-// High 62 bits of a product (the lowest one or two units are dropped).
+// High 62 bits of a product, rounded (the two low halves' product, below one unit,
+// is left out).
 __device__ __forceinline__ long long mul62(long long a, long long b) {
     const int ah = (int)(a >> 31), bh = (int)(b >> 31);
     const int al = (int)((unsigned)a & 0x7fffffffu), bl = (int)((unsigned)b & 0x7fffffffu);
-    return wide(ah, bh, (wide(ah, bl, 0) >> 31) + (wide(al, bh, 0) >> 31));
+    return wide(ah, bh, wide(ah, bl, wide(al, bh, 1 << 30)) >> 31);
 }
 __device__ __forceinline__ Sc mul(Sc a, Sc b) {
     const long long r = mul62(a.m, b.m);
@@ -404,26 +440,26 @@ struct Warps {
             for (int j = 0; j < ND; ++j) out[j] = Sc{shfl(d.m, home<32, ND>(j)), shfl(d.e, home<32, ND>(j))};
             return;
         }
-        // slot of a warp: hi[3] (24 bytes) | lo[3] | 4 unused | mask (4 or 8 bytes), 48 in all
+        // slot of a warp: hi[3] | lo[3] | mask (4 or 8 bytes), 64 bytes in all
         unsigned char* r = half();
         if (w < ND && tm.lane == home<32, ND>(w)) {
-            unsigned char* slot = r + tm.warp * 48;
+            unsigned char* slot = r + tm.warp * 64;
             reinterpret_cast<long long*>(slot)[w] = k.hi;
-            reinterpret_cast<int*>(slot + 24)[w] = k.lo;
-            if (w == 0) *reinterpret_cast<O*>(slot + 40) = o;
+            reinterpret_cast<long long*>(slot + 24)[w] = k.lo;
+            if (w == 0) *reinterpret_cast<O*>(slot + 48) = o;
         }
         tm.sync();
         Part t[ND];
 #pragma unroll
         for (int j = 0; j < ND; ++j) t[j] = Part{0, 0};
         for (int v = 0; v < tm.nwarps; ++v) {
-            const unsigned char* slot = r + v * 48;
+            const unsigned char* slot = r + v * 64;
 #pragma unroll
             for (int j = 0; j < ND; ++j) {
                 t[j].hi += reinterpret_cast<const long long*>(slot)[j];
-                t[j].lo += reinterpret_cast<const int*>(slot + 24)[j];
+                t[j].lo += reinterpret_cast<const long long*>(slot + 24)[j];
             }
-            o |= *reinterpret_cast<const O*>(slot + 40);
+            o |= *reinterpret_cast<const O*>(slot + 48);
         }
 #pragma unroll
         for (int j = 0; j < ND; ++j) out[j] = value(t[j], e[j]);
@@ -782,11 +818,11 @@ __device__ __forceinline__ void folded_finish(const Mat<double>& A, const Mat<do
 // the vectors are block fixed point. A: the system in its own format FMT
 // (diagonal lookups), S: the staged copy in format SF, whose values this
 // overwrites with digits once the system has qualified. `valid` is false for
-// a group without a system of its own (it reads, and never writes). Returns
-// whether the system was solved here; if not, the staged values, x and the
-// log are untouched.
+// a group without a system of its own (it reads, and never writes). A system
+// that FP64 has to solve (one that does not fit, or has broken down, stagnated or
+// met a non-finite scalar here) has its x and its log untouched.
 template <int FMT, int SF, int R, class G>
-__device__ __forceinline__ bool bicgstab_fixed(const Mat<double>& A, const Mat<double>& S, const SysIO& io, bool valid,
+__device__ __forceinline__ Fit bicgstab_fixed(const Mat<double>& A, const Mat<double>& S, const SysIO& io, bool valid,
                                                const SolveCfg& C, const TeamSmem& sm, G g, const Team& team) {
     const int n = io.n;
     Team tm = team;
@@ -804,7 +840,7 @@ __device__ __forceinline__ bool bicgstab_fixed(const Mat<double>& A, const Mat<d
         // (the block's other warps count on this one at their barriers)
         for (int it = 1; it <= C.max_iters && g.live(false); ++it) {
         }
-        return false;
+        return kUnfit;
     }
     const bool last = tm.row(R - 1) < n;  // only a lane's last row may lie past the end
     const Sc tol2 = unpack(C.tol * C.tol), tau2 = C.tol_type == 1 ? mul(tol2, nb2) : tol2;
@@ -853,16 +889,14 @@ __device__ __forceinline__ bool bicgstab_fixed(const Mat<double>& A, const Mat<d
         }
         unsigned op;
         {  // r to 56 bits, p = r + beta (p - omega v)
-            const int k = max(0, min(31, 56 - bR));
-            eR -= k;
-            bR += k;
+            fill_up(Rv, eR, bR, g);
             const Sc beta = mul(rho, cfac), bo = neg(mul(beta, omega));
             const int eo = max(max(eR + max(0, bR - 55), eP + ex(beta) + max(-2, bP - 55)),
                                eV + ex(bo) + max(-2, bV - 55));
             const Dig c1 = coef(beta, eP, eo), c2 = coef(bo, eV, eo);
             long long t[R];
 #pragma unroll
-            for (int q = 0; q < R; ++q) t[q] = Rv[q] = shl31(Rv[q], k);
+            for (int q = 0; q < R; ++q) t[q] = Rv[q];
             shr_rows(t, eo - eR, g);
             op = 0;
 #pragma unroll
@@ -1037,7 +1071,7 @@ __device__ __forceinline__ bool bicgstab_fixed(const Mat<double>& A, const Mat<d
                     status = ST_CONVERGED;
                     active = false;
                 } else if (++restarts > kMaxRestarts) {
-                    status = ST_MAX_ITER;
+                    status = kStagnated;
                     active = false;
                 } else {
                     have_res = false;
@@ -1067,30 +1101,33 @@ __device__ __forceinline__ bool bicgstab_fixed(const Mat<double>& A, const Mat<d
         }
     }
     if (active) status = ST_MAX_ITER;
-    const bool need = run && !have_res;
+    const bool done = run && accepted(status), need = done && !have_res;
     if (g.any(need)) {
         const Sc res = residual(false);
         if (need) res2 = res;
     }
-    folded_finish<FMT, SF>(A, S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, run, iters, status, res2, nb2, sm, g, tm);
-    return run;
+    folded_finish<FMT, SF>(A, S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, done, iters, status, res2, nb2, sm, g, tm);
+    return done ? kDone : run ? kLeft : kUnfit;
 }
 
 }  // namespace fx
 
 // --------------------------------------------------- teams of whole warps
 
-// BiCGSTAB with Jacobi on staged values: block fixed point, or FP64 for the
-// systems that do not fit it (and for teams of more warps than the fixed-point
-// reductions hold).
+// BiCGSTAB with Jacobi on staged values (`count` of them): block fixed point, or
+// FP64 for the systems that do not fit it (and for teams of more warps than the
+// fixed-point reductions hold).
 template <int FMT, int R>
-__device__ __forceinline__ void bicgstab_staged_jacobi(const Op<FMT, R, double, double>& op, const SysIO& io,
-                                                       const SolveCfg& C, const TeamSmem& sm, const Team& tm) {
+__device__ __forceinline__ void bicgstab_staged_jacobi(const Op<FMT, R, double, double>& op, size_t count,
+                                                       const SysIO& io, const SolveCfg& C, const TeamSmem& sm,
+                                                       const Team& tm) {
     if (tm.nwarps <= fx::kMaxWarps) {
         const Mat<double> S{op.as, op.A.row_ptrs, op.A.cols, op.A.n, op.A.k};
         const fx::Warps g{tm, reinterpret_cast<unsigned char*>(sm.red), 0};
-        if (fx::bicgstab_fixed<FMT, FMT, R>(op.A, S, io, true, C, sm, g, tm)) return;
+        const fx::Fit fit = fx::bicgstab_fixed<FMT, FMT, R>(op.A, S, io, true, C, sm, g, tm);
+        if (fit == fx::kDone) return;
         tm.sync();
+        if (fit == fx::kLeft) make_op<FMT, R>(op.A, count, const_cast<double*>(op.as), tm);
     }
     bicgstab_scaled_system<FMT, R>(op, io, C, sm, tm);
 }
@@ -1106,6 +1143,6 @@ __global__ void __launch_bounds__(max_threads_for(R), 1)
     const Team tm = Team::block();
     const int sys = blockIdx.x;
     const auto op = make_op<FMT, R>(P, sys, raw, tm);
-    bicgstab_staged_jacobi<FMT, R>(op, sys_io(P, sys), solve_cfg(P, sys), team_smem(raw, P.n_pad), tm);
+    bicgstab_staged_jacobi<FMT, R>(op, P.vps, sys_io(P, sys), solve_cfg(P, sys), team_smem(raw, P.n_pad), tm);
 }
 }  // namespace bbs

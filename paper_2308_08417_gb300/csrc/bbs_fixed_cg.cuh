@@ -15,9 +15,9 @@
 namespace bbs {
 namespace fx {
 
-// As bicgstab_fixed: returns whether the system was solved here.
+// As bicgstab_fixed.
 template <int SF, int R, class G>
-__device__ __forceinline__ bool cg_fixed(const Mat<double>& A, const Mat<double>& S, const SysIO& io, bool valid, const SolveCfg& C,
+__device__ __forceinline__ Fit cg_fixed(const Mat<double>& A, const Mat<double>& S, const SysIO& io, bool valid, const SolveCfg& C,
                                          const TeamSmem& sm, G g, const Team& team) {
     const int n = io.n;
     Team tm = team;
@@ -68,7 +68,7 @@ __device__ __forceinline__ bool cg_fixed(const Mat<double>& A, const Mat<double>
         if (!g.any(run)) {  // (the block's other warps count on this one at their barriers)
             for (int it = 1; it <= C.max_iters && g.live(false); ++it) {
             }
-            return false;
+            return kUnfit;
         }
         sigma = (top >> 23) - 126;  // row sums < 2^sigma
         eD = (inv >> 23) - 126 - 1;  // |1 / a_ii| < 2^(eD + 1)
@@ -227,11 +227,7 @@ __device__ __forceinline__ bool cg_fixed(const Mat<double>& A, const Mat<double>
         Dig z[R];
         int eZ, bZ;
         {  // r to 56 bits, r -= alpha t, z = D^-1 r
-            const int k = max(0, min(31, 56 - bR));
-            eR -= k;
-            bR += k;
-#pragma unroll
-            for (int q = 0; q < R; ++q) Rv[q] = shl31(Rv[q], k);
+            fill_up(Rv, eR, bR, g);
             const int eo = max(eR + max(0, bR - 56), eT + ex(alpha) + max(-2, bT - 56));
             const Dig c = coef(neg(alpha), eT, eo);
             shr_rows(Rv, eo - eR, g);
@@ -313,7 +309,7 @@ __device__ __forceinline__ bool cg_fixed(const Mat<double>& A, const Mat<double>
                     status = ST_CONVERGED;
                     active = false;
                 } else if (++restarts > kMaxRestarts) {
-                    status = ST_MAX_ITER;
+                    status = kStagnated;
                     active = false;
                 } else {
                     have_res = false;
@@ -331,12 +327,12 @@ __device__ __forceinline__ bool cg_fixed(const Mat<double>& A, const Mat<double>
         if (!restarted) rho = rho_hat;
     }
     if (active) status = ST_MAX_ITER;
-    const bool need = run && !have_res;
+    const bool done = run && accepted(status), need = done && !have_res;
     if (g.any(need)) {
         const Sc res = true_residual<SF>(S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, false, g, tm);
         if (need) res2 = res;
     }
-    const bool moved = run && iters > 0;
+    const bool moved = done && iters > 0;
 #pragma unroll
     for (int q = 0; q < R; ++q) {
         const int row = tm.row(q);
@@ -353,13 +349,13 @@ __device__ __forceinline__ bool cg_fixed(const Mat<double>& A, const Mat<double>
         const Sc res = true_residual<SF>(S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, false, g, tm);
         if (close) res2 = res;
     }
-    if (run && tm.tid == 0) {
+    if (done && tm.tid == 0) {
         *io.iters = iters;
         *io.rel_res = sqrt(to_double(res2) / to_double(nb2));
         *io.status = status;
         if (io.inner != nullptr) *io.inner = 0;
     }
-    return run;
+    return done ? kDone : run ? kLeft : kUnfit;
 }
 
 }  // namespace fx
@@ -376,8 +372,10 @@ __global__ void __launch_bounds__(max_threads_for(R), 1) cg_kernel(const SolvePa
     if (op.as != nullptr && P.precond == 1 && tm.nwarps <= fx::kMaxWarps) {
         const Mat<double> S{op.as, op.A.row_ptrs, op.A.cols, op.A.n, op.A.k};
         const fx::Warps g{tm, reinterpret_cast<unsigned char*>(sm.red), 0};
-        if (fx::cg_fixed<FMT, R>(op.A, S, sys_io(P, sys), true, solve_cfg(P, sys), sm, g, tm)) return;
+        const fx::Fit fit = fx::cg_fixed<FMT, R>(op.A, S, sys_io(P, sys), true, solve_cfg(P, sys), sm, g, tm);
+        if (fit == fx::kDone) return;
         tm.sync();
+        if (fit == fx::kLeft) make_op<FMT, R>(P, sys, raw, tm);
     }
     cg_system<FMT, R>(op, sys_io(P, sys), solve_cfg(P, sys), sm, tm);
 }

@@ -16,10 +16,10 @@
 namespace bbs {
 namespace fx {
 
-// As bicgstab_fixed: returns whether the system was solved here. ext: the group's
+// As bicgstab_fixed. ext: the group's
 // small arrays, as gmres_packed_system lays them out.
 template <int FMT, int SF, int R, class G>
-__device__ __forceinline__ bool gmres_fixed(const Mat<double>& A, const Mat<double>& S, const SysIO& io, bool valid,
+__device__ __forceinline__ Fit gmres_fixed(const Mat<double>& A, const Mat<double>& S, const SysIO& io, bool valid,
                                             const SolveCfg& C, const TeamSmem& sm, double* ext_generic, G g,
                                             const Team& team) {
     const int n = io.n, m = C.restart;
@@ -33,7 +33,7 @@ __device__ __forceinline__ bool gmres_fixed(const Mat<double>& A, const Mat<doub
     int eX, bX, eR, bR, sigma;
     bool run;
     Sc nb2;
-    if (!folded_setup<FMT, SF>(A, S, io, valid, sm, g, tm, X, eX, bX, Rv, eR, bR, sigma, run, nb2)) return false;
+    if (!folded_setup<FMT, SF>(A, S, io, valid, sm, g, tm, X, eX, bX, Rv, eR, bR, sigma, run, nb2)) return kUnfit;
     const bool last = tm.row(R - 1) < n;  // only a lane's last row may lie past the end
     // exponent of w = A v and what is left of it: every ||w|| is at most the
     // matrix's Frobenius norm (below 2^fexp), and orthogonalising only shortens w, so
@@ -270,23 +270,24 @@ __device__ __forceinline__ bool gmres_fixed(const Mat<double>& A, const Mat<doub
                     status = ST_MAX_ITER;
                     active = false;
                 } else if (estimate_ok && ++restarts > kMaxRestarts) {
-                    status = ST_MAX_ITER;
+                    status = kStagnated;
                     active = false;
                 }
             }
         }
     }
+    const bool done = run && accepted(status);
     // The basis is dead scratch from here on: its whole 128-byte lines are dropped
     // from L2 without a write-back (as gmres_packed_system).
     g.sync();
-    if (valid && V != nullptr) {
+    if (done && V != nullptr) {
         const uintptr_t first = (reinterpret_cast<uintptr_t>(V) + 127) & ~static_cast<uintptr_t>(127);
         const uintptr_t end = (reinterpret_cast<uintptr_t>(V) + (size_t)(m + 1) * vs * 8) & ~static_cast<uintptr_t>(127);
         for (uintptr_t a = first + (uintptr_t)tm.tid * 128; a < end; a += (uintptr_t)tm.nt * 128)
             asm volatile("discard.global.L2 [%0], 128;" ::"l"(a) : "memory");
     }
-    folded_finish<FMT, SF>(A, S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, run, it, status, beta2, nb2, sm, g, tm);
-    return run;
+    folded_finish<FMT, SF>(A, S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, done, it, status, beta2, nb2, sm, g, tm);
+    return done ? kDone : run ? kLeft : kUnfit;
 }
 
 }  // namespace fx

@@ -51,6 +51,26 @@ template <int FMT, int R>
 struct PackedOp {
     Mat<double> A;
     Mat<double> S;
+    const int32_t* src;  // CSR: position of each staged value (-1: padding)
+    int count;           // staged values
+    // Stages the values (CSR: gathered into ELL order by 8-byte asynchronous
+    // copies); the warp synchronises afterwards.
+    __device__ __forceinline__ void stage(const Team& tm) const {
+        double* as = const_cast<double*>(S.vals);
+        if constexpr (FMT == FMT_CSR) {
+#pragma unroll 4
+            for (int i = tm.tid; i < count; i += tm.nt) {
+                const int s = ldg(src + i);
+                if (s >= 0)
+                    cp_async8(as + i, A.vals + s);
+                else
+                    as[i] = 0.0;
+            }
+            cp_async_wait_all();
+        } else {
+            stage_values(A.vals, as, (size_t)count, tm);
+        }
+    }
     __device__ __forceinline__ void apply(const double* xs, double (&y)[R], const Team& tm) const {
         spmv_staged<staged_fmt<FMT>(), R>(S, S.vals, xs, y, tm);
     }
@@ -334,25 +354,26 @@ __device__ __forceinline__ void bicgstab_packed_system(const PackedOp<FMT, R>& o
 
 // BiCGSTAB of a warp's groups: with Jacobi in block fixed point (the integer
 // pipe); the groups it leaves (and all of them without Jacobi) in FP64. The
-// FP64 form is compiled as a function of its own.
+// FP64 form is compiled as a function of its own. `again` (per group): the staged
+// values have been overwritten.
 template <int FMT, int L, int R>
-__device__ __noinline__ void bicgstab_packed_fp64(const PackedOp<FMT, R> op, const SysIO io, bool valid,
+__device__ __noinline__ void bicgstab_packed_fp64(const PackedOp<FMT, R> op, const SysIO io, bool valid, bool again,
                                                   const SolveCfg C, const TeamSmem sm, const Team tm) {
+    if (again) op.stage(tm);
+    __syncwarp();
     bicgstab_packed_system<FMT, L, R>(op, io, valid, C, sm, tm);
 }
 
 template <int FMT, int L, int R>
 __device__ __forceinline__ void bicgstab_packed_any(const PackedOp<FMT, R>& op, const SysIO& io, bool valid,
                                                     const SolveCfg& C, const TeamSmem& sm, const Team& tm) {
-    bool left = valid;
-    if (C.precond == 1) {  // every lane takes part, those without a system too
-        const bool done =
-            fx::bicgstab_fixed<FMT, staged_fmt<FMT>(), R>(op.A, op.S, io, valid, C, sm, fx::Lanes<L>{tm.lane}, tm);
-        left = valid && !done;
-    }
+    fx::Fit fit = fx::kUnfit;
+    if (C.precond == 1)  // every lane takes part, those without a system too
+        fit = fx::bicgstab_fixed<FMT, staged_fmt<FMT>(), R>(op.A, op.S, io, valid, C, sm, fx::Lanes<L>{tm.lane}, tm);
+    const bool left = valid && fit != fx::kDone;
     if (__any_sync(kFull, left)) {
         __syncwarp();
-        bicgstab_packed_fp64<FMT, L, R>(op, io, left, C, sm, tm);
+        bicgstab_packed_fp64<FMT, L, R>(op, io, left, left && fit == fx::kLeft, C, sm, tm);
     }
 }
 
@@ -538,22 +559,23 @@ __device__ __forceinline__ void cg_packed_system(const PackedOp<FMT, R>& op, con
 
 // CG of a warp's groups: with Jacobi in block fixed point, as BiCGSTAB above.
 template <int FMT, int L, int R>
-__device__ __noinline__ void cg_packed_fp64(const PackedOp<FMT, R> op, const SysIO io, bool valid, const SolveCfg C,
-                                            const TeamSmem sm, const Team tm) {
+__device__ __noinline__ void cg_packed_fp64(const PackedOp<FMT, R> op, const SysIO io, bool valid, bool again,
+                                            const SolveCfg C, const TeamSmem sm, const Team tm) {
+    if (again) op.stage(tm);
+    __syncwarp();
     cg_packed_system<FMT, L, R>(op, io, valid, C, sm, tm);
 }
 
 template <int FMT, int L, int R>
 __device__ __forceinline__ void cg_packed_any(const PackedOp<FMT, R>& op, const SysIO& io, bool valid,
                                               const SolveCfg& C, const TeamSmem& sm, const Team& tm) {
-    bool left = valid;
-    if (C.precond == 1) {  // every lane takes part, those without a system too
-        const bool done = fx::cg_fixed<staged_fmt<FMT>(), R>(op.A, op.S, io, valid, C, sm, fx::Lanes<L>{tm.lane}, tm);
-        left = valid && !done;
-    }
+    fx::Fit fit = fx::kUnfit;
+    if (C.precond == 1)  // every lane takes part, those without a system too
+        fit = fx::cg_fixed<staged_fmt<FMT>(), R>(op.A, op.S, io, valid, C, sm, fx::Lanes<L>{tm.lane}, tm);
+    const bool left = valid && fit != fx::kDone;
     if (__any_sync(kFull, left)) {
         __syncwarp();
-        cg_packed_fp64<FMT, L, R>(op, io, left, C, sm, tm);
+        cg_packed_fp64<FMT, L, R>(op, io, left, left && fit == fx::kLeft, C, sm, tm);
     }
 }
 
@@ -834,8 +856,10 @@ __device__ __forceinline__ void gmres_packed_system(const PackedOp<FMT, R>& op, 
 }
 
 template <int FMT, int L, int R>
-__device__ __noinline__ void gmres_packed_fp64(const PackedOp<FMT, R> op, const SysIO io, bool valid, const SolveCfg C,
-                                               double* xa, double* ext, const Team tm) {
+__device__ __noinline__ void gmres_packed_fp64(const PackedOp<FMT, R> op, const SysIO io, bool valid, bool again,
+                                               const SolveCfg C, double* xa, double* ext, const Team tm) {
+    if (again) op.stage(tm);
+    __syncwarp();
     gmres_packed_system<FMT, L, R>(op, io, valid, C, xa, ext, tm);
 }
 
@@ -880,22 +904,16 @@ struct PackedGroup {
         const double* vals = P.values + (size_t)sys * P.vps;
         double* as = reinterpret_cast<double*>(slice + P.stage_off);
         op.A = Mat<double>{vals, P.row_ptrs, P.cols, P.n, P.k};
-        if constexpr (FMT == FMT_CSR) {  // gathered into ELL order by 8-byte asynchronous copies
-            const int count = P.xk * P.n;
-#pragma unroll 4
-            for (int i = tm.tid; i < count; i += L) {
-                const int src = ldg(P.xsrc + i);
-                if (src >= 0)
-                    cp_async8(as + i, vals + src);
-                else
-                    as[i] = 0.0;
-            }
-            cp_async_wait_all();
+        if constexpr (FMT == FMT_CSR) {
             op.S = Mat<double>{as, nullptr, P.xcols, P.n, P.xk};
+            op.src = P.xsrc;
+            op.count = P.xk * P.n;
         } else {
-            stage_values(vals, as, P.vps, tm);
             op.S = Mat<double>{as, P.row_ptrs, P.cols, P.n, P.k};
+            op.src = nullptr;
+            op.count = (int)P.vps;
         }
+        op.stage(tm);
         __syncwarp();
     }
 };
@@ -939,16 +957,15 @@ __global__ void __launch_bounds__(32, packed_cg_min_blocks(R)) gmres_packed_kern
     const size_t count = FMT == FMT_CSR ? (size_t)P.xk * P.n : P.vps;
     unsigned char* slice = raw + (size_t)((threadIdx.x & 31) / L) * P.slice;
     double* ext = reinterpret_cast<double*>(slice + P.stage_off + ((count * 8 + 15) & ~(size_t)15));
-    bool left = G.valid;
-    if (P.precond == 1) {  // block fixed point; every lane takes part, those without a system too
-        const bool done = fx::gmres_fixed<FMT, staged_fmt<FMT>(), R>(G.op.A, G.op.S, sys_io(P, G.sys), G.valid,
-                                                                     solve_cfg(P, G.sys), G.sm, ext,
-                                                                     fx::Lanes<L>{G.tm.lane}, G.tm);
-        left = G.valid && !done;
-    }
+    fx::Fit fit = fx::kUnfit;
+    if (P.precond == 1)  // block fixed point; every lane takes part, those without a system too
+        fit = fx::gmres_fixed<FMT, staged_fmt<FMT>(), R>(G.op.A, G.op.S, sys_io(P, G.sys), G.valid, solve_cfg(P, G.sys),
+                                                         G.sm, ext, fx::Lanes<L>{G.tm.lane}, G.tm);
+    const bool left = G.valid && fit != fx::kDone;
     if (__any_sync(kFull, left)) {
         __syncwarp();
-        gmres_packed_fp64<FMT, L, R>(G.op, sys_io(P, G.sys), left, solve_cfg(P, G.sys), G.sm.xa, ext, G.tm);
+        gmres_packed_fp64<FMT, L, R>(G.op, sys_io(P, G.sys), left, left && fit == fx::kLeft, solve_cfg(P, G.sys),
+                                     G.sm.xa, ext, G.tm);
     }
 }
 

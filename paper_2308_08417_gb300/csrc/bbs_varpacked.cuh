@@ -85,20 +85,12 @@ __global__ void __launch_bounds__(32 * kPackedWarps, packed_min_blocks(R) / kPac
     sm.extra = nullptr;
     double* as = reinterpret_cast<double*>(slice + (((size_t)2 * n_pad * 8 + 15) & ~(size_t)15));
     const double* vals = P.values + ldg(P.val_off + sys);
-    const int32_t* xsrc = P.xsrc + toff;
-    const int count = k * n;
-#pragma unroll 4
-    for (int i = tm.tid; i < count; i += L) {
-        const int src = ldg(xsrc + i);
-        if (src >= 0)
-            cp_async8(as + i, vals + src);
-        else
-            as[i] = 0.0;
-    }
-    cp_async_wait_all();
     PackedOp<FMT_CSR, R> op;
     op.A = Mat<double>{vals, P.row_ptrs + ldg(P.rp_off + pat), P.col_idxs + ldg(P.ci_off + pat), n, 0};
     op.S = Mat<double>{as, nullptr, P.xcols + toff, n, k};
+    op.src = P.xsrc + toff;
+    op.count = k * n;
+    op.stage(tm);
     __syncwarp();
     const int64_t vo = ldg(P.vec_off + sys);
     SysIO io;

@@ -74,8 +74,9 @@ __global__ void __launch_bounds__(256, 1) varteam_kernel(const __grid_constant__
         io.inner = nullptr;
         io.n = n;
         const TeamSmem sm = team_smem(raw + 16, (n + 1) & ~1);
-        const auto op = make_op<FMT_CSR, R>(A, (size_t)ldg(P.pat_nnz + pat), sm.extra, tm);
-        bicgstab_staged_jacobi<FMT_CSR, R>(op, io, P.cfg, sm, tm);
+        const size_t nnz = (size_t)ldg(P.pat_nnz + pat);
+        const auto op = make_op<FMT_CSR, R>(A, nnz, sm.extra, tm);
+        bicgstab_staged_jacobi<FMT_CSR, R>(op, nnz, io, P.cfg, sm, tm);
         if (P.counter == nullptr) break;
         __syncthreads();  // every thread has read its item and is done with the area
     }
