@@ -48,13 +48,15 @@ namespace fx {
 
 constexpr int kNone = -1000000;  // exponent of a vector that is zero
 constexpr float kRowSumMax = 31.0f;
-// What became of a system: not begun (the staged values are intact), solved, or
-// given up (they are not).
-enum Fit { kUnfit, kDone, kLeft };
+// What a system must be like to be solved here, and what became of it.
+constexpr float kExcess = 0x1p-7f;    // BiCGSTAB: least diagonal excess of a row, (|a_ii| - sum of the others) / |a_ii|
+constexpr float kRowScale = 0x1p-12f; // smallest row scale against the largest
+constexpr int kRowScaleBits = 12;
 // Statuses that end a solve here; of a system that stops in another way nothing is
 // written.
 constexpr int kStagnated = -2;
 __device__ __forceinline__ bool accepted(int status) { return status == ST_CONVERGED || status == ST_MAX_ITER; }
+enum Fit { kUnfit, kDone, kLeft };    // not begun (the staged values are intact), solved, given up (they are not)
 constexpr int kMaxWarps = 16;  // warps of a team whose partial sums fit the reduction area
 
 struct Dig {
@@ -485,12 +487,22 @@ __device__ __forceinline__ void each_entry(const Mat<double>& S, int row, F f) {
     }
 }
 
+// Sum of |c| |y| to the high digits, as `Sum` for spmv_sums.
+struct Abs {
+    long long hh;
+    __device__ __forceinline__ void add(Dig c, Dig y) { hh = wide(abs(c.hi), abs(y.hi), hh); }
+};
+__device__ __forceinline__ void begin(Sum& s, int round) { s = Sum{0, round}; }
+__device__ __forceinline__ void begin(Abs& s, int) { s = Abs{0}; }
+
 // Dense digits are kept by rows as the values are, but by columns where rows
 // of n 8-byte words put 16 or 32 lanes on the same banks (16,384 systems of n =
 // 144: 42.5 ms by rows, 18.1 ms by columns; n = 54: 1.99 ms by rows, 2.30 ms by
 // columns, whose digits are made from values read again from global memory).
 __device__ __forceinline__ bool by_columns(int n) { return (n & 7) == 0; }
 
+template <int R>
+__device__ __forceinline__ void carry(Abs (&)[R]) {}
 template <int R>
 __device__ __forceinline__ void carry(Sum (&s)[R]) {
 #pragma unroll
@@ -507,11 +519,11 @@ __device__ __forceinline__ void carry(Sum (&s)[R]) {
 // to 2^59, and hh to 2^61). The slots are the outer loop: R rows' loads are in
 // flight at once, and the loop's code stays within the instruction cache (all
 // rows' slots unrolled took 5 times the code and ran 8 times slower).
-template <int SF, int kTerms, int R>
+template <int SF, int kTerms, class T, int R>
 __device__ __forceinline__ void spmv_sums(const Mat<double>& S, const int2* __restrict__ a,
-                                          const int2* __restrict__ y, Sum (&s)[R], int round, const Team& tm) {
+                                          const int2* __restrict__ y, T (&s)[R], int round, const Team& tm) {
 #pragma unroll
-    for (int q = 0; q < R; ++q) s[q] = Sum{0, round};
+    for (int q = 0; q < R; ++q) begin(s[q], round);
     // Only the last row may lie past the end: such a lane repeats its first row
     // in its place (row 0 if it has none) and drops the result, so that the
     // loops need no branch.
@@ -574,7 +586,7 @@ __device__ __forceinline__ void spmv_sums(const Mat<double>& S, const int2* __re
     }
 #pragma unroll
     for (int q = 0; q < R; ++q)
-        if (q + 1 == R && !last) s[q] = Sum{0, 0};
+        if (q + 1 == R && !last) begin(s[q], 0);
 }
 
 // Their digits, rounded to units of y's exponent plus sigma - 2.
@@ -618,7 +630,7 @@ __device__ __forceinline__ Sc norm2_full(long long (&y)[R], int& e, G& g) {
 template <int SF, int R, class G>
 __device__ __forceinline__ Sc true_residual(const Mat<double>& S, const int2* as, int2* buf, const SysIO& io, int sigma,
                                             long long (&X)[R], int& eX, int& bX, long long (&Rv)[R], int& eR, int& bR,
-                                            bool take, G& g, const Team& tm) {
+                                            bool take, G& g, const Team& tm, int* e_digits = nullptr) {
     const int n = io.n;
     // x with 59 bits: shifted up exactly where it holds fewer (a guess far above
     // the solution has left it coarse units), else rounded for the product
@@ -627,6 +639,7 @@ __device__ __forceinline__ Sc true_residual(const Mat<double>& S, const int2* as
     for (int q = 0; q < R; ++q) xo |= (unsigned long long)(X[q] ^ (X[q] >> 63));
     const int k = 59 - g.max_int(64 - __clzll((long long)xo));
     const int up = k > 0 && k < 59 ? k : 0, dx = max(-k, 0), ex4 = eX - up + dx;
+    if (e_digits != nullptr) *e_digits = ex4;
 #pragma unroll
     for (int q = 0; q < R; ++q) {
         const int row = tm.row(q);
@@ -669,7 +682,22 @@ __device__ __forceinline__ Sc true_residual(const Mat<double>& S, const int2* as
 // The set-up of a solve with Jacobi folded in: whether the system fits (`run`;
 // false is returned, and nothing has been overwritten, where no group's does),
 // the staged matrix as digits of A D^-1, x~ = D x0, r = b - A x~ and ||b||^2.
-template <int FMT, int SF, int R, class G>
+//
+// A system fits where 57 bits below one scale per vector are no less than FP64's
+// 53 below each entry's own:
+//   * the scale of each row's equation, y_i + sum_j |a_ij / a_jj| y_j with y =
+//     |b| + |D x0| (to a factor of 2), is at least 2^-12 of the largest y; else
+//     rows in other units, entries that matter at 1e-6 and 1e-20 alike and parts
+//     of a system that hardly meet would lose theirs (A = diag(1, 2^-70), b = (1,
+//     2^-70): x = (1, 0)). folded_finish looks at the solution in the same way;
+//   * BiCGSTAB: each row's diagonal entry exceeds its others by 2^-7. Below that
+//     the Krylov vectors fall and rise by more than the spare bits in a step, and
+//     systems that take more iterations than they have rows took up to 4 % more of
+//     them (3-point, n = 64, excess 0.001: 93.7 for 89.8 in FP64, 0.008: 71.3 for
+//     70.9, 0.016 and more the same; tridiag(-1, 2, -1), n = 256: 315 for 270).
+//     GMRES has no line: it starts afresh from the true residual every few steps.
+enum Method { kBicgstab, kGmres };
+template <int FMT, int SF, Method METHOD, int R, class G>
 __device__ __forceinline__ bool folded_setup(const Mat<double>& A, const Mat<double>& S, const SysIO& io, bool valid,
                                              const TeamSmem& sm, G& g, const Team& tm, long long (&X)[R], int& eX,
                                              int& bX, long long (&Rv)[R], int& eR, int& bR, int& sigma, bool& run,
@@ -683,8 +711,8 @@ __device__ __forceinline__ bool folded_setup(const Mat<double>& A, const Mat<dou
     bX = 0;
     // (loops over the caller's rows stay rolled here: this runs once)
     long long* dm = in_shared<long long>(sm.xb);  // 1 / a_ii: its digits,
-    int2* de = pa;                                // its exponent and FP32 value
-    int bad = 0, eb = 0, exm = 0;
+    int2* de = pa;                                // its exponent beside y_i's biased one, and its FP32 value
+    int bad = 0, eb = 0, exm = 0, yleast = 0x7ff;
 #pragma unroll 1
     for (int row = tm.tid; row < n; row += tm.nt) {
         double d = 0.0;
@@ -694,26 +722,52 @@ __device__ __forceinline__ bool folded_setup(const Mat<double>& A, const Mat<dou
         bad |= normal64(d) ? 0 : 1;
         const Sc di = rcp(unpack(d));
         dm[row] = di.m;
-        de[row] = make_int2(di.e, __float_as_int(fabsf(__frcp_rn((float)d))));
         const double xt = d * io.x[row];
-        eb = max(eb, (__double2hiint(io.b[row]) >> 20) & 0x7ff);
-        exm = max(exm, zero64(xt) ? 0 : max(1, (__double2hiint(xt) >> 20) & 0x7ff));
+        const int yb = (__double2hiint(io.b[row]) >> 20) & 0x7ff;
+        const int yx = zero64(xt) ? 0 : max(1, (__double2hiint(xt) >> 20) & 0x7ff);
+        de[row] = make_int2((int)((unsigned)di.e << 11) | max(yb, yx), __float_as_int(fabsf(__frcp_rn((float)d))));
+        yleast = min(yleast, max(yb, yx));
+        eb = max(eb, yb);
+        exm = max(exm, yx);
     }
     g.sync();
     int top = 0;  // largest row sum (as the bits of a non-negative FP32, NaN on top)
 #pragma unroll 1
     for (int row = tm.tid; row < n; row += tm.nt) {
-        float t = 0.0f;
+        float t = 0.0f, u = 0.0f;
         each_entry<SF>(S, row, [&](int e, int col) {
-            if (col >= 0) t = fmaf(fabsf((float)S.vals[e]), __int_as_float(de[col].y), t);
+            if (col >= 0) {
+                const float v = fabsf((float)S.vals[e]);
+                t = fmaf(v, __int_as_float(de[col].y), t);
+                if (METHOD == kBicgstab) u += v;
+            }
         });
         top = max(top, __float_as_int(t * 1.0001f) & 0x7fffffff);
+        if (METHOD == kBicgstab) bad |= u * __int_as_float(de[row].y) <= 2.0f - kExcess ? 0 : 1;
     }
     top = g.max_int(bad ? 0x7fffffff : top);
     eb = g.max_int(eb);
     exm = g.max_int(exm);
+    yleast = -g.max_int(-yleast);
+    const int ym = max(eb, exm);
     const bool xz = exm == 0;  // the guess is zero
-    run = valid && top < __float_as_int(kRowSumMax) && eb > 623 && eb < 1423 && (xz || (exm > 623 && exm < 1423));
+    run = valid && top < __float_as_int(kRowSumMax) && eb > 623 && eb < 1423 &&
+          (xz || (exm > 623 && exm < 1423));
+    if (g.any(run && ym - yleast >= kRowScaleBits)) {  // y_i alone does not show it: rare
+        int low = 0x7f800000;  // smallest row scale, against 2^ym
+#pragma unroll 1
+        for (int row = tm.tid; row < n; row += tm.nt) {
+            float u = 0.0f;
+            each_entry<SF>(S, row, [&](int e, int col) {
+                if (col >= 0)
+                    u = fmaf(fabsf((float)S.vals[e]) * __int_as_float(de[col].y),
+                             __int_as_float(max(127 + (de[col].x & 0x7ff) - ym, 0) << 23), u);
+            });
+            low = min(low, __float_as_int(u) & 0x7fffffff);
+        }
+        low = -g.max_int(-low);
+        if (ym - yleast >= kRowScaleBits) run = run && low >= __float_as_int(kRowScale);
+    }
     if (!g.any(run)) return false;
     sigma = max(1, (top >> 23) - 126);  // row sums < 2^sigma
     const int ebq = eb - 1022 - 57;
@@ -725,7 +779,7 @@ __device__ __forceinline__ bool folded_setup(const Mat<double>& A, const Mat<dou
             a = 1ll << (60 - sigma);
         } else if (col >= 0) {
             const Sc u = unpack(v);
-            a = round_shr(mul62(u.m, dm[col]), sigma - 122 - u.e - de[col].x);
+            a = round_shr(mul62(u.m, dm[col]), sigma - 122 - u.e - (de[col].x >> 11));
         }
         return pack(split(a));
     };
@@ -769,39 +823,79 @@ __device__ __forceinline__ bool folded_setup(const Mat<double>& A, const Mat<dou
     return true;
 }
 
-// The end of such a solve: x = D^-1 x~ and the log, for the groups that ran.
+// The end of such a solve, for the groups with `take` set: x = D^-1 x~ rounded
+// to FP64 and the log. `known`: res2 is the true residual of x~. Returns whether
+// the result stands: the scales of its rows (setup's, with x~ for y) have to be in
+// reach of each other. If not, nothing has been written and FP64 solves the system.
 template <int FMT, int SF, int R, class G>
-__device__ __forceinline__ void folded_finish(const Mat<double>& A, const Mat<double>& S, const int2* as, int2* pb,
+__device__ __forceinline__ bool folded_finish(const Mat<double>& A, const Mat<double>& S, const int2* as, int2* pb,
                                               const SysIO& io, int sigma, long long (&X)[R], int& eX, int& bX,
-                                              long long (&Rv)[R], int& eR, int& bR, bool run, int iters, int status,
-                                              Sc res2, Sc nb2, const TeamSmem& sm, G& g, const Team& tm) {
+                                              long long (&Rv)[R], int& eR, int& bR, bool take, int iters, int status,
+                                              bool known, Sc res2, Sc nb2, const TeamSmem& sm, G& g, const Team& tm) {
+    if (!g.any(take)) return false;
     const int n = io.n;
     const bool last = tm.row(R - 1) < n;
-    // x = D^-1 x~, rounded to FP64
-    long long* xw = in_shared<long long>(sm.xa);
-    const bool moved = run && iters > 0;
+    long long* xw = in_shared<long long>(sm.xa);  // x~, then the bits of x
+    long long* xr = in_shared<long long>(sm.xb);  // x~ of the rounded x
+    const bool moved = take && iters > 0;
+    // the scales of the rows: |x~_i| + |b_i| shows nearly always that they are
+    int hi = -100000, lo = 100000;
 #pragma unroll
     for (int q = 0; q < R; ++q)
-        if (q + 1 < R || last) xw[tm.row(q)] = X[q];
+        if (q + 1 < R || last) {
+            xw[tm.row(q)] = X[q];
+            const int b = ((__double2hiint(io.b[tm.row(q)]) >> 20) & 0x7ff) - 1022;
+            const int l = max(64 - __clzll(X[q] ^ (X[q] >> 63)) + eX, b);
+            hi = max(hi, l);
+            lo = min(lo, l);
+        }
+    hi = g.max_int(hi);
+    lo = -g.max_int(-lo);
 #pragma unroll 1
     for (int row = moved ? tm.tid : n; row < n; row += tm.nt) {
         const Sc d = unpack(diag_entry<FMT>(A, row));
         const double x = to_double(mul(normal(xw[row], eX), rcp(d)));
-        io.x[row] = x;
-        const Sc xr = unpack(x);
-        xw[row] = round_shr(mul62(xr.m, d.m), eX - xr.e - d.e - 62);
+        xw[row] = __double_as_longlong(x);
+        const Sc u = unpack(x);
+        xr[row] = round_shr(mul62(u.m, d.m), eX - u.e - d.e - 62);
     }
     // where that rounding weighs in the residual (below 4e-12), the log takes
     // the residual of the rounded x
-    const bool close = moved && le(res2, Sc{nb2.m, nb2.e - 76});
-    if (g.any(close)) {
+    const bool exact = !known || (moved && le(res2, Sc{nb2.m, nb2.e - 76}));
+    const bool wide = hi - lo > kRowScaleBits;
+    if (g.any(take && (exact || wide))) {
+        if (moved) {
 #pragma unroll
-        for (int q = 0; q < R; ++q)
-            if (q + 1 < R || last) X[q] = xw[tm.row(q)];
-        const Sc res = true_residual<SF>(S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, false, g, tm);
-        if (close) res2 = res;
+            for (int q = 0; q < R; ++q)
+                if (q + 1 < R || last) X[q] = xr[tm.row(q)];
+        }
+        int ey = 0;
+        const Sc res = true_residual<SF>(S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, false, g, tm, &ey);
+        if (exact) res2 = res;
+        if (g.any(take && wide)) {
+            Abs t[R];
+            spmv_sums<SF, 64>(S, as, pb, t, 0, tm);
+            int h = -100000, l = 100000;
+#pragma unroll
+            for (int q = 0; q < R; ++q)
+                if (q + 1 < R || last) {
+                    const int b = ((__double2hiint(io.b[tm.row(q)]) >> 20) & 0x7ff) - 1022;
+                    const int v = max(64 - __clzll(t[q].hh) + ey + sigma - 2, b);
+                    h = max(h, v);
+                    l = min(l, v);
+                }
+            h = g.max_int(h);
+            l = -g.max_int(-l);
+            if (wide) {
+                hi = h;
+                lo = l;
+            }
+        }
     }
-    if (run) {
+    const bool good = take && hi - lo <= kRowScaleBits + 1;
+    if (good) {
+#pragma unroll 1
+        for (int row = moved ? tm.tid : n; row < n; row += tm.nt) io.x[row] = __longlong_as_double(xw[row]);
         if (tm.tid == 0) {
             *io.iters = iters;
             *io.rel_res = sqrt(to_double(res2) / to_double(nb2));
@@ -809,6 +903,7 @@ __device__ __forceinline__ void folded_finish(const Mat<double>& A, const Mat<do
             if (io.inner != nullptr) *io.inner = 0;
         }
     }
+    return good;
 }
 
 // --------------------------------------------------------------- BiCGSTAB
@@ -836,7 +931,7 @@ __device__ __forceinline__ Fit bicgstab_fixed(const Mat<double>& A, const Mat<do
     int eX = kNone, bX = 0, eR, bR, sigma;
     bool run;
     Sc nb2;
-    if (!folded_setup<FMT, SF>(A, S, io, valid, sm, g, tm, X, eX, bX, Rv, eR, bR, sigma, run, nb2)) {
+    if (!folded_setup<FMT, SF, kBicgstab>(A, S, io, valid, sm, g, tm, X, eX, bX, Rv, eR, bR, sigma, run, nb2)) {
         // (the block's other warps count on this one at their barriers)
         for (int it = 1; it <= C.max_iters && g.live(false); ++it) {
         }
@@ -851,14 +946,10 @@ __device__ __forceinline__ Fit bicgstab_fixed(const Mat<double>& A, const Mat<do
     int eH = eR;  // r^ = r
     int status = -1, iters = 0, restarts = 0;
     Sc res2 = rr;
-    bool have_res = true, active = run;
-    if (active) {
-        if (le(rr, tau2)) {
-            status = ST_CONVERGED;
-            active = false;
-        } else {
-            have_res = false;
-        }
+    bool active = run;
+    if (active && le(rr, tau2)) {
+        status = ST_CONVERGED;
+        active = false;
     }
     Sc rho = rr, alpha = one(), omega = one(), cfac = one();
     int eP = kNone, bP = 0, eV = kNone, bV = 0;
@@ -1063,18 +1154,16 @@ __device__ __forceinline__ Fit bicgstab_fixed(const Mat<double>& A, const Mat<do
             const Sc res = residual(cand);
             if (cand) {
                 res2 = res;
-                have_res = true;
-                if (!finite(res2)) {
+                if (!finite(res)) {
                     status = ST_NAN;
                     active = false;
-                } else if (le(res2, tau2)) {
+                } else if (le(res, tau2)) {
                     status = ST_CONVERGED;
                     active = false;
                 } else if (++restarts > kMaxRestarts) {
                     status = kStagnated;
                     active = false;
                 } else {
-                    have_res = false;
 #pragma unroll
                     for (int q = 0; q < R; ++q) {
                         const int row = tm.row(q);
@@ -1085,7 +1174,7 @@ __device__ __forceinline__ Fit bicgstab_fixed(const Mat<double>& A, const Mat<do
                     eH = eR;
                     eP = eV = kNone;
                     bP = bV = 0;
-                    rho = res2;
+                    rho = res;
                     alpha = omega = cfac = one();
                     restarted = true;
                 }
@@ -1101,13 +1190,10 @@ __device__ __forceinline__ Fit bicgstab_fixed(const Mat<double>& A, const Mat<do
         }
     }
     if (active) status = ST_MAX_ITER;
-    const bool done = run && accepted(status), need = done && !have_res;
-    if (g.any(need)) {
-        const Sc res = residual(false);
-        if (need) res2 = res;
-    }
-    folded_finish<FMT, SF>(A, S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, done, iters, status, res2, nb2, sm, g, tm);
-    return done ? kDone : run ? kLeft : kUnfit;
+    return folded_finish<FMT, SF>(A, S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, run && accepted(status), iters, status,
+                                  status == ST_CONVERGED, res2, nb2, sm, g, tm)
+               ? kDone
+               : run ? kLeft : kUnfit;
 }
 
 }  // namespace fx

@@ -33,7 +33,7 @@ __device__ __forceinline__ Fit gmres_fixed(const Mat<double>& A, const Mat<doubl
     int eX, bX, eR, bR, sigma;
     bool run;
     Sc nb2;
-    if (!folded_setup<FMT, SF>(A, S, io, valid, sm, g, tm, X, eX, bX, Rv, eR, bR, sigma, run, nb2)) return kUnfit;
+    if (!folded_setup<FMT, SF, kGmres>(A, S, io, valid, sm, g, tm, X, eX, bX, Rv, eR, bR, sigma, run, nb2)) return kUnfit;
     const bool last = tm.row(R - 1) < n;  // only a lane's last row may lie past the end
     // exponent of w = A v and what is left of it: every ||w|| is at most the
     // matrix's Frobenius norm (below 2^fexp), and orthogonalising only shortens w, so
@@ -276,17 +276,16 @@ __device__ __forceinline__ Fit gmres_fixed(const Mat<double>& A, const Mat<doubl
             }
         }
     }
-    const bool done = run && accepted(status);
+    const bool done = folded_finish<FMT, SF>(A, S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, run && accepted(status), it,
+                                             status, true, beta2, nb2, sm, g, tm);
     // The basis is dead scratch from here on: its whole 128-byte lines are dropped
     // from L2 without a write-back (as gmres_packed_system).
-    g.sync();
     if (done && V != nullptr) {
         const uintptr_t first = (reinterpret_cast<uintptr_t>(V) + 127) & ~static_cast<uintptr_t>(127);
         const uintptr_t end = (reinterpret_cast<uintptr_t>(V) + (size_t)(m + 1) * vs * 8) & ~static_cast<uintptr_t>(127);
         for (uintptr_t a = first + (uintptr_t)tm.tid * 128; a < end; a += (uintptr_t)tm.nt * 128)
             asm volatile("discard.global.L2 [%0], 128;" ::"l"(a) : "memory");
     }
-    folded_finish<FMT, SF>(A, S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, done, it, status, beta2, nb2, sm, g, tm);
     return done ? kDone : run ? kLeft : kUnfit;
 }
 
