@@ -824,14 +824,17 @@ __device__ __forceinline__ bool folded_setup(const Mat<double>& A, const Mat<dou
 }
 
 // The end of such a solve, for the groups with `take` set: x = D^-1 x~ rounded
-// to FP64 and the log. `known`: res2 is the true residual of x~. Returns whether
-// the result stands: the scales of its rows (setup's, with x~ for y) have to be in
-// reach of each other. If not, nothing has been written and FP64 solves the system.
+// to FP64, its residual, and the log. `known`: res2 is the true residual of x~.
+// Returns whether the result stands: a system that has converged has to have done
+// so as it is returned, and the scales of its rows (setup's, with x~ for y) have
+// to be in reach of each other. If not, nothing has been written and FP64 solves
+// the system.
 template <int FMT, int SF, int R, class G>
 __device__ __forceinline__ bool folded_finish(const Mat<double>& A, const Mat<double>& S, const int2* as, int2* pb,
                                               const SysIO& io, int sigma, long long (&X)[R], int& eX, int& bX,
                                               long long (&Rv)[R], int& eR, int& bR, bool take, int iters, int status,
-                                              bool known, Sc res2, Sc nb2, const TeamSmem& sm, G& g, const Team& tm) {
+                                              bool known, Sc res2, Sc tau2, Sc nb2, const TeamSmem& sm, G& g,
+                                              const Team& tm) {
     if (!g.any(take)) return false;
     const int n = io.n;
     const bool last = tm.row(R - 1) < n;
@@ -859,9 +862,12 @@ __device__ __forceinline__ bool folded_finish(const Mat<double>& A, const Mat<do
         const Sc u = unpack(x);
         xr[row] = round_shr(mul62(u.m, d.m), eX - u.e - d.e - 62);
     }
-    // where that rounding weighs in the residual (below 4e-12), the log takes
-    // the residual of the rounded x
-    const bool exact = !known || (moved && le(res2, Sc{nb2.m, nb2.e - 76}));
+    // Rounding moves the residual by at most 2^-53 of the row sums of |A~| |x~|:
+    // below 2^(sigma + hi - 53 + 6) in the norm (2,048 rows). Where that is below 2^-12 of
+    // the known residual, the log states it, and a converged system has converged
+    // unless the two are as close to the tolerance.
+    const int slack = 2 * (sigma + hi - 53 + 6 + 12);
+    const bool exact = !known || (moved && (res2.e + 61 < slack || (status == ST_CONVERGED && !le(res2, normal(tau2.m - (tau2.m >> 11), tau2.e)))));
     const bool wide = hi - lo > kRowScaleBits;
     if (g.any(take && (exact || wide))) {
         if (moved) {
@@ -892,7 +898,8 @@ __device__ __forceinline__ bool folded_finish(const Mat<double>& A, const Mat<do
             }
         }
     }
-    const bool good = take && hi - lo <= kRowScaleBits + 1;
+    const bool good = take && hi - lo <= kRowScaleBits + 1 && finite(res2) &&
+                      (status != ST_CONVERGED || le(res2, tau2));
     if (good) {
 #pragma unroll 1
         for (int row = moved ? tm.tid : n; row < n; row += tm.nt) io.x[row] = __longlong_as_double(xw[row]);
@@ -1191,7 +1198,7 @@ __device__ __forceinline__ Fit bicgstab_fixed(const Mat<double>& A, const Mat<do
     }
     if (active) status = ST_MAX_ITER;
     return folded_finish<FMT, SF>(A, S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, run && accepted(status), iters, status,
-                                  status == ST_CONVERGED, res2, nb2, sm, g, tm)
+                                  status == ST_CONVERGED, res2, tau2, nb2, sm, g, tm)
                ? kDone
                : run ? kLeft : kUnfit;
 }

@@ -277,7 +277,7 @@ __device__ __forceinline__ Fit gmres_fixed(const Mat<double>& A, const Mat<doubl
         }
     }
     const bool done = folded_finish<FMT, SF>(A, S, as, pb, io, sigma, X, eX, bX, Rv, eR, bR, run && accepted(status), it,
-                                             status, true, beta2, nb2, sm, g, tm);
+                                             status, true, beta2, tau2, nb2, sm, g, tm);
     // The basis is dead scratch from here on: its whole 128-byte lines are dropped
     // from L2 without a write-back (as gmres_packed_system).
     if (done && V != nullptr) {

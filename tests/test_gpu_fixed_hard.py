@@ -114,3 +114,20 @@ def test_small_entries_survive(bbs, handle, name, guess, solver, tps):
     xr, _, _, sr = oracle.solve_batch(A, b, x0, solver=solver)[:4]
     assert np.array_equal(st, sr) and (sr == 0).all()
     assert (np.abs(x - xr) <= 1e-8 * np.abs(xr)).all(), np.abs(x / xr - 1).max()
+
+
+@pytest.mark.parametrize("solver,fmt,tol", [("bicgstab", "csr", 1e-14), ("bicgstab", "ell", 4e-15),
+                                            ("gmres", "csr", 4e-15), ("bicgstab", "csr", 1e-10)])
+def test_status_and_log_are_those_of_the_returned_x(bbs, handle, solver, fmt, tol):
+    """At tolerances where rounding x to FP64 weighs: a system is CONVERGED only with
+    a logged residual within the tolerance, and the log is the returned x's (to
+    1e-3, or to the 1e-15 that FP64's own residual is good to)."""
+    rng = np.random.default_rng(14)
+    pat, vals = recipe("2d5", 12, 12, 8000, 0.05, 0.5, rng, symmetric=solver == "cg")
+    b = rng.uniform(-1, 1, (len(vals), pat.n))
+    x, _, rel, st = gpu_solve(bbs, handle, W.make_batch(pat, vals, fmt), b, None, solver=solver, tol=tol)[:4]
+    assert (rel[st == 0] <= tol).all(), (int((rel[st == 0] > tol).sum()), rel[st == 0].max())
+    pick = np.argsort(rel)[:: len(rel) // 200]
+    D = W.to_dense(pat, vals[pick]).reshape(-1, pat.n, pat.n)
+    rh = host_rel_residual(D, x[pick], b[pick])
+    assert (np.abs(rel[pick] - rh) <= 1e-3 * rh + 1e-15).all()
