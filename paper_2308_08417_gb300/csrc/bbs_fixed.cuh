@@ -50,8 +50,10 @@ constexpr int kNone = -1000000;  // exponent of a vector that is zero
 constexpr float kRowSumMax = 31.0f;
 // What a system must be like to be solved here, and what became of it.
 constexpr float kExcess = 0x1p-7f;    // BiCGSTAB: least diagonal excess of a row, (|a_ii| - sum of the others) / |a_ii|
+constexpr float kExcessCg = 0x1p-9f;  // CG
 constexpr float kRowScale = 0x1p-12f; // smallest row scale against the largest
 constexpr int kRowScaleBits = 12;
+constexpr int kDiagonalBits = 24;     // CG: spread of the diagonal
 // Statuses that end a solve here; of a system that stops in another way nothing is
 // written.
 constexpr int kStagnated = -2;
@@ -690,13 +692,15 @@ __device__ __forceinline__ Sc true_residual(const Mat<double>& S, const int2* as
 //     rows in other units, entries that matter at 1e-6 and 1e-20 alike and parts
 //     of a system that hardly meet would lose theirs (A = diag(1, 2^-70), b = (1,
 //     2^-70): x = (1, 0)). folded_finish looks at the solution in the same way;
-//   * BiCGSTAB: each row's diagonal entry exceeds its others by 2^-7. Below that
-//     the Krylov vectors fall and rise by more than the spare bits in a step, and
-//     systems that take more iterations than they have rows took up to 4 % more of
-//     them (3-point, n = 64, excess 0.001: 93.7 for 89.8 in FP64, 0.008: 71.3 for
-//     70.9, 0.016 and more the same; tridiag(-1, 2, -1), n = 256: 315 for 270).
-//     GMRES has no line: it starts afresh from the true residual every few steps.
-enum Method { kBicgstab, kGmres };
+//   * BiCGSTAB and CG: each row's diagonal entry exceeds its others by 2^-7 and by
+//     2^-9. Below that the Krylov vectors fall and rise by more than the spare bits
+//     in a step, and systems that take more iterations than they have rows took up
+//     to 4 % more of them (3-point, n = 64; BiCGSTAB with excess 0.001: 93.7 for 89.8
+//     in FP64, 0.008: 71.3 for 70.9, 0.016 and more the same; CG 0.0001: 74.8 for
+//     74.0, 0.001: 67.9 for 67.7, 0.004 and more the same). GMRES has no line: it
+//     starts afresh from the true residual every few steps;
+//   * CG: the diagonal is positive and within 2^24 of itself (bbs_fixed_cg.cuh).
+enum Method { kBicgstab, kCg, kGmres };
 template <int FMT, int SF, Method METHOD, int R, class G>
 __device__ __forceinline__ bool folded_setup(const Mat<double>& A, const Mat<double>& S, const SysIO& io, bool valid,
                                              const TeamSmem& sm, G& g, const Team& tm, long long (&X)[R], int& eX,
@@ -712,7 +716,7 @@ __device__ __forceinline__ bool folded_setup(const Mat<double>& A, const Mat<dou
     // (loops over the caller's rows stay rolled here: this runs once)
     long long* dm = in_shared<long long>(sm.xb);  // 1 / a_ii: its digits,
     int2* de = pa;                                // its exponent beside y_i's biased one, and its FP32 value
-    int bad = 0, eb = 0, exm = 0, yleast = 0x7ff;
+    int bad = 0, eb = 0, exm = 0, yleast = 0x7ff, dmost = -100000, dleast = 100000;
 #pragma unroll 1
     for (int row = tm.tid; row < n; row += tm.nt) {
         double d = 0.0;
@@ -722,6 +726,11 @@ __device__ __forceinline__ bool folded_setup(const Mat<double>& A, const Mat<dou
         bad |= normal64(d) ? 0 : 1;
         const Sc di = rcp(unpack(d));
         dm[row] = di.m;
+        if (METHOD == kCg) {
+            bad |= d > 0.0 ? 0 : 1;
+            dmost = max(dmost, di.e);
+            dleast = min(dleast, di.e);
+        }
         const double xt = d * io.x[row];
         const int yb = (__double2hiint(io.b[row]) >> 20) & 0x7ff;
         const int yx = zero64(xt) ? 0 : max(1, (__double2hiint(xt) >> 20) & 0x7ff);
@@ -739,11 +748,12 @@ __device__ __forceinline__ bool folded_setup(const Mat<double>& A, const Mat<dou
             if (col >= 0) {
                 const float v = fabsf((float)S.vals[e]);
                 t = fmaf(v, __int_as_float(de[col].y), t);
-                if (METHOD == kBicgstab) u += v;
+                if (METHOD != kGmres) u += v;
             }
         });
         top = max(top, __float_as_int(t * 1.0001f) & 0x7fffffff);
-        if (METHOD == kBicgstab) bad |= u * __int_as_float(de[row].y) <= 2.0f - kExcess ? 0 : 1;
+        if (METHOD != kGmres)
+            bad |= u * __int_as_float(de[row].y) <= 2.0f - (METHOD == kCg ? kExcessCg : kExcess) ? 0 : 1;
     }
     top = g.max_int(bad ? 0x7fffffff : top);
     eb = g.max_int(eb);
@@ -751,7 +761,8 @@ __device__ __forceinline__ bool folded_setup(const Mat<double>& A, const Mat<dou
     yleast = -g.max_int(-yleast);
     const int ym = max(eb, exm);
     const bool xz = exm == 0;  // the guess is zero
-    run = valid && top < __float_as_int(kRowSumMax) && eb > 623 && eb < 1423 &&
+    const int spread = METHOD == kCg ? g.max_int(dmost) + g.max_int(-dleast) : 0;
+    run = valid && top < __float_as_int(kRowSumMax) && spread <= kDiagonalBits && eb > 623 && eb < 1423 &&
           (xz || (exm > 623 && exm < 1423));
     if (g.any(run && ym - yleast >= kRowScaleBits)) {  // y_i alone does not show it: rare
         int low = 0x7f800000;  // smallest row scale, against 2^ym

@@ -571,7 +571,7 @@ __device__ __forceinline__ void cg_packed_any(const PackedOp<FMT, R>& op, const 
                                               const SolveCfg& C, const TeamSmem& sm, const Team& tm) {
     fx::Fit fit = fx::kUnfit;
     if (C.precond == 1)  // every lane takes part, those without a system too
-        fit = fx::cg_fixed<staged_fmt<FMT>(), R>(op.A, op.S, io, valid, C, sm, fx::Lanes<L>{tm.lane}, tm);
+        fit = fx::cg_fixed<FMT, staged_fmt<FMT>(), R>(op.A, op.S, io, valid, C, sm, fx::Lanes<L>{tm.lane}, tm);
     const bool left = valid && fit != fx::kDone;
     if (__any_sync(kFull, left)) {
         __syncwarp();

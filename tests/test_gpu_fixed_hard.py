@@ -6,7 +6,7 @@ import pytest
 
 import oracle
 from paper_2308_08417_gb300 import workloads as W
-from tests.parity import host_rel_residual
+from tests.parity import compare, host_rel_residual, iteration_spread
 from tests.test_gpu_parity import gpu_solve
 
 pytestmark = pytest.mark.gpu
@@ -97,7 +97,7 @@ def graded(name, n, batch, rng):
 
 
 @pytest.mark.parametrize("tps", [0, 64])
-@pytest.mark.parametrize("solver", ["bicgstab", "gmres"])
+@pytest.mark.parametrize("solver", ["bicgstab", "cg", "gmres"])
 @pytest.mark.parametrize("guess", [False, True])
 @pytest.mark.parametrize("name", ["diagonal", "weakly coupled", "rows 2^-30", "rows 2^-70", "b 2^-30", "b 2^-70"])
 def test_small_entries_survive(bbs, handle, name, guess, solver, tps):
@@ -106,6 +106,9 @@ def test_small_entries_survive(bbs, handle, name, guess, solver, tps):
     rng = np.random.default_rng(13)
     n, B = 24, 9
     pat, vals, b = graded(name, n, B, rng)
+    if solver == "cg" and name.startswith("rows"):  # symmetric: the columns too
+        s = np.where(np.arange(n) < n // 2, 1.0, 2.0 ** -int(name.split("^-")[1]))
+        vals = vals * s[pat.col_idxs]
     A = W.make_batch(pat, vals, "csr")
     x0 = None
     if guess:
@@ -116,7 +119,7 @@ def test_small_entries_survive(bbs, handle, name, guess, solver, tps):
     assert (np.abs(x - xr) <= 1e-8 * np.abs(xr)).all(), np.abs(x / xr - 1).max()
 
 
-@pytest.mark.parametrize("solver,fmt,tol", [("bicgstab", "csr", 1e-14), ("bicgstab", "ell", 4e-15),
+@pytest.mark.parametrize("solver,fmt,tol", [("bicgstab", "csr", 1e-14), ("bicgstab", "ell", 4e-15), ("cg", "csr", 4e-15),
                                             ("gmres", "csr", 4e-15), ("bicgstab", "csr", 1e-10)])
 def test_status_and_log_are_those_of_the_returned_x(bbs, handle, solver, fmt, tol):
     """At tolerances where rounding x to FP64 weighs: a system is CONVERGED only with
@@ -131,3 +134,27 @@ def test_status_and_log_are_those_of_the_returned_x(bbs, handle, solver, fmt, to
     D = W.to_dense(pat, vals[pick]).reshape(-1, pat.n, pat.n)
     rh = host_rel_residual(D, x[pick], b[pick])
     assert (np.abs(rel[pick] - rh) <= 1e-3 * rh + 1e-15).all()
+
+
+@pytest.mark.parametrize("fmt,tps", [("csr", 0), ("ell", 4), ("dense", 16), ("csr", 32), ("ell", 64)])
+@pytest.mark.parametrize("bits", [6, 20, 30])
+def test_cg_with_diagonals_far_apart(bbs, handle, fmt, tps, bits):
+    """Symmetric systems whose diagonal entries lie 2^bits apart (inside the range of
+    the weights, near its end and beyond it), as a 3-point batch has them at its
+    corners: the oracle's x, iterations and status."""
+    rng = np.random.default_rng(bits)
+    n, B = 40, 33
+    pat, vals = recipe("1d3", n, 1, B, 0.05, 0.5, rng, symmetric=True)
+    rows = np.repeat(np.arange(n), np.diff(pat.row_ptrs))
+    s = np.ones((B, n))
+    s[np.arange(B), rng.integers(0, n, B)] = 2.0 ** (-bits / 2)  # one small row and column
+    vals = vals * s[:, rows] * s[:, pat.col_idxs]
+    b = rng.uniform(-1, 1, (B, n)) * s
+    for x0 in (None, rng.uniform(-1, 1, (B, n))):
+        A = W.make_batch(pat, vals, fmt)
+        g = gpu_solve(bbs, handle, A, b, x0, solver="cg", threads_per_system=tps)
+        r = oracle.solve_batch(A, b, x0, solver="cg")
+        D = W.to_dense(pat, vals).reshape(-1, n, n)
+        fails = compare(*g[:4], r[0], r[1], r[3], rel_host=host_rel_residual(D, g[0], b), label=f"{fmt} {tps}",
+                        iter_tol=2 + iteration_spread(oracle.solve_batch, A, b, x0, solver="cg"))
+        assert not fails, "\n".join(fails)
