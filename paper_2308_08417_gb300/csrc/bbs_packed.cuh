@@ -352,6 +352,22 @@ __device__ __forceinline__ void bicgstab_packed_system(const PackedOp<FMT, R>& o
     }
 }
 
+// The arguments of a function of its own, as its caller knows them: the group's
+// lanes, and pointers into shared memory. Batches of n = 144 that FP64 solves
+// whole, without -> with: 8,192 systems, 63 iterations 5.16 -> 5.06 ms; 16,384, 20
+// iterations 3.30 -> 3.18 ms. (CG is slower with them, 3.17 -> 3.49 ms, and goes without.)
+template <int FMT, int L, int R>
+struct PackedArgs {
+    PackedOp<FMT, R> op;
+    TeamSmem sm;
+    Team tm;
+    __device__ __forceinline__ PackedArgs(const PackedOp<FMT, R>& o, const TeamSmem& s, const Team& t)
+        : op(o), sm{nullptr, fx::in_shared<double>(s.xa), fx::in_shared<double>(s.xb), nullptr},
+          tm{t.lane & (L - 1), L, t.lane, 0, 1, 0} {
+        op.S.vals = fx::in_shared<double>(o.S.vals);
+    }
+};
+
 // BiCGSTAB of a warp's groups: with Jacobi in block fixed point (the integer
 // pipe); the groups it leaves (and all of them without Jacobi) in FP64. The
 // FP64 form is compiled as a function of its own. `again` (per group): the staged
@@ -359,9 +375,10 @@ __device__ __forceinline__ void bicgstab_packed_system(const PackedOp<FMT, R>& o
 template <int FMT, int L, int R>
 __device__ __noinline__ void bicgstab_packed_fp64(const PackedOp<FMT, R> op, const SysIO io, bool valid, bool again,
                                                   const SolveCfg C, const TeamSmem sm, const Team tm) {
-    if (again) op.stage(tm);
+    const PackedArgs<FMT, L, R> a(op, sm, tm);
+    if (again) a.op.stage(a.tm);
     __syncwarp();
-    bicgstab_packed_system<FMT, L, R>(op, io, valid, C, sm, tm);
+    bicgstab_packed_system<FMT, L, R>(a.op, io, valid, C, a.sm, a.tm);
 }
 
 template <int FMT, int L, int R>
@@ -857,10 +874,11 @@ __device__ __forceinline__ void gmres_packed_system(const PackedOp<FMT, R>& op, 
 
 template <int FMT, int L, int R>
 __device__ __noinline__ void gmres_packed_fp64(const PackedOp<FMT, R> op, const SysIO io, bool valid, bool again,
-                                               const SolveCfg C, double* xa, double* ext, const Team tm) {
-    if (again) op.stage(tm);
+                                               const SolveCfg C, const TeamSmem sm, double* ext, const Team tm) {
+    const PackedArgs<FMT, L, R> a(op, sm, tm);
+    if (again) a.op.stage(a.tm);
     __syncwarp();
-    gmres_packed_system<FMT, L, R>(op, io, valid, C, xa, ext, tm);
+    gmres_packed_system<FMT, L, R>(a.op, io, valid, C, a.sm.xa, fx::in_shared<double>(ext), a.tm);
 }
 
 // ------------------------------------------------------------- kernels
@@ -965,7 +983,7 @@ __global__ void __launch_bounds__(32, packed_cg_min_blocks(R)) gmres_packed_kern
     if (__any_sync(kFull, left)) {
         __syncwarp();
         gmres_packed_fp64<FMT, L, R>(G.op, sys_io(P, G.sys), left, left && fit == fx::kLeft, solve_cfg(P, G.sys),
-                                     G.sm.xa, ext, G.tm);
+                                     G.sm, ext, G.tm);
     }
 }
 

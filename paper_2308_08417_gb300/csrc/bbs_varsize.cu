@@ -401,7 +401,7 @@ bbs_status build_plan(bbs_handle* h, const PlanInputs& in, bbs_var_plan** out) {
         c.smem = (size_t)c.P.slice * (size_t)(32 / c.L);
         // blocks of several warps in step, as bbs_solve launches full batches
         const int warps = (c.P.count + 32 / c.L - 1) / (32 / c.L);
-        if (warps > bbs::kPackedWarps * sms &&
+        if (in.o->precond == BBS_PREC_JACOBI && warps > bbs::kPackedWarps * sms &&
             c.smem * bbs::kPackedWarps <= (size_t)optin)
             c.warps = bbs::kPackedWarps;
         c.smem *= (size_t)c.warps;
