@@ -44,6 +44,18 @@ struct bbs_handle {
     std::mutex checked_mutex;
 };
 
+namespace bbs {
+cudaError_t allow_smem(const void* fn, size_t smem) {
+    if (smem <= 48 * 1024) return cudaSuccess;
+    static std::mutex mutex;
+    std::lock_guard<std::mutex> lock(mutex);
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, fn);
+    if (e != cudaSuccess || (size_t)a.maxDynamicSharedSizeBytes >= smem) return e;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+}  // namespace bbs
+
 namespace {
 
 thread_local std::string g_last_error;
@@ -366,14 +378,6 @@ const void* pick_kernel(const bbs_options* o, int fmt, int R, bool staged, int e
     }
 }
 
-std::mutex g_attr_mutex;
-
-cudaError_t allow_smem(const void* fn, size_t smem) {
-    if (smem <= 48 * 1024) return cudaSuccess;
-    std::lock_guard<std::mutex> lock(g_attr_mutex);
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
 // Packed CSR solves stage each system's values through an ELL table of
 // width ell_k, so a row longer than ell_k is an argument error. The row
 // pointers are device data: the first solve with a pattern (keyed by its
@@ -647,7 +651,7 @@ bbs_status bbs_solve(bbs_handle* h, const bbs_batch_matrix* A, const double* b, 
     }
     if (p.ilu && p.lanes == 32) {
         const void* fn = bbs::bicgstab_ilu_fn(p.R);
-        if ((e = allow_smem(fn, p.smem)) != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
+        if ((e = bbs::allow_smem(fn, p.smem)) != cudaSuccess) return cuda_fail(e, "shared memory limit");
         void* args[] = {&P, &csched};
         e = cudaLaunchKernel(fn, dim3((unsigned)A->num_batch), dim3((unsigned)p.threads), args, p.smem, st);
         return e == cudaSuccess ? BBS_OK : cuda_fail(e, "ILU(0) solver launch");
@@ -673,7 +677,7 @@ bbs_status bbs_solve(bbs_handle* h, const bbs_batch_matrix* A, const double* b, 
                          : o->solver == BBS_SOLVER_CG ? bbs::cg_packed_fn(A->fmt, p.lanes, p.R)
                          : o->solver == BBS_SOLVER_GMRES ? bbs::gmres_packed_fn(A->fmt, p.lanes, p.R)
                                                          : bbs::bicgstab_packed_fn(A->fmt, p.lanes, p.R);
-        if ((e = allow_smem(fn, p.smem * p.warps)) != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
+        if ((e = bbs::allow_smem(fn, p.smem * p.warps)) != cudaSuccess) return cuda_fail(e, "shared memory limit");
         void* args[] = {&P, &csched};  // the ILU(0) kernels take the schedule as a second argument
         const unsigned warps = (unsigned)((A->num_batch + per_block - 1) / per_block);
         const unsigned blocks = (warps + p.warps - 1) / p.warps;
@@ -681,7 +685,7 @@ bbs_status bbs_solve(bbs_handle* h, const bbs_batch_matrix* A, const double* b, 
         return e == cudaSuccess ? BBS_OK : cuda_fail(e, "packed solver launch");
     }
     const void* fn = pick_kernel(o, A->fmt, p.R, p.stage, A->ell_k, p.threads);
-    if ((e = allow_smem(fn, p.smem)) != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
+    if ((e = bbs::allow_smem(fn, p.smem)) != cudaSuccess) return cuda_fail(e, "shared memory limit");
     void* args[] = {&P};
     e = cudaLaunchKernel(fn, dim3((unsigned)A->num_batch), dim3((unsigned)p.threads), args, p.smem, st);
     if (e != cudaSuccess) return cuda_fail(e, "solver launch");

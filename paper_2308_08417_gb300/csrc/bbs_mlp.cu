@@ -753,9 +753,12 @@ bool gemm_maps(CUtensorMap* ta, CUtensorMap* tb, const __nv_bfloat16* A, int lda
            make_operand_map(tb, B, N, K, ldb, BN, bbs::umma::kBK);
 }
 
-template <class Kernel>
-cudaError_t gemm_attr(Kernel k) {
-    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bbs::umma::smem_bytes(64));
+// What the tcgen05 GEMMs need of the current device (once per object: the launches
+// of a step do not look again).
+cudaError_t allow_gemms() {
+    const size_t smem = bbs::umma::smem_bytes(64);
+    const cudaError_t e = bbs::allow_smem((const void*)bbs::mlp::gemm_umma_kernel, smem);
+    return e != cudaSuccess ? e : bbs::allow_smem((const void*)bbs::mlp::weight_grads_kernel, smem);
 }
 
 // C = A B^T through the chosen tensor-core path (kind 1: tcgen05 with the
@@ -767,12 +770,6 @@ cudaError_t gemm_any(int kind, const __nv_bfloat16* A, int lda, const __nv_bfloa
         const Tiles t = gemm_tiles(M, N, K, e.mode == bbs::mlp::EPI_F32 && part != nullptr, part_cap, sms);
         CUtensorMap ta, tb;
         if (!gemm_maps(&ta, &tb, A, lda, B, ldb, M, N, K, t.BN)) return cudaErrorInvalidValue;
-        static bool attr_set = false;
-        if (!attr_set) {
-            cudaError_t a = gemm_attr(bbs::mlp::gemm_umma_kernel);
-            if (a != cudaSuccess) return a;
-            attr_set = true;
-        }
         dim3 grid(t.nt, t.mt, t.splits);
         const size_t smem = bbs::umma::smem_bytes(t.BN);
         if (t.splits == 1) {
@@ -930,11 +927,6 @@ cudaError_t backward(bbs_mlp* m, int M, float* loss, const bbs::mlp::Adam* adam,
         }
     }
     if (tc) {
-        static bool attr_set = false;
-        if (!attr_set) {
-            if ((e = gemm_attr(weight_grads_kernel)) != cudaSuccess) return e;
-            attr_set = true;
-        }
         if ((e = launch_early(weight_grads_kernel, dim3(w.first[kLayers]), bbs::umma::kThreads,
                               bbs::umma::smem_bytes(64), st, w, M, m->err)) != cudaSuccess)
             return e;
@@ -1045,11 +1037,10 @@ bbs_status bbs_mlp_create(bbs_handle* h, int32_t n, int32_t hidden, uint64_t see
         m->fused = make_operand_map(&m->infer_maps[l], m->Wb[l], outs[l], m->pad_in[l], m->pad_in[l],
                                     l < 3 ? hidden : m->n_mma);
     if (m->fused)
-        m->fused = cudaFuncSetAttribute(bbs::mlp::mlp_infer_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)L.total) == cudaSuccess &&
-                   cudaFuncSetAttribute(bbs::mlp::mlp_infer_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)L.total) == cudaSuccess;
-    cudaError_t e = cudaDeviceSynchronize();
+        m->fused = bbs::allow_smem((const void*)bbs::mlp::mlp_infer_kernel<false>, L.total) == cudaSuccess &&
+                   bbs::allow_smem((const void*)bbs::mlp::mlp_infer_kernel<true>, L.total) == cudaSuccess;
+    cudaError_t e = allow_gemms();
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         bbs_mlp_destroy(m);
         return errf(BBS_ERR_CUDA, "MLP init: %s", cudaGetErrorString(e));
@@ -1201,8 +1192,10 @@ bbs_status bbs_gemm_bf16(bbs_handle* h, int32_t kind, const uint16_t* A, int32_t
     if (kind == BBS_GEMM_TCGEN05 && cudaMalloc(&part, part_cap * sizeof(float)) != cudaSuccess) part = nullptr;
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, bbs::handle_device(h));
-    e = gemm_any(kind, reinterpret_cast<const __nv_bfloat16*>(A), lda, reinterpret_cast<const __nv_bfloat16*>(B),
-                 ldb, M, N, K, ep, err, nullptr, part, part ? part_cap : 0, sms > 0 ? sms : 152);
+    e = allow_gemms();
+    if (e == cudaSuccess)
+        e = gemm_any(kind, reinterpret_cast<const __nv_bfloat16*>(A), lda, reinterpret_cast<const __nv_bfloat16*>(B),
+                     ldb, M, N, K, ep, err, nullptr, part, part ? part_cap : 0, sms > 0 ? sms : 152);
     int flag = 0;
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e == cudaSuccess) e = cudaMemcpy(&flag, err, sizeof(int), cudaMemcpyDeviceToHost);

@@ -8,7 +8,6 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
-#include <mutex>
 #include <numeric>
 #include <vector>
 
@@ -94,18 +93,6 @@ int pow2_at_least(int v) {
     int p = 1;
     while (p < v) p <<= 1;
     return p;
-}
-
-// Lets fn use smem bytes of dynamic shared memory. The limit belongs to the
-// function, which the plan's other classes and other plans use too: it is only
-// ever raised.
-cudaError_t allow_smem(const void* fn, size_t smem) {
-    static std::mutex mutex;
-    std::lock_guard<std::mutex> lock(mutex);
-    cudaFuncAttributes a;
-    const cudaError_t e = cudaFuncGetAttributes(&a, fn);
-    if (e != cudaSuccess || (size_t)a.maxDynamicSharedSizeBytes >= smem) return e;
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
 bool is_pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
@@ -480,7 +467,7 @@ bbs_status build_plan(bbs_handle* h, const PlanInputs& in, bbs_var_plan** out) {
                         pl->smem, optin);
         }
         pl->fn = rmax == 8 ? bbs::varsize_kernel8_fn() : bbs::varsize_kernel4_fn();
-        if ((e = allow_smem(pl->fn, pl->smem)) != cudaSuccess) {
+        if ((e = bbs::allow_smem(pl->fn, pl->smem)) != cudaSuccess) {
             delete pl;
             return cuda_err(e, "cudaFuncSetAttribute");
         }
@@ -503,10 +490,10 @@ bbs_status build_plan(bbs_handle* h, const PlanInputs& in, bbs_var_plan** out) {
         if (left.empty()) pl->has_team = false;
     }
     for (auto& c : pl->classes)
-        if ((e = allow_smem(c.fn, c.smem)) != cudaSuccess)
+        if ((e = bbs::allow_smem(c.fn, c.smem)) != cudaSuccess)
             return plan_fail(pl, cuda_err(e, "shared memory limit (packed)"));
     for (auto& c : pl->blocks) {
-        if ((e = allow_smem(c.fn, c.smem)) != cudaSuccess)
+        if ((e = bbs::allow_smem(c.fn, c.smem)) != cudaSuccess)
             return plan_fail(pl, cuda_err(e, "shared memory limit (one block per system)"));
         c.grid = c.P.count;
         if (!c.wide) {
