@@ -316,8 +316,10 @@ typedef struct {
  * many warps still leave an SM 8 warps; the others run in the persistent
  * launches). With BiCGSTAB and Jacobi a system that one block can stage takes
  * the fewest warps, a power of two, that leave 8 rows per thread (2 where its
- * rows hold more than 24 values on average), whatever team_warps and
- * stage_values say. block_warps is 8 (up to 8 rows per thread) or 16 (up to 4 rows per
+ * rows hold more than 24 values on average): team_warps, stage_values and
+ * block_warps are choices for the systems that no block can stage (and for CG and
+ * unpreconditioned systems), and bbs_var_tune leaves them at the default in
+ * buckets without any. block_warps is 8 (up to 8 rows per thread) or 16 (up to 4 rows per
  * thread). The planner lowers a bucket's warps to those of the next larger
  * bucket if they exceed them and raises them to the minimum its rows need. */
 typedef struct {

@@ -901,9 +901,26 @@ bbs_status bbs_var_tune(bbs_handle* h, const bbs_var_batch* vb, const bbs_var_ho
             if (host->pat_n[host->sys_pattern[i]] <= kVarPackMaxN) has_small[k] = 1;
     }
 
+    // Team warps, staging and block warps are choices of the persistent launch of
+    // warp teams: with BiCGSTAB and Jacobi only systems that no block can stage
+    // reach it. A bucket without such systems keeps the default's.
+    int optin = 0;
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, bbs::handle_device(h));
+    const bool blocks = o->solver == BBS_SOLVER_BICGSTAB && o->precond == BBS_PREC_JACOBI;
+    std::vector<char> teams(B, 0);
+    bool any_teams = false;
+    for (int k = 0; k < B; ++k)
+        for (int i : samp[k]) {
+            const int p = host->sys_pattern[i];
+            if (blocks && bbs::varteam_smem(host->pat_n[p], host->pat_nnz[p]) <= (size_t)optin) continue;
+            teams[k] = 1;
+            any_teams = true;
+        }
+
     bbs_var_tuning best_overall = base;
     double best_total = INFINITY;
     for (int bw : {8, 16}) {
+        if (!any_teams && bw != base.block_warps) continue;
         bbs_var_tuning cand = base;
         cand.block_warps = bw;
         const int rmax = bw == 8 ? 8 : 4;
@@ -919,8 +936,10 @@ bbs_status bbs_var_tune(bbs_handle* h, const bbs_var_batch* vb, const bbs_var_ho
             const int wmin = pow2_at_least((nk + 32 * rmax - 1) / (32 * rmax));
             double best = INFINITY;
             int bestw = wmin, bests = 0, bestp = 0;
+            const int w0 = std::max(wmin, std::min(base.team_warps[k], bw));
             for (int w = wmin; w <= bw; w *= 2)
                 for (int stg = 0; stg <= 1; ++stg) {
+                    if (!teams[k] && (w != w0 || stg != base.stage_values[k])) continue;
                     const double per = trial(k, bw, w, stg, 0, 0);
                     if (per < best) {
                         best = per;
