@@ -3,11 +3,11 @@
 // reading its own system's pattern).
 //
 // The planner (bbs_varsize.cu) puts every system of up to L * kMaxPackedR
-// rows whose group fits the shared-memory rule into a class (L, R): the
-// narrowest L of 4, 8, 16 that covers its n in R <= kMaxPackedR rows per lane.
-// Each class is one launch of varpacked_kernel<SOLVER, L, R> over the class's
-// systems (32 / L systems per warp, in lockstep; one or kPackedWarps warps per
-// block), and the
+// rows whose group fits the shared-memory rule into a class (L, R): L = 16 with
+// Jacobi, else the narrowest L of 4, 8, 16 that covers its n in R <= kMaxPackedR
+// rows per lane. Each class is one launch of varpacked_kernel over the class's
+// systems (32 / L systems per warp, in lockstep; one or, with Jacobi, kPackedWarps
+// warps per block), and the
 // plan's CUDA graph holds these launches beside the persistent team kernel.
 // Each pattern of a packed system has an ELL column table built once when
 // the plan is made; the values are gathered through it into shared memory in
@@ -53,9 +53,13 @@ struct VarPackedParams {
     SolveCfg cfg;
 };
 
-// SOLVER: 0 = BiCGSTAB, 1 = CG (the uneven path's two solvers).
-template <int SOLVER, int L, int R>
-__global__ void __launch_bounds__(32 * kPackedWarps, packed_min_blocks(R) / kPackedWarps)
+// SOLVER: 0 = BiCGSTAB, 1 = CG (the uneven path's two solvers). JACOBI: block
+// fixed point with its FP64 fallback (L = 16); without it FP64 alone, one warp to a
+// block: a kernel of its own, since the code for both is slower at it (11,275
+// systems of n = 26 to 181, no preconditioner: 3.06 ms with both, 2.77 alone).
+template <int SOLVER, bool JACOBI, int L, int R>
+__global__ void __launch_bounds__(JACOBI ? 32 * kPackedWarps : 32,
+                                  packed_min_blocks(R) / (JACOBI ? kPackedWarps : 1))
     varpacked_kernel(const __grid_constant__ VarPackedParams P) {
     extern __shared__ __align__(16) unsigned char raw[];
     constexpr int G = 32 / L;
@@ -101,16 +105,23 @@ __global__ void __launch_bounds__(32 * kPackedWarps, packed_min_blocks(R) / kPac
     io.status = P.status + sys;
     io.inner = nullptr;
     io.n = n;
-    if constexpr (SOLVER == 1)
+    if constexpr (JACOBI && SOLVER == 1)
         cg_packed_any<FMT_CSR, L, R>(op, io, valid, P.cfg, sm, tm);
-    else
+    else if constexpr (JACOBI)
         bicgstab_packed_any<FMT_CSR, L, R>(op, io, valid, P.cfg, sm, tm);
+    else if constexpr (SOLVER == 1)
+        cg_packed_system<FMT_CSR, L, R>(op, io, valid, P.cfg, sm, tm);
+    else
+        bicgstab_packed_system<FMT_CSR, L, R>(op, io, valid, P.cfg, sm, tm);
 }
 
-// Kernel of class (L, R) for the solver (0 BiCGSTAB, 1 CG); one table per L.
-const void* varpacked_fn(int solver, int L, int R);
+// Kernel of class (L, R) for the solver (0 BiCGSTAB, 1 CG); one table per L, and
+// one per solver with Jacobi (L = 16).
+const void* varpacked_fn(int solver, bool jacobi, int L, int R);
 const void* varpacked_fn_l4(int solver, int R);
 const void* varpacked_fn_l8(int solver, int R);
 const void* varpacked_fn_l16(int solver, int R);
+const void* varpacked_fn_bicgstab(int R);
+const void* varpacked_fn_cg(int R);
 
 }  // namespace bbs

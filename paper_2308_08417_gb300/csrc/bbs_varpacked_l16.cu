@@ -1,14 +1,14 @@
-// Uneven batches: packed small-system kernels with L = 16 lanes per system,
-// R = 1..kMaxPackedR rows per lane, for BiCGSTAB and CG.
+// Uneven batches without a preconditioner: packed small-system kernels with L = 16
+// lanes per system, R = 1..kMaxPackedR rows per lane, for BiCGSTAB and CG.
 #include "bbs_varpacked.cuh"
 
 namespace bbs {
-#define BBS_ROW(S)                                                                                    \
-    {(const void*)varpacked_kernel<S, 16, 1>, (const void*)varpacked_kernel<S, 16, 2>,                  \
-     (const void*)varpacked_kernel<S, 16, 3>, (const void*)varpacked_kernel<S, 16, 4>,                  \
-     (const void*)varpacked_kernel<S, 16, 5>, (const void*)varpacked_kernel<S, 16, 6>,                  \
-     (const void*)varpacked_kernel<S, 16, 7>, (const void*)varpacked_kernel<S, 16, 8>,                  \
-     (const void*)varpacked_kernel<S, 16, 9>, (const void*)varpacked_kernel<S, 16, 10>}
+#define BBS_ROW(S) \
+    {(const void*)varpacked_kernel<S, false, 16, 1>, (const void*)varpacked_kernel<S, false, 16, 2>,  \
+     (const void*)varpacked_kernel<S, false, 16, 3>, (const void*)varpacked_kernel<S, false, 16, 4>,  \
+     (const void*)varpacked_kernel<S, false, 16, 5>, (const void*)varpacked_kernel<S, false, 16, 6>,  \
+     (const void*)varpacked_kernel<S, false, 16, 7>, (const void*)varpacked_kernel<S, false, 16, 8>,  \
+     (const void*)varpacked_kernel<S, false, 16, 9>, (const void*)varpacked_kernel<S, false, 16, 10>}
 static_assert(kMaxPackedR == 10, "tables cover R = 1..10");
 const void* varpacked_fn_l16(int solver, int R) {
     static const void* const kTable[2][kMaxPackedR] = {BBS_ROW(0), BBS_ROW(1)};

@@ -1,14 +1,14 @@
-// Uneven batches: packed small-system kernels with L = 4 lanes per system,
-// R = 1..kMaxPackedR rows per lane, for BiCGSTAB and CG.
+// Uneven batches without a preconditioner: packed small-system kernels with L = 4
+// lanes per system, R = 1..kMaxPackedR rows per lane, for BiCGSTAB and CG.
 #include "bbs_varpacked.cuh"
 
 namespace bbs {
-#define BBS_ROW(S)                                                                                    \
-    {(const void*)varpacked_kernel<S, 4, 1>, (const void*)varpacked_kernel<S, 4, 2>,                  \
-     (const void*)varpacked_kernel<S, 4, 3>, (const void*)varpacked_kernel<S, 4, 4>,                  \
-     (const void*)varpacked_kernel<S, 4, 5>, (const void*)varpacked_kernel<S, 4, 6>,                  \
-     (const void*)varpacked_kernel<S, 4, 7>, (const void*)varpacked_kernel<S, 4, 8>,                  \
-     (const void*)varpacked_kernel<S, 4, 9>, (const void*)varpacked_kernel<S, 4, 10>}
+#define BBS_ROW(S) \
+    {(const void*)varpacked_kernel<S, false, 4, 1>, (const void*)varpacked_kernel<S, false, 4, 2>,  \
+     (const void*)varpacked_kernel<S, false, 4, 3>, (const void*)varpacked_kernel<S, false, 4, 4>,  \
+     (const void*)varpacked_kernel<S, false, 4, 5>, (const void*)varpacked_kernel<S, false, 4, 6>,  \
+     (const void*)varpacked_kernel<S, false, 4, 7>, (const void*)varpacked_kernel<S, false, 4, 8>,  \
+     (const void*)varpacked_kernel<S, false, 4, 9>, (const void*)varpacked_kernel<S, false, 4, 10>}
 static_assert(kMaxPackedR == 10, "tables cover R = 1..10");
 const void* varpacked_fn_l4(int solver, int R) {
     static const void* const kTable[2][kMaxPackedR] = {BBS_ROW(0), BBS_ROW(1)};

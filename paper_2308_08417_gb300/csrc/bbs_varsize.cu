@@ -21,7 +21,8 @@
 #include "bbs_varsize.cuh"
 
 namespace bbs {
-const void* varpacked_fn(int solver, int L, int R) {
+const void* varpacked_fn(int solver, bool jacobi, int L, int R) {
+    if (jacobi) return solver == 1 ? varpacked_fn_cg(R) : varpacked_fn_bicgstab(R);
     return L == 4 ? varpacked_fn_l4(solver, R) : L == 8 ? varpacked_fn_l8(solver, R) : varpacked_fn_l16(solver, R);
 }
 const void* varteam_fn(int R) { return R <= 5 ? varteam_fn_lo(R) : varteam_fn_hi(R); }
@@ -152,9 +153,10 @@ struct PlanInputs {
 };
 
 // Packed small systems (bbs_varpacked.cuh): a class (L, R) per pattern,
-// chosen by the rule of the uniform packed kernels: the narrowest group of 4,
-// 8 or 16 lanes that covers n in at most kMaxPackedR rows per lane and leaves
-// at least kVarPackedMinWarps one-warp blocks resident per SM.
+// chosen by decide_pattern: 16 lanes with Jacobi, else, as the uniform packed
+// kernels, the narrowest group of 4, 8 or 16 lanes that covers n in at most
+// kMaxPackedR rows per lane and leaves at least kVarPackedMinWarps one-warp blocks
+// resident per SM.
 constexpr int kVarWideMinR = 9, kVarWideMaxR = 16;  // rows per thread that make a team wide
 constexpr int kVarPackMaxN = 16 * bbs::kMaxPackedR;
 constexpr int kVarPackedMinWarps = 8;
@@ -185,7 +187,17 @@ int packed_resident(size_t smem, int R) {
 // Reads pattern p's row pointers (the ELL width k is its longest row) and
 // picks its class; a pattern whose row pointers do not ascend within
 // [0, nnz] is rejected.
-bbs_status decide_pattern(const bbs_var_batch* vb, int p, int n, int nnz, int64_t rp_off, int optin,
+//
+// With Jacobi every group has 16 lanes. Each class is a code of its own, and the
+// fixed-point loops of two of them evict each other from an SM's instruction cache:
+// 14 uniform batches of 800 systems take 2.64 ms one after the other and 0.88 ms at
+// once where they share one code, 2.83 and 1.87 ms where they are of two. So few
+// classes with short loops beat few warps: 11,275 systems of n = 26 to 181 3.0 ms
+// with the narrowest groups (14 classes), 1.28 ms with 16 lanes (FP64: 1.95 ms);
+// 20,000 of 16 to 64 1.13 and 0.68 ms (1.36); 20,000 of 16 to 1,024 7.4 and 6.8 ms (12.4);
+// CG on the first 1.41 and 1.04 ms (1.34). The batch's size stays out of it, as a
+// system's bits depend on its group.
+bbs_status decide_pattern(const bbs_var_batch* vb, int p, int n, int nnz, int64_t rp_off, int optin, bool jacobi,
                           PatPack& pp) {
     std::vector<int32_t> rp(n + 1);
     cudaError_t e = cudaMemcpy(rp.data(), vb->row_ptrs + rp_off, sizeof(int32_t) * (n + 1), cudaMemcpyDeviceToHost);
@@ -198,7 +210,7 @@ bbs_status decide_pattern(const bbs_var_batch* vb, int p, int n, int nnz, int64_
     }
     pp.state = 2;
     const int n_pad = (n + 1) & ~1;
-    for (int L = 4; L <= 16; L *= 2) {
+    for (int L = jacobi ? 16 : 4; L <= 16; L *= 2) {
         const int R = (n + L - 1) / L;
         if (R > bbs::kMaxPackedR) continue;
         const size_t raw = align16((size_t)2 * n_pad * 8) + align16((size_t)k * n * 8);
@@ -271,7 +283,8 @@ bbs_status build_plan(bbs_handle* h, const PlanInputs& in, bbs_var_plan** out) {
                                            cudaMemcpyDeviceToHost);
                 if (e != cudaSuccess) return cuda_err(e, "pattern offsets");
             }
-            bbs_status s = decide_pattern(vb, p, n, in.host->pat_nnz[p], rp_off[p], optin, pat[p]);
+            bbs_status s = decide_pattern(vb, p, n, in.host->pat_nnz[p], rp_off[p], optin,
+                                          in.o->precond == BBS_PREC_JACOBI, pat[p]);
             if (s != BBS_OK) return s;
         }
         packed[i] = pat[p].state == 1;
@@ -393,7 +406,7 @@ bbs_status build_plan(bbs_handle* h, const PlanInputs& in, bbs_var_plan** out) {
             c.warps = bbs::kPackedWarps;
         c.smem *= (size_t)c.warps;
         c.grid = (warps + c.warps - 1) / c.warps;
-        c.fn = bbs::varpacked_fn(in.o->solver == BBS_SOLVER_CG ? 1 : 0, c.L, c.R);
+        c.fn = bbs::varpacked_fn(in.o->solver == BBS_SOLVER_CG ? 1 : 0, in.o->precond == BBS_PREC_JACOBI, c.L, c.R);
         pl->packed_count += c.P.count;
         pl->classes.push_back(c);
     }

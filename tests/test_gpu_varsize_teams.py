@@ -114,3 +114,27 @@ def test_tuner_leaves_choices_without_effect(bbs, handle):
     want = bbs.bbs_var_default_tuning(int(vb.sys_n().max())).as_dict()
     for key in ("team_warps", "stage_values", "block_warps"):
         assert tuned[key] == want[key], key
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(solver="cg"), dict(precond="none")])
+def test_packed_sizes_at_the_edges_of_their_classes(bbs, handle, kw):
+    """n = 3 and every multiple of 16 with its neighbours up to 160, with Jacobi in
+    ten classes of 16 lanes (few codes at once; narrower groups, 4 and 8 lanes too,
+    without a preconditioner)."""
+    rng = np.random.default_rng(17)
+    sizes = [3] + sorted({n for k in range(1, 11) for n in (16 * k - 1, 16 * k, 16 * k + 1) if n <= 160})
+    pats = [W.stencil_pattern("1d3", n) for n in sizes]
+    index = np.tile(np.arange(len(pats), dtype=np.int32), 11)
+    vals = [W.stencil_values(pats[p], 1, rng, 0.05, 0.5, symmetric=True)[0] for p in index]
+    n = np.array([pats[p].n for p in index])
+    nnz = np.array([pats[p].nnz for p in index])
+    b = rng.uniform(-1, 1, int(n.sum()))
+    vb = W.VarBatch(pats, index, np.cumsum(nnz) - nnz, np.cumsum(n) - n, np.concatenate(vals), b, np.zeros(len(b)),
+                    "edges")
+    plan = bbs.VarPlan(handle, bbs.VarDeviceBatch.from_varbatch(vb), bbs.bbs_default_options(**kw))
+    d = plan.describe()
+    assert d["packed_systems"] == vb.num_batch
+    assert d["packed_launches"] == 10 or "precond" in kw and d["packed_launches"] > 10
+    got = run_plan(bbs, plan, vb)
+    assert (got[3] == 0).all()
+    check(vb, got, np.arange(0, vb.num_batch, 2), **kw)
