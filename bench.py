@@ -53,12 +53,21 @@ METRIC = "systems solved/s to rel. residual 1e-10"
 FP64_FLOP_PER_CLK_SM = 4.0
 # FP32 (non-tensor) FMA lanes: 128 per SM per clock = 256 FLOP/clk/SM.
 FP32_FLOP_PER_CLK_SM = 256.0
-# The Jacobi solvers work in 62-bit block fixed point on the integer pipe: 64
-# lanes of 32 x 32 + 64-bit multiply-add per SM per clock, up to four of them
-# per multiply-add of the algorithm = 32 FLOP/clk/SM.
+# The Jacobi solvers work in block fixed point (57 bits below one exponent per
+# vector, results confirmed and returned in FP64) on the integer pipe where a
+# system fits it: 64 lanes of 32 x 32 + 64-bit multiply-add per SM per clock, up
+# to four of them per multiply-add of the algorithm = 32 FLOP/clk/SM.
 INT64_FLOP_PER_CLK_SM = 32.0
 FIXED_POINT_KERNELS = {"bicgstab_packed_kernel", "bicgstab_folded_kernel", "cg_packed_kernel", "cg_kernel",
                        "gmres_packed_kernel", "varteam_kernel", "varpacked_kernel", "varteam_kernel+varpacked_kernel"}
+
+
+def arithmetic(kernel, precond, staged):
+    """What a launch computes in: "int64" (block fixed point, FP64 for systems that
+    do not fit it) with Jacobi on staged values, else "fp64"."""
+    return "int64" if precond == 1 and staged and kernel in FIXED_POINT_KERNELS else "fp64"
+
+
 NUM_SMS = 152
 HBM_GBS = 6789.0  # measured copy bandwidth of this pool's GB300s
 
@@ -256,8 +265,7 @@ class Uniform:
             inner = self.log.inner_iters.cpu().numpy().astype(np.int64)
             return float(inner.sum()) * per_it, "fp32"
         it = self.log.iters.cpu().numpy().astype(np.int64)
-        fixed = o.precond == 1 and self.kernel in FIXED_POINT_KERNELS
-        return float(it.sum()) * per_it, "int64" if fixed else "fp64"
+        return float(it.sum()) * per_it, arithmetic(self.kernel, o.precond, self.launch["staged"])
 
     def compulsory_bytes(self):
         B, A = self.num_batch, self.A
@@ -369,7 +377,7 @@ class Uneven:
     def work(self):
         it = self.log.iters.cpu().numpy().astype(np.int64)
         per_it = 4 * self.vb.sys_nnz().astype(np.int64) + 26 * self.vb.sys_n().astype(np.int64)
-        return float((it * per_it).sum()), "int64" if self.kernel in FIXED_POINT_KERNELS else "fp64"
+        return float((it * per_it).sum()), arithmetic(self.kernel, 1, True)
 
     def compulsory_bytes(self):
         return 8 * (self.vb.values.size + 3 * self.vb.b.size) + 16 * self.num_batch
@@ -898,6 +906,9 @@ def main():
             "dtype": "f64+f32" if r.mixed else "f64", "data": "synthetic",
             "config": {"workload": r.label, "num_batch_per_gpu": r.num_batch, "tol": 1e-10,
                        "solver": f"{args.solver}+{args.precond}" if args.workload == "scale" else "bicgstab+jacobi",
+                       "arithmetic": {"int64": "64-bit block fixed point, x and log in FP64; FP64 for systems "
+                                               "that do not fit", "fp64": "FP64",
+                                      "fp32": "FP32 inner solves in FP64 refinement"}[r.work()[1]],
                        "l2": "inputs larger than L2 (no flush)"},
             "gpu_launches": args.steps * r.launches_per_step,
             "launch": getattr(r, "launch", None),
