@@ -56,8 +56,14 @@ typedef enum { BBS_PREC_NONE = 0, BBS_PREC_JACOBI = 1, BBS_PREC_ILU0 = 2 } bbs_p
 /* Stopping criteria, Table "Batched feature support": stop when
  * ||b - A x||_2 <= tol (absolute) or <= tol * ||b||_2 (relative). */
 typedef enum { BBS_TOL_ABSOLUTE = 0, BBS_TOL_RELATIVE = 1 } bbs_tol_type;
-/* FP64 throughout, or FP32 inner BiCGSTAB inside FP64 iterative refinement
- * (residual, update and exit test in FP64). */
+/* FP64: matrix, vectors, results and tests of FP64's accuracy, or FP32 inner
+ * BiCGSTAB inside FP64 iterative refinement (residual, update and exit test in
+ * FP64). With Jacobi and staged values, FP64 BiCGSTAB, CG and packed GMRES work in
+ * 64-bit block fixed point (57 bits and more below one exponent per vector) for the
+ * systems where that keeps no fewer bits: equations of one scale (within 2^12), a
+ * diagonal excess of 2^-7 (BiCGSTAB) or 2^-9 (CG). The residual of the returned x decides
+ * the status; every other system, and one that stops early, is solved in FP64
+ * arithmetic. values_in_smem = -1 solves all of a call in FP64 arithmetic. */
 typedef enum { BBS_PRECISION_FP64 = 0, BBS_PRECISION_MIXED_IR = 1 } bbs_precision;
 /* Per-system outcome written to bbs_log.status. */
 typedef enum {
@@ -305,8 +311,8 @@ typedef struct {
  * of warps that solve one of its systems (1, 2, 4, 8 or 16; at most
  * block_warps), whether its systems' values are staged in shared memory, and
  * whether its small systems are packed (pack[b] = 1: a system of at most 160
- * rows whose group fits shared memory is solved by 4, 8 or 16 lanes, with
- * 8, 4 or 2 systems per warp in lockstep, as bbs_solve packs uniform batches;
+ * rows whose group fits shared memory is solved by 16 lanes with Jacobi, by 4, 8
+ * or 16 without, with 2, or 8, 4 or 2, systems per warp in lockstep;
  * 0: one team per system), and which of its large systems run as wide teams
  * (wide[b], BiCGSTAB with Jacobi only, a bit set: 1 = systems whose rows hold
  * at most 4 stored values on average, 2 = the others, 3 = both, 0 = none. Such

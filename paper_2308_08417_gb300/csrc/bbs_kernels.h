@@ -35,7 +35,9 @@ const void* refine_ell_fn(int R, int K);
 // Packed BiCGSTAB, CG and GMRES (32 / L systems per warp): L = 4, 8 or 16
 // lanes per system, R = 1..kMaxPackedR rows per lane.
 constexpr int kMaxPackedR = 10;
-constexpr int kPackedWarps = 4;  // warps of a packed BiCGSTAB block, one on each of an SM's schedulers
+// Warps of a packed fixed-point block (BiCGSTAB and CG, uniform and uneven), one on
+// each of an SM's schedulers.
+constexpr int kPackedWarps = 4;
 #define BBS_DECL_PACKED(S)                       \
     const void* S##_packed_fn(int fmt, int L, int R); \
     const void* S##_packed_fn_csr_l4(int R);          \

@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kInferThreads, 1)
         const int q = warp & 3, group = warp >> 2;
         const int r = q * 32 + lane;
         const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
-        // the tile's features: the 256 threads walk the tile's rows of b and
+        // the tile's features: the 512 threads walk the tile's rows of b and
         // x_prev (contiguous across the tile's systems) and its diagonal
         // entries with coalesced loads, and scatter the standardised BF16
         // values into the core-matrix layout; padding columns get zeros

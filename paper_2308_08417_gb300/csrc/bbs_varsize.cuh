@@ -5,8 +5,9 @@
 // Uneven batches: one persistent, graph-captured launch over systems of
 // different sizes and patterns, with the team size per size bucket chosen by
 // a measured autotuner (the per-device experimental thresholds of Sec. 3.6).
-// BiCGSTAB with Jacobi does not come here: it has a block per system
-// (bbs_varteam.cuh) and packed launches (bbs_varpacked.cuh).
+// With BiCGSTAB and Jacobi only the systems whose values no block can stage come
+// here: the others have a block per system (bbs_varteam.cuh) and packed launches
+// (bbs_varpacked.cuh).
 //
 // Scheduling. The planner orders the systems by team size (largest first)
 // and, within a team size, by estimated cost (longest first), and cuts the
