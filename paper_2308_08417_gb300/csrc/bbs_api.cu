@@ -673,10 +673,12 @@ bbs_status bbs_solve(bbs_handle* h, const bbs_batch_matrix* A, const double* b, 
             P.xflag = flag;
             P.xk = A->ell_k;
         }
-        const void* fn = p.ilu ? bbs::bicgstab_ilu_packed_fn(p.lanes, p.R)
-                         : o->solver == BBS_SOLVER_CG ? bbs::cg_packed_fn(A->fmt, p.lanes, p.R)
-                         : o->solver == BBS_SOLVER_GMRES ? bbs::gmres_packed_fn(A->fmt, p.lanes, p.R)
-                                                         : bbs::bicgstab_packed_fn(A->fmt, p.lanes, p.R);
+        const bool jacobi = o->precond == BBS_PREC_JACOBI;
+        const auto pick = o->solver == BBS_SOLVER_CG ? (jacobi ? bbs::cg_packed_fn : bbs::cg_plain_packed_fn)
+                          : o->solver == BBS_SOLVER_GMRES
+                              ? (jacobi ? bbs::gmres_packed_fn : bbs::gmres_plain_packed_fn)
+                              : (jacobi ? bbs::bicgstab_packed_fn : bbs::bicgstab_plain_packed_fn);
+        const void* fn = p.ilu ? bbs::bicgstab_ilu_packed_fn(p.lanes, p.R) : pick(A->fmt, p.lanes, p.R);
         if ((e = bbs::allow_smem(fn, p.smem * p.warps)) != cudaSuccess) return cuda_fail(e, "shared memory limit");
         void* args[] = {&P, &csched};  // the ILU(0) kernels take the schedule as a second argument
         const unsigned warps = (unsigned)((A->num_batch + per_block - 1) / per_block);

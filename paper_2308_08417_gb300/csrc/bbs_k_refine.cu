@@ -133,6 +133,9 @@ BBS_FRONT(refine)
 BBS_PACKED_FRONT(bicgstab)
 BBS_PACKED_FRONT(cg)
 BBS_PACKED_FRONT(gmres)
+BBS_PACKED_FRONT(bicgstab_plain)
+BBS_PACKED_FRONT(cg_plain)
+BBS_PACKED_FRONT(gmres_plain)
 #undef BBS_PACKED_FRONT
 
 }  // namespace bbs

@@ -52,6 +52,9 @@ constexpr int kPackedWarps = 4;
 BBS_DECL_PACKED(bicgstab)
 BBS_DECL_PACKED(cg)
 BBS_DECL_PACKED(gmres)
+BBS_DECL_PACKED(bicgstab_plain)  // without a preconditioner
+BBS_DECL_PACKED(cg_plain)
+BBS_DECL_PACKED(gmres_plain)
 #undef BBS_DECL_PACKED
 
 cudaError_t launch_check_pattern(int fmt, int n, int nnz, int k, const int32_t* rp, const int32_t* cols,

@@ -368,8 +368,8 @@ struct PackedArgs {
     }
 };
 
-// BiCGSTAB of a warp's groups: with Jacobi in block fixed point (the integer
-// pipe); the groups it leaves (and all of them without Jacobi) in FP64. The
+// BiCGSTAB of a warp's groups with Jacobi: block fixed point (the integer pipe),
+// and FP64 for the groups that it leaves. The
 // FP64 form is compiled as a function of its own. `again` (per group): the staged
 // values have been overwritten.
 template <int FMT, int L, int R>
@@ -384,9 +384,9 @@ __device__ __noinline__ void bicgstab_packed_fp64(const PackedOp<FMT, R> op, con
 template <int FMT, int L, int R>
 __device__ __forceinline__ void bicgstab_packed_any(const PackedOp<FMT, R>& op, const SysIO& io, bool valid,
                                                     const SolveCfg& C, const TeamSmem& sm, const Team& tm) {
-    fx::Fit fit = fx::kUnfit;
-    if (C.precond == 1)  // every lane takes part, those without a system too
-        fit = fx::bicgstab_fixed<FMT, staged_fmt<FMT>(), R>(op.A, op.S, io, valid, C, sm, fx::Lanes<L>{tm.lane}, tm);
+    // every lane takes part, those without a system too
+    const fx::Fit fit =
+        fx::bicgstab_fixed<FMT, staged_fmt<FMT>(), R>(op.A, op.S, io, valid, C, sm, fx::Lanes<L>{tm.lane}, tm);
     const bool left = valid && fit != fx::kDone;
     if (__any_sync(kFull, left)) {
         __syncwarp();
@@ -586,9 +586,8 @@ __device__ __noinline__ void cg_packed_fp64(const PackedOp<FMT, R> op, const Sys
 template <int FMT, int L, int R>
 __device__ __forceinline__ void cg_packed_any(const PackedOp<FMT, R>& op, const SysIO& io, bool valid,
                                               const SolveCfg& C, const TeamSmem& sm, const Team& tm) {
-    fx::Fit fit = fx::kUnfit;
-    if (C.precond == 1)  // every lane takes part, those without a system too
-        fit = fx::cg_fixed<FMT, staged_fmt<FMT>(), R>(op.A, op.S, io, valid, C, sm, fx::Lanes<L>{tm.lane}, tm);
+    const fx::Fit fit =
+        fx::cg_fixed<FMT, staged_fmt<FMT>(), R>(op.A, op.S, io, valid, C, sm, fx::Lanes<L>{tm.lane}, tm);
     const bool left = valid && fit != fx::kDone;
     if (__any_sync(kFull, left)) {
         __syncwarp();
@@ -975,10 +974,10 @@ __global__ void __launch_bounds__(32, packed_cg_min_blocks(R)) gmres_packed_kern
     const size_t count = FMT == FMT_CSR ? (size_t)P.xk * P.n : P.vps;
     unsigned char* slice = raw + (size_t)((threadIdx.x & 31) / L) * P.slice;
     double* ext = reinterpret_cast<double*>(slice + P.stage_off + ((count * 8 + 15) & ~(size_t)15));
-    fx::Fit fit = fx::kUnfit;
-    if (P.precond == 1)  // block fixed point; every lane takes part, those without a system too
-        fit = fx::gmres_fixed<FMT, staged_fmt<FMT>(), R>(G.op.A, G.op.S, sys_io(P, G.sys), G.valid, solve_cfg(P, G.sys),
-                                                         G.sm, ext, fx::Lanes<L>{G.tm.lane}, G.tm);
+    // block fixed point; every lane takes part, those without a system too
+    const fx::Fit fit =
+        fx::gmres_fixed<FMT, staged_fmt<FMT>(), R>(G.op.A, G.op.S, sys_io(P, G.sys), G.valid, solve_cfg(P, G.sys), G.sm,
+                                                   ext, fx::Lanes<L>{G.tm.lane}, G.tm);
     const bool left = G.valid && fit != fx::kDone;
     if (__any_sync(kFull, left)) {
         __syncwarp();
@@ -993,6 +992,36 @@ __global__ void __launch_bounds__(32 * kPackedWarps, packed_cg_min_blocks(R) / k
     const PackedGroup<FMT, L, R> G(P, raw, blockIdx.x);
     if (packed_reject(P, G)) return;
     cg_packed_any<FMT, L, R>(G.op, sys_io(P, G.sys), G.valid, solve_cfg(P, G.sys), G.sm, G.tm);
+}
+
+// The same methods without a preconditioner: FP64, one warp to a block, in kernels of
+// their own (behind a branch of the ones above 16,384 systems of n = 144 took 2 to 3 %
+// longer with BiCGSTAB and CG).
+template <int FMT, int L, int R>
+__global__ void __launch_bounds__(32, packed_min_blocks(R)) bicgstab_plain_packed_kernel(const SolveParams P) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    const PackedGroup<FMT, L, R> G(P, raw, blockIdx.x);
+    if (packed_reject(P, G)) return;
+    bicgstab_packed_system<FMT, L, R>(G.op, sys_io(P, G.sys), G.valid, solve_cfg(P, G.sys), G.sm, G.tm);
+}
+
+template <int FMT, int L, int R>
+__global__ void __launch_bounds__(32, packed_cg_min_blocks(R)) cg_plain_packed_kernel(const SolveParams P) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    const PackedGroup<FMT, L, R> G(P, raw, blockIdx.x);
+    if (packed_reject(P, G)) return;
+    cg_packed_system<FMT, L, R>(G.op, sys_io(P, G.sys), G.valid, solve_cfg(P, G.sys), G.sm, G.tm);
+}
+
+template <int FMT, int L, int R>
+__global__ void __launch_bounds__(32, packed_cg_min_blocks(R)) gmres_plain_packed_kernel(const SolveParams P) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    const PackedGroup<FMT, L, R> G(P, raw, blockIdx.x);
+    if (packed_reject(P, G)) return;
+    const size_t count = FMT == FMT_CSR ? (size_t)P.xk * P.n : P.vps;
+    unsigned char* slice = raw + (size_t)((threadIdx.x & 31) / L) * P.slice;
+    double* ext = reinterpret_cast<double*>(slice + P.stage_off + ((count * 8 + 15) & ~(size_t)15));
+    gmres_packed_system<FMT, L, R>(G.op, sys_io(P, G.sys), G.valid, solve_cfg(P, G.sys), G.sm.xa, ext, G.tm);
 }
 
 }  // namespace bbs
