@@ -78,10 +78,10 @@ HBM_GBS = 6789.0  # measured copy bandwidth of the GB300s
 # compulsory bytes, which grow in proportion). A kernel run on a workload
 # without a capture reports null, and an entry is removed when its kernel
 # changes.
-TRAFFIC = {("bicgstab_packed_kernel", "stencil2d5_12x12"): (135.44e6, 16384),
-           ("bicgstab_folded_kernel", "stencil2d5_12x12"): (280.15e6, 32768),
-           ("cg_packed_kernel", "sym_stencil2d5_12x12_cg+jacobi"): (132.32e6, 16384),
-           ("gmres_packed_kernel", "stencil2d5_12x12_gmres+jacobi"): (149.97e6, 16384),
+TRAFFIC = {("bicgstab_packed_kernel", "stencil2d5_12x12"): (135.47e6, 16384),
+           ("bicgstab_folded_kernel", "stencil2d5_12x12"): (280.28e6, 32768),
+           ("cg_packed_kernel", "sym_stencil2d5_12x12_cg+jacobi"): (134.51e6, 16384),
+           ("gmres_packed_kernel", "stencil2d5_12x12_gmres+jacobi"): (153.78e6, 16384),
            ("bicgstab_ilu_packed_kernel", "stencil2d5_12x12_bicgstab+ilu0"): (134.60e6, 16384),
            ("refine_kernel", "stencil2d9_32x32"): (396.44e6, 4096)}
 
