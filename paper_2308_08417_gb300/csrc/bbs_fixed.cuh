@@ -151,7 +151,7 @@ __device__ __forceinline__ void fill_up(long long (&y)[R], int& e, int& bits, G&
         for (int q = 0; q < R; ++q) y[q] = (long long)((unsigned long long)y[q] << far);
         k -= far;
         e -= far;
-        bits = min(bits, 56 - k);
+        if (bits <= 44) bits = 56 - k;  // (the others' k is theirs: no group sees its neighbours)
     }
     e -= k;
     bits += k;

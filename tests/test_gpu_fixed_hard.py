@@ -158,3 +158,26 @@ def test_cg_with_diagonals_far_apart(bbs, handle, fmt, tps, bits):
         fails = compare(*g[:4], r[0], r[1], r[3], rel_host=host_rel_residual(D, g[0], b), label=f"{fmt} {tps}",
                         iter_tol=2 + iteration_spread(oracle.solve_batch, A, b, x0, solver="cg"))
         assert not fails, "\n".join(fails)
+
+
+@pytest.mark.parametrize("solver", ["bicgstab", "cg", "gmres"])
+@pytest.mark.parametrize("tps,tol", [(4, 1e-10), (4, 2e-15), (8, 2e-15), (16, 2e-15)])
+def test_bits_do_not_depend_on_the_warps_other_systems(bbs, handle, solver, tps, tol):
+    """Systems whose residuals fall by 1 to 40 bits a step, restart, break down or do not
+    fit, in one batch: each keeps its bits wherever it stands in it."""
+    rng = np.random.default_rng(19)
+    n, B = 30, 4000
+    pat, vals = recipe("1d3", n, 1, B, 0.01, 0.02, rng, symmetric=True)
+    rows = np.repeat(np.arange(n), np.diff(pat.row_ptrs))
+    diag = pat.col_idxs == rows
+    vals[:, diag] *= 10.0 ** (6 * rng.uniform(0, 1, (B, 1)) ** 3)
+    b = rng.uniform(-1, 1, (B, n))
+    b[::7] *= 2.0 ** -(30 * rng.uniform(0, 1, (len(b[::7]), n)))
+    x0 = np.where(rng.uniform(0, 1, (B, 1)) < 0.3, rng.uniform(-1, 1, (B, n)), 0.0)
+    kw = dict(solver=solver, threads_per_system=tps, tol=tol, max_iters=200)
+    want = gpu_solve(bbs, handle, W.make_batch(pat, vals, "ell"), b, x0, **kw)
+    for _ in range(3):
+        p = rng.permutation(B)
+        got = gpu_solve(bbs, handle, W.make_batch(pat, vals[p], "ell"), b[p], x0[p], **kw)
+        for w, g in zip(want[:4], got[:4]):
+            assert np.array_equal(w[p], g, equal_nan=w.dtype.kind == "f")
